@@ -160,6 +160,15 @@ struct RecordHook {
   }
 };
 
+// A second read of a value read before, which the compiler must not keep in
+// registers in between (the step holds x twice otherwise, FP64 and double-float,
+// through all its stages).
+__device__ __forceinline__ double reload_f64(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+
 // One time step of particle i of store s in mesh m, starting in cell K.
 // TWO: the mesh carries a second field (time interpolation).
 // Writes the new x and x-hat in place when the particle survives and returns
@@ -182,14 +191,12 @@ __device__ __forceinline__ uint32_t advect_particle_cells(const Cells& cs, const
     return PIC_LOST;
   }
   uint32_t Ks = K;
-  double x[D];
   df xd[D], ts[D], k[D], acc[D], y[D];
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    x[a] = s.x[a * s.cap + i];
     const float2 v = s.xhat[a * s.cap + i];
     ts[a] = df_make(v.x, v.y);
-    xd[a] = df_from_double(x[a]);
+    xd[a] = df_from_double(s.x[a * s.cap + i]);
     acc[a] = df_make(0.f, 0.f);
   }
 #pragma unroll 1
@@ -225,7 +232,7 @@ __device__ __forceinline__ uint32_t advect_particle_cells(const Cells& cs, const
   }
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    d.x[a * d.cap + j] = (x[a] + (double)acc[a].hi) + (double)acc[a].lo;
+    d.x[a * d.cap + j] = (reload_f64(s.x + a * s.cap + i) + (double)acc[a].hi) + (double)acc[a].lo;
     d.xhat[a * d.cap + j] = make_float2(ts[a].hi, ts[a].lo);
   }
   return Ks;

@@ -21,6 +21,10 @@
 
 namespace pic {
 
+struct LdgLoader {
+  __device__ __forceinline__ float4 ld(const float4* p) const { return __ldg(p); }
+};
+
 // 1 / a: FP32 reciprocal refined by one Newton step in double-float.
 __device__ __forceinline__ df df_recip(df a) {
   const float r = __frcp_rn(a.hi);
@@ -33,19 +37,15 @@ __device__ __forceinline__ df df_recip(df a) {
 // q2_eval_df reads them) at s0, s1: its value g and its derivatives g0 along
 // s0 and g1 along s1.  Along s0 each row q gives its value h and derivative
 // h' = c_1 + 2 c_2 s0; along s1 the rows combine the same way.
-__device__ __forceinline__ void grad_slice_df(const float4* __restrict__ sl, df s0, df s1, df& g, df& g0, df& g1) {
-  float f[20];  // ten high parts, then ten low parts
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    const float4 v = __ldg(sl + k);
-    f[4 * k] = v.x;
-    f[4 * k + 1] = v.y;
-    f[4 * k + 2] = v.z;
-    f[4 * k + 3] = v.w;
-  }
+template <int D, class Ld>
+__device__ __forceinline__ void grad_slice_df(const Ld& ld, const float4* __restrict__ sl, int r, df s0, df s1, df& g,
+                                              df& g0, df& g1) {
+  float hi[10], lo[10];
+  load_slice(ld, sl, hi, lo);
   df c[9];
 #pragma unroll
-  for (int e = 0; e < 9; ++e) c[e] = df_make(f[e], f[10 + e]);
+  for (int e = 0; e < 9; ++e)
+    c[e] = df_make(D == 3 && qc_on_grid(e % 3, e / 3, r) ? __fsub_rn(hi[e], hi[9]) : hi[e], lo[e]);
   df h[3], h0[3];
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
@@ -69,12 +69,13 @@ __device__ __forceinline__ void q2_grad_mono_df(const float4* __restrict__ Qc, u
 #pragma unroll
   for (int a = 0; a < D; ++a) s[a] = centred(t[a]);
   const float4* cell = Qc + (size_t)K * D * (5 * NS);
+  const LdgLoader ld;
 #pragma unroll 1
   for (int comp = 0; comp < D; ++comp) {
     const float4* cq = cell + comp * (5 * NS);
     df g[NS], g0[NS], g1[NS];
 #pragma unroll
-    for (int r = 0; r < NS; ++r) grad_slice_df(cq + 5 * r, s[0], s[1], g[r], g0[r], g1[r]);
+    for (int r = 0; r < NS; ++r) grad_slice_df<D>(ld, cq + 5 * r, r, s[0], s[1], g[r], g0[r], g1[r]);
     if constexpr (D == 3) {
       Gu[comp][0] = df_norm(df_horner(df_horner(g0[2], s[2], g0[1]), s[2], g0[0]));
       Gu[comp][1] = df_norm(df_horner(df_horner(g1[2], s[2], g1[1]), s[2], g1[0]));
@@ -88,32 +89,36 @@ __device__ __forceinline__ void q2_grad_mono_df(const float4* __restrict__ Qc, u
 
 // J_ij = dPhi_i/dt_j from the monomial block: in 3D the monomials are
 // (t0, t1, t2, t0 t1, t0 t2, t1 t2, t0 t1 t2), in 2D (t0, t1, t0 t1).
-template <int D>
-__device__ __forceinline__ void map_jacobian_df(const CellBlock<D>& cb, const df t[D], df J[D][D]) {
+template <int D, class Ld>
+__device__ __forceinline__ void map_jacobian_df(const Ld& ld, const float4* B, const df t[D], df J[D][D]) {
+  df t01, t02, t12;
   if constexpr (D == 3) {
-    const df t01 = df_mul(t[0], t[1]), t02 = df_mul(t[0], t[2]), t12 = df_mul(t[1], t[2]);
+    t01 = df_mul(t[0], t[1]);
+    t02 = df_mul(t[0], t[2]);
+    t12 = df_mul(t[1], t[2]);
+  }
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      df_acc j0 = acc_init(cb.a[0][i]), j1 = acc_init(cb.a[1][i]), j2 = acc_init(cb.a[2][i]);
-      acc_mad(j0, cb.a[3][i], t[1]);
-      acc_mad(j0, cb.a[4][i], t[2]);
-      acc_mad(j0, cb.a[6][i], t12);
-      acc_mad(j1, cb.a[3][i], t[0]);
-      acc_mad(j1, cb.a[5][i], t[2]);
-      acc_mad(j1, cb.a[6][i], t02);
-      acc_mad(j2, cb.a[4][i], t[0]);
-      acc_mad(j2, cb.a[5][i], t[1]);
-      acc_mad(j2, cb.a[6][i], t01);
+  for (int i = 0; i < D; ++i) {
+    const MapRow<D> hi = load_row<D>(ld, B, 0, i), lo = load_row<D>(ld, B, 1, i);
+    auto a = [&](int k) { return df_make(hi.a[k], lo.a[k]); };
+    if constexpr (D == 3) {
+      df_acc j0 = acc_init(a(0)), j1 = acc_init(a(1)), j2 = acc_init(a(2));
+      acc_mad(j0, a(3), t[1]);
+      acc_mad(j0, a(4), t[2]);
+      acc_mad(j0, a(6), t12);
+      acc_mad(j1, a(3), t[0]);
+      acc_mad(j1, a(5), t[2]);
+      acc_mad(j1, a(6), t02);
+      acc_mad(j2, a(4), t[0]);
+      acc_mad(j2, a(5), t[1]);
+      acc_mad(j2, a(6), t01);
       J[i][0] = acc_result(j0);
       J[i][1] = acc_result(j1);
       J[i][2] = acc_result(j2);
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      df_acc j0 = acc_init(cb.a[0][i]), j1 = acc_init(cb.a[1][i]);
-      acc_mad(j0, cb.a[2][i], t[1]);
-      acc_mad(j1, cb.a[2][i], t[0]);
+    } else {
+      df_acc j0 = acc_init(a(0)), j1 = acc_init(a(1));
+      acc_mad(j0, a(2), t[1]);
+      acc_mad(j1, a(2), t[0]);
       J[i][0] = acc_result(j0);
       J[i][1] = acc_result(j1);
     }
@@ -164,9 +169,7 @@ template <int D>
 __device__ __forceinline__ void velocity_gradient_df(const MeshView& m, uint32_t K, const df t[D], df G[D][D]) {
   df Gu[D][D], J[D][D], Ji[D][D];
   q2_grad_mono_df<D>(m.Qc, K, t, Gu);
-  CellBlock<D> cb;
-  load_block<D>(m, K, cb);
-  map_jacobian_df<D>(cb, t, J);
+  map_jacobian_df<D>(LdgLoader(), m.blk + (size_t)K * block_float4s<D>(), t, J);
   invert_df<D>(J, Ji);
 #pragma unroll
   for (int c = 0; c < D; ++c)

@@ -67,9 +67,9 @@ __device__ __forceinline__ float2 split_df(double v) {
 //   a_t0 = e1, a_t1 = e2, a_t2 = e4, a_t0t1 = e3 - e1 - e2,
 //   a_t0t2 = e5 - e1 - e4, a_t1t2 = e6 - e2 - e4,
 //   a_t0t1t2 = e7 - e3 - e5 - e6 + e1 + e2 + e4.
-// Stored as the NF high parts (X_0, then a_k,c in (k, c) order) followed by
-// the NF low parts in the same order, so that the FP32 Newton iterations
-// read only the first half.
+// Stored as one row (X_0, a_1, a_2, ...) per component, the high parts of every
+// row and then the low parts, so that the FP32 Newton iterations read only the
+// first half and take a component at a time.
 template <int D>
 __global__ void cell_block_kernel(const __grid_constant__ MeshView m, float* __restrict__ blk) {
   constexpr int NK = (1 << D) - 1;
@@ -83,7 +83,7 @@ __global__ void cell_block_kernel(const __grid_constant__ MeshView m, float* __r
       out[idx] = p.x;
       out[NF + idx] = p.y;
     };
-    for (int a = 0; a < D; ++a) put(a, g.x0[a]);
+    for (int a = 0; a < D; ++a) put(a * (NK + 1), g.x0[a]);
     for (int a = 0; a < D; ++a) {
       double coef[NK];
       if constexpr (D == 2) {
@@ -99,7 +99,7 @@ __global__ void cell_block_kernel(const __grid_constant__ MeshView m, float* __r
         coef[5] = g.e[6][a] - g.e[2][a] - g.e[4][a];
         coef[6] = g.e[7][a] - g.e[3][a] - g.e[5][a] - g.e[6][a] + g.e[1][a] + g.e[2][a] + g.e[4][a];
       }
-      for (int k = 0; k < NK; ++k) put(D + k * D + a, coef[k]);
+      for (int k = 0; k < NK; ++k) put(a * (NK + 1) + 1 + k, coef[k]);
     }
   }
 }
@@ -135,7 +135,9 @@ __global__ void to_df_nodes_kernel(const double* __restrict__ U, float2* __restr
 // exact; sums and differences carry ~2^-47 of their operands, the order of
 // the storage rounding itself), stored as double-float pairs:
 // per cell and component, slice r (3 in 3D, 1 in 2D) holds C[r][q][p] at
-// pair q*3 + p of 5 float4 (the tenth pair is zero).
+// pair q*3 + p of 5 float4.  In 3D the coefficients that q2_eval_df adds in
+// grid steps (qc_on_grid) are stored biased by the component's grid bias and
+// the tenth pair holds that bias; in 2D the tenth pair is zero.
 __device__ __forceinline__ void t_axis(df v0, df v1, df v2, df& c0, df& c1, df& c2) {
   c0 = v1;
   c1 = df_sub(v2, v0);
@@ -186,13 +188,37 @@ __global__ void __launch_bounds__(32 * D) q2_coeff_kernel(const __grid_constant_
 #pragma unroll
           for (int p = 0; p < 3; ++p) t_axis(V[0][q][p], V[1][q][p], V[2][q][p], V[0][q][p], V[1][q][p], V[2][q][p]);
       }
+      // 3D: the bound of the partial sums of q2_eval_df's grid steps (|s| <= 1/2;
+      // the inner ones without the half, which covers their derivatives)
+      float bias = 0.f;
+      if constexpr (D == 3) {
+        auto A = [&](int p, int q, int r) { return fabsf(V[r][q][p].hi); };
+        float M = A(2, 0, 0), h[3][3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            const float x = (q + r > 0 ? A(1, q, r) : 0.f) + A(2, q, r);
+            h[r][q] = (q + r >= 2 ? A(0, q, r) : 0.f) + 0.5f * x;
+            M = fmaxf(M, q + r >= 2 ? fmaxf(x, h[r][q]) : x);
+          }
+        M = fmaxf(M, fmaxf(h[1][1] + h[1][2], h[2][1] + h[2][2]));
+        M = fmaxf(M, h[2][0] + 0.5f * (h[2][1] + h[2][2]));
+        bias = grid_bias(M);
+      }
       float4* out = sh + (lane * D + comp) * PER;
 #pragma unroll
       for (int r = 0; r < NS; ++r) {
         df pr[10];
 #pragma unroll
-        for (int e = 0; e < 9; ++e) pr[e] = V[r][e / 3][e % 3];
-        pr[9] = df_make(0.f, 0.f);
+        for (int e = 0; e < 9; ++e) {
+          pr[e] = V[r][e / 3][e % 3];
+          if (D == 3 && qc_on_grid(e % 3, e / 3, r)) {
+            const float b = __fadd_rn(bias, pr[e].hi);
+            pr[e] = df_make(b, __fadd_rn(__fsub_rn(pr[e].hi, __fsub_rn(b, bias)), pr[e].lo));
+          }
+        }
+        pr[9] = df_make(bias, 0.f);
         float f[20];  // the ten high parts, then the ten low parts
 #pragma unroll
         for (int e = 0; e < 10; ++e) {
