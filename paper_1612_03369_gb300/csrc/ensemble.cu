@@ -33,13 +33,20 @@ constexpr int kMaxEnsemble = 128;
 constexpr int kEnsBlock = 128;
 constexpr int kMaxBlocksPerSm = 32;  // the hardware's limit of resident blocks
 
-// Resident blocks per SM the ensemble kernels are compiled for (72
-// registers).  On the 64-problem 2D ensemble, 7 against 6: per-step mode
-// 8.48 against 8.65 ms per step, persistent kernel 8.89 against 8.95 ms; 8
-// (64 registers) made the persistent kernel slower (9.19 ms).
-#ifndef PIC_ENSEMBLE_MIN_BLOCKS
-#define PIC_ENSEMBLE_MIN_BLOCKS 7
+// Resident blocks per SM the ensemble kernels are compiled for.  2D: the step
+// waits on loads more than on issue, and 9 blocks (56 registers) of the 64-problem
+// ensemble's ten steps with its export take 80.8 ms against 82.4 at 8, 83.1 at
+// 7, 87.3 at 6 and 82.6 at 10.  3D: 72 registers, as the single-mesh step.
+#ifndef PIC_ENSEMBLE_MIN_BLOCKS_2D
+#define PIC_ENSEMBLE_MIN_BLOCKS_2D 9
 #endif
+#ifndef PIC_ENSEMBLE_MIN_BLOCKS_3D
+#define PIC_ENSEMBLE_MIN_BLOCKS_3D 7
+#endif
+template <int D>
+constexpr int ens_min_blocks() {
+  return D == 2 ? PIC_ENSEMBLE_MIN_BLOCKS_2D : PIC_ENSEMBLE_MIN_BLOCKS_3D;
+}
 
 struct GridBarrier {
   unsigned int count;
@@ -100,20 +107,20 @@ __device__ __forceinline__ int problem_of(const uint32_t* sbase, int P, uint32_t
   return lo;
 }
 
+// The problems' first cells and time steps, searched per particle; the mesh
+// views stay in global memory, where L1 serves them (15 KB for 64 problems,
+// one copy per SM).  A copy of the views per block took 29 KB of shared
+// memory, 206 KB of an SM's 256 KB at 7 blocks, and left the cells' blocks an
+// L1 of 28-50 KB (hit rate 35-53 %).
 struct EnsShared {
-  MeshView views[kMaxEnsemble];
   uint32_t base[kMaxEnsemble + 1];
   df dt[kMaxEnsemble];
 };
 
-__device__ __forceinline__ void load_ensemble(EnsShared& sh, const MeshView* views, const uint32_t* base,
-                                              const df* dts, int P) {
+__device__ __forceinline__ void load_ensemble(EnsShared& sh, const uint32_t* base, const df* dts, int P) {
   for (int q = threadIdx.x; q <= P; q += blockDim.x) {
     sh.base[q] = base[q];
-    if (q < P) {
-      sh.views[q] = views[q];
-      sh.dt[q] = dts[q];
-    }
+    if (q < P) sh.dt[q] = dts[q];
   }
   __syncthreads();
 }
@@ -127,7 +134,8 @@ __device__ __forceinline__ void load_ensemble(EnsShared& sh, const MeshView* vie
 // the way).  Returns the new global cell (PIC_LOST if none); *full is set
 // when the full step ran.
 template <int D, int RK>
-__device__ __forceinline__ uint32_t ensemble_particle(const EnsShared& sh, int P, const StoreView& s,
+__device__ __forceinline__ uint32_t ensemble_particle(const EnsShared& sh, const MeshView* __restrict__ views,
+                                                      int P, const StoreView& s,
                                                       const StoreView& d, const uint32_t* __restrict__ perm, uint32_t j,
                                                       int& iters, unsigned& flags, uint32_t& full) {
   uint32_t i = j, g;
@@ -148,7 +156,7 @@ __device__ __forceinline__ uint32_t ensemble_particle(const EnsShared& sh, int P
     return PIC_LOST;
   }
   const int p = problem_of(sh.base, P, g);
-  const MeshView& m = sh.views[p];
+  const MeshView& m = views[p];
   const uint32_t K = g - sh.base[p];
   uint32_t Kn = advect_particle_cells<D, RK, false, false, NoHook, true>(GlobalCells<D, false>{m}, m, s, i, d, j, K,
                                                                          sh.dt[p], iters, flags);
@@ -168,7 +176,8 @@ __device__ __forceinline__ uint32_t ensemble_particle(const EnsShared& sh, int P
 // counted (warp-aggregated) and written to cell_new.  Warps that finish
 // early take more tiles, so the grid ends together.
 template <int D, int RK>
-__device__ __forceinline__ void ensemble_advect_tiles(const EnsShared& sh, int P, const StoreView& s,
+__device__ __forceinline__ void ensemble_advect_tiles(const EnsShared& sh, const MeshView* __restrict__ views,
+                                                      int P, const StoreView& s,
                                                       const StoreView& d, const uint32_t* __restrict__ perm,
                                                       uint32_t n, uint32_t tile, uint32_t* tile_ctr,
                                                       uint32_t* __restrict__ cell_new, uint32_t* __restrict__ counts,
@@ -191,7 +200,7 @@ __device__ __forceinline__ void ensemble_advect_tiles(const EnsShared& sh, int P
       uint32_t Kc = PIC_LOST, full = 0;
       if (j < end) {
         steps = 1;
-        Kc = ensemble_particle<D, RK>(sh, P, s, d, perm, j, iters, flags, full);
+        Kc = ensemble_particle<D, RK>(sh, views, P, s, d, perm, j, iters, flags, full);
         cell_new[j] = Kc;
         lost = Kc == PIC_LOST ? 1u : 0u;
       }
@@ -208,13 +217,13 @@ __device__ __forceinline__ void ensemble_advect_tiles(const EnsShared& sh, int P
 // Per-step mode: one step's advect over the whole ensemble (tiles from the
 // store's work counter, cleared before the launch).
 template <int D, int RK>
-__global__ void __launch_bounds__(kEnsBlock, PIC_ENSEMBLE_MIN_BLOCKS) ensemble_advect_kernel(
+__global__ void __launch_bounds__(kEnsBlock, ens_min_blocks<D>()) ensemble_advect_kernel(
     const MeshView* __restrict__ views, const uint32_t* __restrict__ base, const df* __restrict__ dts, int P,
     const __grid_constant__ StoreView s, const __grid_constant__ StoreView d, const uint32_t* __restrict__ perm,
     uint32_t tile, uint32_t* __restrict__ cell_new, uint32_t* __restrict__ counts, DevCounters* __restrict__ ctr) {
   __shared__ EnsShared sh;
-  load_ensemble(sh, views, base, dts, P);
-  ensemble_advect_tiles<D, RK>(sh, P, s, d, perm, ctr->n_alive, tile, &ctr->tile_next, cell_new, counts, ctr);
+  load_ensemble(sh, base, dts, P);
+  ensemble_advect_tiles<D, RK>(sh, views, P, s, d, perm, ctr->n_alive, tile, &ctr->tile_next, cell_new, counts, ctr);
 }
 
 struct PersistArgs {
@@ -241,9 +250,9 @@ struct PersistArgs {
 // built, nothing reads them again); the rank.  counts and the tile counters
 // are cleared before the launch.
 template <int D, int RK>
-__global__ void __launch_bounds__(kEnsBlock, PIC_ENSEMBLE_MIN_BLOCKS) ensemble_persistent_kernel(PersistArgs A) {
+__global__ void __launch_bounds__(kEnsBlock, ens_min_blocks<D>()) ensemble_persistent_kernel(PersistArgs A) {
   __shared__ EnsShared sh;
-  load_ensemble(sh, A.views, A.base, A.dts, A.P);
+  load_ensemble(sh, A.base, A.dts, A.P);
   const uint32_t nb = gridDim.x, bid = blockIdx.x;
   const uint32_t gtid = bid * blockDim.x + threadIdx.x, gthreads = nb * blockDim.x;
   // The particles of buffer curb stand in the order of the previous rebin
@@ -254,7 +263,7 @@ __global__ void __launch_bounds__(kEnsBlock, PIC_ENSEMBLE_MIN_BLOCKS) ensemble_p
   bool pending = false;
   uint32_t n = *(volatile uint32_t*)&A.ctr->n_alive;
   for (int step = 0; step < A.n_steps; ++step) {
-    ensemble_advect_tiles<D, RK>(sh, A.P, A.sv[curb], A.sv[pending ? 1 - curb : curb], pending ? A.perm : nullptr, n,
+    ensemble_advect_tiles<D, RK>(sh, A.views, A.P, A.sv[curb], A.sv[pending ? 1 - curb : curb], pending ? A.perm : nullptr, n,
                                  (uint32_t)A.tile, A.tile_ctr + step, A.cell_new, A.counts, A.ctr);
     if (pending) curb = 1 - curb;
     const StoreView& cur = A.sv[curb];
