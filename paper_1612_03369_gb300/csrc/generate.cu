@@ -28,6 +28,7 @@
 #include <cmath>
 #include <cstdlib>
 
+#include "fastpath.cuh"
 #include "pic_internal.cuh"
 #include "seed.cuh"
 
@@ -129,45 +130,185 @@ struct DrawInfo {
   unsigned bad;      // a weight was negative or not finite
 };
 
-// The accumulated weights as one left fold, by one warp: every lane runs the
-// same sequential sum over a 32-value chunk read with one coalesced load
-// (values broadcast by shuffles), lane q keeps the q-th partial sum and the
-// chunk is stored coalesced.  The next chunk is loaded before the fold.
-__global__ void __launch_bounds__(32) accumulate_weights_kernel(const double* __restrict__ w, uint32_t C,
-                                                                double* __restrict__ acc, DrawInfo* __restrict__ info) {
-  const int lane = threadIdx.x;
-  double s = 0.0;
-  long long last = -1;
-  unsigned bad = 0;
-  double next = lane < (int)C ? w[lane] : 0.0;
-  for (uint32_t base = 0; base < C; base += 32) {
-    const double v = next;
-    const uint32_t nb = base + 32 + lane;
-    next = nb < C ? w[nb] : 0.0;
-    const uint32_t k = base + lane;
-    if (k < C) {
-      if (!(v >= 0.0) || !isfinite(v)) bad = 1;
-      if (v > 0.0) last = k;
-    }
-    double mine = 0.0;
-    const int lim = (C - base) < 32u ? (int)(C - base) : 32;
-    for (int q = 0; q < lim; ++q) {
-      s = __dadd_rn(s, __shfl_sync(0xffffffffu, v, q));
-      if (lane == q) mine = s;
-    }
-    if (k < C) acc[k] = mine;
+// The accumulated weights as one left fold, rounded after every addition, by
+// one block.
+//
+// Between two powers of two the running sum S is an integer multiple n of one
+// spacing g = ulp(S), and adding w >= 0 moves it to n + RN(w / g): an integer
+// that does not depend on S, except that a remainder of exactly g / 2 rounds
+// to the even sum, so on n's parity.  So each weight is a pair of increments,
+// one per parity of the sum it meets (FoldInc), pairs compose associatively,
+// and a block scan of 4,096 pairs gives 4,096 sums of the sequential fold at
+// once.  The first sum to reach the next power of two ends the run: it is
+// formed by one rounded addition, and the scan goes on behind it with the new
+// spacing (about log2(C) such breaks).  One warp folding value by value, each
+// addition waiting for the last, took 6.0 ms for 110,592 cells; this 0.07.
+struct FoldInc {
+  unsigned long long d[2];  // increment of n when n is even / odd, at most kFoldCap
+};
+constexpr unsigned long long kFoldTop = 1ull << 53;  // n of the next power of two
+constexpr unsigned long long kFoldCap = 1ull << 54;  // increments saturate here: past kFoldTop only the order counts
+
+__host__ __device__ __forceinline__ unsigned long long fold_cap(unsigned long long v) {
+  return v < kFoldCap ? v : kFoldCap;
+}
+
+// First a, then b.
+__host__ __device__ __forceinline__ FoldInc fold_compose(FoldInc a, FoldInc b) {
+  FoldInc r;
+  r.d[0] = fold_cap(a.d[0] + b.d[a.d[0] & 1u]);
+  r.d[1] = fold_cap(a.d[1] + b.d[(a.d[1] + 1u) & 1u]);
+  return r;
+}
+
+// A non-negative finite double's significand as an integer multiple of
+// 2^(exp - 1075), exp >= 1 (subnormals share the first binade's spacing).
+__host__ __device__ __forceinline__ void fold_split(unsigned long long bits, unsigned long long& n, int& exp) {
+  exp = (int)((bits >> 52) & 0x7ffu);
+  n = bits & ((1ull << 52) - 1);
+  if (exp)
+    n += 1ull << 52;
+  else
+    exp = 1;
+}
+
+// The bits of the sum n 2^(exp - 1075), n < kFoldTop.
+__host__ __device__ __forceinline__ unsigned long long fold_join(unsigned long long n, int exp) {
+  return n < (1ull << 52) ? n : (((unsigned long long)exp << 52) + (n - (1ull << 52)));
+}
+
+// Increments of n by the weight with these bits where the spacing is
+// 2^(exp - 1075).
+__host__ __device__ __forceinline__ FoldInc fold_inc(unsigned long long wbits, int exp) {
+  unsigned long long m;
+  int ew;
+  fold_split(wbits, m, ew);
+  FoldInc r;
+  const int up = ew - exp;
+  if (up >= 0) {
+    r.d[0] = r.d[1] = up >= 2 ? (m ? kFoldCap : 0ull) : fold_cap(m << up);
+    return r;
   }
-  bad = __reduce_or_sync(0xffffffffu, bad);
-  long long lmax = last;
+  const int down = -up;
+  if (down > 54) {
+    r.d[0] = r.d[1] = 0;
+    return r;
+  }
+  const unsigned long long q = m >> down, rem = m & ((1ull << down) - 1), half = 1ull << (down - 1);
+  r.d[0] = q + ((rem > half || (rem == half && (q & 1u))) ? 1u : 0u);
+  r.d[1] = q + ((rem > half || (rem == half && !(q & 1u))) ? 1u : 0u);
+  return r;
+}
+
+constexpr int kFoldThreads = 1024;
+constexpr int kFoldItems = 4;
+
+__device__ __forceinline__ FoldInc fold_shfl_up(FoldInc v, int o) {
+  FoldInc r;
+  r.d[0] = __shfl_up_sync(0xffffffffu, v.d[0], o);
+  r.d[1] = __shfl_up_sync(0xffffffffu, v.d[1], o);
+  return r;
+}
+
+__global__ void __launch_bounds__(kFoldThreads) accumulate_weights_kernel(const double* __restrict__ w, uint32_t C,
+                                                                          double* __restrict__ acc,
+                                                                          DrawInfo* __restrict__ info) {
+  __shared__ FoldInc s_warp[kFoldThreads / 32];
+  __shared__ unsigned long long s_sum;  // bits of the running sum
+  __shared__ uint32_t s_stop;           // first position of the batch that the scan cannot form
+  __shared__ unsigned s_bad;
+  __shared__ uint32_t s_last;           // 1 + last position of a positive weight
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  if (tid == 0) {
+    s_sum = 0;
+    s_bad = 0;
+    s_last = 0;
+  }
+  __syncthreads();
+  for (uint64_t base = 0; base < C;) {
+    const unsigned long long sum = s_sum;
+    unsigned long long n0;
+    int exp;
+    fold_split(sum, n0, exp);
+    if (tid == 0) s_stop = 0xffffffffu;
+    // the batch's weights, kFoldItems consecutive ones per thread; a weight
+    // that is not a finite number >= 0 counts as 0 (the call then fails)
+    unsigned long long wb[kFoldItems];
+    FoldInc inc[kFoldItems], mine;
+    uint32_t pos = 0xffffffffu;  // this thread's first positive weight
+    mine.d[0] = mine.d[1] = 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long other = __shfl_xor_sync(0xffffffffu, lmax, o);
-    lmax = other > lmax ? other : lmax;
+    for (int q = 0; q < kFoldItems; ++q) {
+      const uint64_t k = base + (uint64_t)tid * kFoldItems + q;
+      const double v = k < C ? w[k] : 0.0;
+      const bool good = v >= 0.0 && isfinite(v);
+      if (!good) s_bad = 1;
+      wb[q] = good && v > 0.0 ? (unsigned long long)__double_as_longlong(v) : 0ull;
+      if (wb[q]) {
+        if (pos == 0xffffffffu) pos = tid * kFoldItems + q;
+        atomicMax(&s_last, (uint32_t)k + 1u);
+      }
+      inc[q] = fold_inc(wb[q], exp);
+      mine = fold_compose(mine, inc[q]);
+    }
+    // exclusive composition over the threads before this one
+    FoldInc inc_warp = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const FoldInc v = fold_shfl_up(inc_warp, o);
+      if ((int)lane >= o) inc_warp = fold_compose(v, inc_warp);
+    }
+    if (lane == 31) s_warp[warp] = inc_warp;
+    __syncthreads();
+    if (warp == 0) {
+      FoldInc v = s_warp[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const FoldInc u = fold_shfl_up(v, o);
+        if ((int)lane >= o) v = fold_compose(u, v);
+      }
+      s_warp[lane] = v;
+    }
+    __syncthreads();
+    unsigned long long n = n0;
+    if (warp > 0) n += s_warp[warp - 1].d[n & 1u];
+    const FoldInc before = fold_shfl_up(inc_warp, 1);
+    if (lane > 0) n += before.d[n & 1u];
+    // a sum of zero has no spacing: the first positive weight is the sum
+    const bool zero = sum == 0;
+    uint32_t stop = zero ? pos : 0xffffffffu;
+    unsigned long long nq[kFoldItems];
+#pragma unroll
+    for (int q = 0; q < kFoldItems; ++q) {
+      nq[q] = n;  // the sum that item q meets
+      n += inc[q].d[n & 1u];
+      if (!zero && n >= kFoldTop && stop == 0xffffffffu) stop = tid * kFoldItems + q;
+    }
+    if (stop != 0xffffffffu) atomicMin(&s_stop, stop);
+    __syncthreads();
+    const uint32_t end = s_stop;
+#pragma unroll
+    for (int q = 0; q < kFoldItems; ++q) {
+      const uint32_t i = tid * kFoldItems + q;
+      const uint64_t k = base + i;
+      if (k >= C || i > end) continue;
+      const unsigned long long after = q + 1 < kFoldItems ? nq[q + 1 < kFoldItems ? q + 1 : q] : n;
+      unsigned long long bits = zero ? 0ull : fold_join(after, exp);
+      if (i == end)
+        bits = (unsigned long long)__double_as_longlong(
+            __dadd_rn(__longlong_as_double((long long)(zero ? 0ull : fold_join(nq[q], exp))),
+                      __longlong_as_double((long long)wb[q])));
+      acc[k] = __longlong_as_double((long long)bits);
+      if (i == end || (end == 0xffffffffu && (k + 1 == C || i + 1 == kFoldThreads * kFoldItems))) s_sum = bits;
+    }
+    __syncthreads();
+    base += end == 0xffffffffu ? (uint64_t)(kFoldThreads * kFoldItems) : (uint64_t)end + 1u;
+    if (((s_sum >> 52) & 0x7ffu) == 0x7ffu) break;  // overflowed: the call fails
   }
-  if (lane == 0) {
-    info->W = s;
-    info->last = lmax;
-    info->bad = bad;
+  if (tid == 0) {
+    info->W = __longlong_as_double((long long)s_sum);
+    info->last = (long long)s_last - 1;
+    info->bad = s_bad;
   }
 }
 
@@ -196,49 +337,177 @@ __global__ void __launch_bounds__(256) draw_cells_kernel(const double* __restric
 
 // ------------------------------------------------------ Metropolis-Hastings
 
+// A point of the unit cell as the generator's raw outputs (coordinate a is
+// unit53(r[a])).
+template <int D>
+struct RawPoint {
+  uint64_t r[D];
+};
+
+template <int D>
+__device__ __forceinline__ void raw_coordinates(RawPoint<D> p, double t[D]) {
+#pragma unroll
+  for (int a = 0; a < D; ++a) t[a] = unit53(p.r[a]);
+}
+
+// The acceptance test as defined: u rho-hat(current) < rho-hat(proposal) in
+// the written sequence of IEEE operations.
+template <int D>
+__device__ __noinline__ bool mh_accept_rn(const MeshView& m, uint32_t K, const double* __restrict__ rho, RawPoint<D> cur,
+                                          RawPoint<D> prop, bool at_centre, double u) {
+  double t[D], y[D];
+  raw_coordinates<D>(cur, t);
+  if (at_centre)
+#pragma unroll
+    for (int a = 0; a < D; ++a) t[a] = 0.5;
+  raw_coordinates<D>(prop, y);
+  const double rc = rho_hat_rn<D>(m, K, rho, t), ry = rho_hat_rn<D>(m, K, rho, y);
+  return __dmul_rn(u, rc) < ry;
+}
+
+// Writes particle q of cell K at the chain's state.  Out of line: its two dozen
+// FP64 vertex values would otherwise be held through the steps.
+template <int D>
+__device__ __noinline__ void mh_emit(const MeshView& m, const StoreView& s, uint32_t K, RawPoint<D> cur, bool at_centre,
+                                     uint32_t q, uint64_t id) {
+  double t[D], x[D];
+  raw_coordinates<D>(cur, t);
+  if (at_centre)
+#pragma unroll
+    for (int a = 0; a < D; ++a) t[a] = 0.5;
+  phi_rn<D>(m, K, t, x);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    s.x[a * s.cap + q] = x[a];
+    const float hi = __double2float_rn(t[a]);
+    s.xhat[a * s.cap + q] = make_float2(hi, __double2float_rn(t[a] - (double)hi));
+  }
+  s.id[q] = id;
+  s.cell[q] = K;
+  for (int p = 0; p < s.n_props; ++p) s.props[(size_t)p * s.cap + q] = 0.0;
+}
+
+// rho-hat in FP32, with a bound of its error: the density's monomial
+// coefficients in the cell and the rows of the map's Jacobian.
+template <int D>
+struct RhoHat32 {
+  float c[1 << D];      // 1, t0, t1, (t2,) mixed ones
+  MapRow<D> row[D];
+  float tau;            // |rho-hat in FP32 - rho-hat| for t within 2^-24 of the given one
+
+  __device__ __forceinline__ void load(const MeshView& m, uint32_t K, const double* __restrict__ rho) {
+    int ijk[3];
+    cell_ijk<D>(m, K, ijk);
+    double v[1 << D];
+#pragma unroll
+    for (int q = 0; q < (1 << D); ++q) v[q] = __ldg(rho + local_vertex<D>(m, ijk, q));
+    // differences along each axis: v[q] becomes the coefficient of the monomial
+    // with the axes of q's set bits
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+#pragma unroll
+      for (int q = 0; q < (1 << D); ++q)
+        if ((q >> a) & 1) v[q] -= v[q & ~(1 << a)];
+    constexpr int order[8] = {0, 1, 2, D == 2 ? 3 : 4, 3, 5, 6, 7};  // as mixed32 orders the monomials
+    float R = 0.f;
+#pragma unroll
+    for (int q = 0; q < (1 << D); ++q) {
+      c[q] = (float)v[order[q]];
+      R += fabsf(c[q]);
+    }
+    const GlobalCells<D, false> cs{m};
+    const float4* B = cs.block(K);
+    float S = 1.f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      row[a] = load_row<D>(cs, B, 0, a);
+      float r = 0.f;  // bounds every entry of the row
+#pragma unroll
+      for (int k = 0; k < (1 << D) - 1; ++k) r += fabsf(row[a].a[k]);
+      S *= r;
+    }
+    // With s_i the bound of row i and e = 2^-24: every entry of J is off by at
+    // most 7 e s_i (coefficient, coordinate and FMA roundings), the determinant,
+    // a sum of D! products, by 26 e D! s_0..s_(D-1), rho_h by 11 e R; the product
+    // by less than 256 e R S.  Doubled.
+    tau = 0x1p-15f * R * S;
+  }
+
+  __device__ __forceinline__ float at(const float t[D]) const {
+    float m[4], J[D][D], r;
+    mixed32<D>(t, m);
+    if constexpr (D == 2) {
+      r = c[0] + (c[1] * t[0] + (c[2] * t[1] + c[3] * m[0]));
+    } else {
+      r = c[0] + (c[1] * t[0] + (c[2] * t[1] + (c[3] * t[2] + (c[4] * m[0] + (c[5] * m[1] + (c[6] * m[2] + c[7] * m[3]))))));
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) jacobian_row32<D>(row[i], t, m, J[i]);
+    float det;
+    if constexpr (D == 2)
+      det = J[0][0] * J[1][1] - J[0][1] * J[1][0];
+    else
+      det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) + J[0][1] * (J[1][2] * J[2][0] - J[1][0] * J[2][2]) +
+            J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
+    return r * fabsf(det);
+  }
+};
+
 // Thread per cell: the cell's chain, started at the centre; step st of the
 // chain is global step g = J * cell_off[K] + st and uses SplitMix64 outputs
 // g (D+1) + a (proposal coordinate a) and g (D+1) + D (acceptance uniform).
 // States J, 2J, ... become the cell's particles, in order.
+//
+// A step only needs the sign of u rho-hat(current) - rho-hat(proposal).  It is
+// taken from FP32 values where they differ by more than their error bound, and
+// from the written IEEE sequence otherwise (about one step in 10^4), so the
+// decisions are those of the sequence.  Evaluating the sequence at every
+// proposal, 239 FP64 operations, held the FP64 pipe 83 % busy: 12.8 ms for
+// 1.77 M particles at J = 8.
 template <int D>
-__global__ void __launch_bounds__(128) mh_seed_kernel(const __grid_constant__ MeshView m, const __grid_constant__ StoreView s, const uint32_t* __restrict__ cell_off,
+__global__ void __launch_bounds__(128, 5) mh_seed_kernel(const __grid_constant__ MeshView m, const __grid_constant__ StoreView s, const uint32_t* __restrict__ cell_off,
                                                       const double* __restrict__ rho, uint32_t J, uint64_t seed,
                                                       uint64_t first_id) {
+  constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
   for (uint32_t K = blockIdx.x * blockDim.x + threadIdx.x; K < m.C; K += gridDim.x * blockDim.x) {
     const uint32_t beg = cell_off[K], end = cell_off[K + 1];
     if (end > s.cap || beg >= end) continue;
-    double cur[D];
+    RhoHat32<D> f;
+    f.load(m, K, rho);
+    const float sure = 2.5f * f.tau;
+    RawPoint<D> cur;
+    float t32[D];
 #pragma unroll
-    for (int a = 0; a < D; ++a) cur[a] = 0.5;
-    double rc = rho_hat_rn<D>(m, K, rho, cur);
+    for (int a = 0; a < D; ++a) {
+      cur.r[a] = 0;
+      t32[a] = 0.5f;
+    }
+    bool at_centre = true;
+    float rc = f.at(t32);
     const uint64_t g0 = (uint64_t)J * beg, len = (uint64_t)J * (end - beg);
+    uint64_t z = seed + g0 * (D + 1) * kGamma;  // the generator's state before the step's first output
     uint32_t q = beg;
     uint32_t phase = 0;
     for (uint64_t st = 0; st < len; ++st) {
-      const uint64_t g = g0 + st;
-      double y[D];
+      RawPoint<D> y;
 #pragma unroll
-      for (int a = 0; a < D; ++a) y[a] = unit53(splitmix64_at(seed, g * (D + 1) + a));
-      const double u = unit53(splitmix64_at(seed, g * (D + 1) + D));
-      const double ry = rho_hat_rn<D>(m, K, rho, y);
-      if (__dmul_rn(u, rc) < ry) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) cur[a] = y[a];
+      for (int a = 0; a < D; ++a) {
+        y.r[a] = splitmix64_mix(z += kGamma);
+        t32[a] = (float)(uint32_t)(y.r[a] >> 40) * 0x1p-24f;
+      }
+      const uint64_t ur = splitmix64_mix(z += kGamma);
+      const float ry = f.at(t32);
+      const float diff = ry - (float)(uint32_t)(ur >> 40) * 0x1p-24f * rc;
+      bool accept = diff > sure;
+      if (!(fabsf(diff) > sure)) accept = mh_accept_rn<D>(m, K, rho, cur, y, at_centre, unit53(ur));
+      if (accept) {
+        cur = y;
         rc = ry;
+        at_centre = false;
       }
       if (++phase == J) {
         phase = 0;
-        double x[D];
-        phi_rn<D>(m, K, cur, x);
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-          s.x[a * s.cap + q] = x[a];
-          const float hi = __double2float_rn(cur[a]);
-          s.xhat[a * s.cap + q] = make_float2(hi, __double2float_rn(cur[a] - (double)hi));
-        }
-        s.id[q] = first_id + q;
-        s.cell[q] = K;
-        for (int p = 0; p < s.n_props; ++p) s.props[(size_t)p * s.cap + q] = 0.0;
+        mh_emit<D>(m, s, K, cur, at_centre, q, first_id + q);
         ++q;
       }
     }
@@ -319,7 +588,7 @@ extern "C" pic_status pic_draw_cell_counts(uint32_t n_cells, const double* w, ui
     cudaFree(info);
     return (set_error("pic_draw_cell_counts: device allocation failed"), PIC_ERR_OOM);
   }
-  accumulate_weights_kernel<<<1, 32, 0, st>>>(w, n_cells, acc, info);
+  accumulate_weights_kernel<<<1, kFoldThreads, 0, st>>>(w, n_cells, acc, info);
   DrawInfo h{};
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, info, sizeof(h), cudaMemcpyDeviceToHost, st);

@@ -9,11 +9,13 @@ namespace pic {
 // SplitMix64 (Steele, Lea & Flood, OOPSLA 2014) used as a counter-based
 // generator: output n of the stream seeded with `seed` is the finaliser
 // applied to seed + (n + 1) * 0x9E3779B97F4A7C15.
-__device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t n) {
-  uint64_t z = seed + (n + 1ull) * 0x9E3779B97F4A7C15ull;
+__device__ __forceinline__ uint64_t splitmix64_mix(uint64_t z) {
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
   z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
   return z ^ (z >> 31);
+}
+__device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t n) {
+  return splitmix64_mix(seed + (n + 1ull) * 0x9E3779B97F4A7C15ull);
 }
 
 static __global__ void fill_counts_kernel(const uint32_t* __restrict__ per_cell, uint32_t uniform, uint32_t* __restrict__ counts,
