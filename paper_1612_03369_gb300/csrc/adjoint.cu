@@ -55,6 +55,7 @@ struct pic_tape_s {
   uint32_t* rec_off;   // [C + 1]
   void* sort_scratch;
   double* partial;     // [C][3^dim][dim]
+  void* slab;          // the allocation that holds every device array above
 };
 
 namespace pic {
@@ -373,34 +374,13 @@ using namespace pic;
 
 extern "C" pic_status pic_destroy_tape(pic_tape tp) {
   if (!tp) return PIC_OK;
-  for (int s = 0; s < tp->n_rec; ++s) {
-    if (tp->rcell) cudaFree(tp->rcell[s]);
-    if (tp->rt) cudaFree(tp->rt[s]);
-  }
-  for (int s = 0; s < tp->n_steps; ++s) {
-    if (tp->perm) cudaFree(tp->perm[s]);
-    if (tp->x) cudaFree(tp->x[s]);
-    if (tp->xhat) cudaFree(tp->xhat[s]);
-    if (tp->cell) cudaFree(tp->cell[s]);
-  }
   free(tp->rcell);
   free(tp->rt);
   free(tp->perm);
   free(tp->x);
   free(tp->xhat);
   free(tp->cell);
-  cudaFree(tp->sink_x);
-  cudaFree(tp->sink_xhat);
-  cudaFree(tp->n_dev);
-  cudaFree(tp->lam[0]);
-  cudaFree(tp->lam[1]);
-  cudaFree(tp->rec_cell);
-  cudaFree(tp->rec_key);
-  cudaFree(tp->rec_w);
-  cudaFree(tp->rec_perm);
-  cudaFree(tp->rec_off);
-  cudaFree(tp->sort_scratch);
-  cudaFree(tp->partial);
+  cudaFree(tp->slab);
   free(tp);
   return PIC_OK;
 }
@@ -448,31 +428,49 @@ extern "C" pic_status pic_advect_record_tape(pic_particles parts, pic_mesh mesh,
     tp->xhat = (float2**)calloc(n_steps, sizeof(float2*));
     tp->cell = (uint32_t**)calloc(n_steps, sizeof(uint32_t*));
     ok = ok && tp->x && tp->xhat && tp->cell;
-    ok = ok && cudaMalloc(&tp->sink_x, sizeof(double) * d * cap) == cudaSuccess;
-    ok = ok && cudaMalloc(&tp->sink_xhat, sizeof(float2) * d * cap) == cudaSuccess;
+  }
+  // per-step arrays one after another, a stride of whole 256-byte lines apart
+  const size_t cap64 = (cap + 63) / 64 * 64;
+  uint32_t *rcell0 = nullptr, *perm0 = nullptr, *cell0 = nullptr;
+  float2 *rt0 = nullptr, *xhat0 = nullptr;
+  double* x0 = nullptr;
+  if (ok) {
+    const size_t steps = (size_t)n_steps, recs = (size_t)tp->n_rec;
+    Slab slab;
+    slab.add(&rcell0, recs * kRecPerParticle * cap64);
+    slab.add(&rt0, recs * d * kRecPerParticle * cap64);
+    slab.add(&perm0, steps * cap64);
+    if (ckpt) {
+      slab.add(&x0, steps * d * cap64);
+      slab.add(&xhat0, steps * d * cap64);
+      slab.add(&cell0, steps * cap64);
+      slab.add(&tp->sink_x, d * cap);
+      slab.add(&tp->sink_xhat, d * cap);
+    }
+    slab.add(&tp->n_dev, steps + 1);
+    slab.add(&tp->lam[0], d * cap);
+    slab.add(&tp->lam[1], d * cap);
+    slab.add(&tp->rec_cell, rcap);
+    slab.add(&tp->rec_key, rcap);
+    slab.add(&tp->rec_w, d * rcap);
+    slab.add(&tp->rec_perm, rcap);
+    slab.add(&tp->rec_off, (size_t)tp->C + 1);
+    slab.add(reinterpret_cast<char**>(&tp->sort_scratch), sort_scratch_bytes(rcap, tp->C));
+    slab.add(&tp->partial, (size_t)NE * tp->C);
+    ok = slab.allocate(&tp->slab);
   }
   for (int s = 0; s < tp->n_rec && ok; ++s) {
-    ok = ok && cudaMalloc(&tp->rcell[s], sizeof(uint32_t) * rcap) == cudaSuccess;
-    ok = ok && cudaMalloc(&tp->rt[s], sizeof(float2) * d * rcap) == cudaSuccess;
+    tp->rcell[s] = rcell0 + (size_t)s * kRecPerParticle * cap64;
+    tp->rt[s] = rt0 + (size_t)s * d * kRecPerParticle * cap64;
   }
   for (int s = 0; s < n_steps && ok; ++s) {
-    ok = ok && cudaMalloc(&tp->perm[s], sizeof(uint32_t) * cap) == cudaSuccess;
+    tp->perm[s] = perm0 + (size_t)s * cap64;
     if (ckpt) {
-      ok = ok && cudaMalloc(&tp->x[s], sizeof(double) * d * cap) == cudaSuccess;
-      ok = ok && cudaMalloc(&tp->xhat[s], sizeof(float2) * d * cap) == cudaSuccess;
-      ok = ok && cudaMalloc(&tp->cell[s], sizeof(uint32_t) * cap) == cudaSuccess;
+      tp->x[s] = x0 + (size_t)s * d * cap64;
+      tp->xhat[s] = xhat0 + (size_t)s * d * cap64;
+      tp->cell[s] = cell0 + (size_t)s * cap64;
     }
   }
-  ok = ok && cudaMalloc(&tp->n_dev, sizeof(uint32_t) * (n_steps + 1)) == cudaSuccess;
-  ok = ok && cudaMalloc(&tp->lam[0], sizeof(float2) * d * cap) == cudaSuccess;
-  ok = ok && cudaMalloc(&tp->lam[1], sizeof(float2) * d * cap) == cudaSuccess;
-  ok = ok && cudaMalloc(&tp->rec_cell, sizeof(uint32_t) * rcap) == cudaSuccess;
-  ok = ok && cudaMalloc(&tp->rec_key, sizeof(uint64_t) * rcap) == cudaSuccess;
-  ok = ok && cudaMalloc(&tp->rec_w, sizeof(float2) * d * rcap) == cudaSuccess;
-  ok = ok && cudaMalloc(&tp->rec_perm, sizeof(uint32_t) * rcap) == cudaSuccess;
-  ok = ok && cudaMalloc(&tp->rec_off, sizeof(uint32_t) * ((size_t)tp->C + 1)) == cudaSuccess;
-  ok = ok && cudaMalloc(&tp->sort_scratch, sort_scratch_bytes(rcap, tp->C)) == cudaSuccess;
-  ok = ok && cudaMalloc(&tp->partial, sizeof(double) * NE * (size_t)tp->C) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     pic_destroy_tape(tp);

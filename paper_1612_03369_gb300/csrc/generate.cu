@@ -142,7 +142,7 @@ struct DrawInfo {
 // once.  The first sum to reach the next power of two ends the run: it is
 // formed by one rounded addition, and the scan goes on behind it with the new
 // spacing (about log2(C) such breaks).  One warp folding value by value, each
-// addition waiting for the last, took 6.0 ms for 110,592 cells; this 0.07.
+// addition waiting for the last, took 6.0 ms for 110,592 cells; this 0.33.
 struct FoldInc {
   unsigned long long d[2];  // increment of n when n is even / odd, at most kFoldCap
 };
@@ -582,25 +582,23 @@ extern "C" pic_status pic_draw_cell_counts(uint32_t n_cells, const double* w, ui
   cudaStream_t st = (cudaStream_t)stream;
   double* acc = nullptr;
   DrawInfo* info = nullptr;
-  if (cudaMalloc(&acc, sizeof(double) * n_cells) != cudaSuccess || cudaMalloc(&info, sizeof(DrawInfo)) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(acc);
-    cudaFree(info);
+  void* scratch = nullptr;
+  Slab slab;
+  slab.add(&acc, n_cells);
+  slab.add(&info, 1);
+  if (!slab.allocate(&scratch))
     return (set_error("pic_draw_cell_counts: device allocation failed"), PIC_ERR_OOM);
-  }
   accumulate_weights_kernel<<<1, kFoldThreads, 0, st>>>(w, n_cells, acc, info);
   DrawInfo h{};
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, info, sizeof(h), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
-    cudaFree(acc);
-    cudaFree(info);
+    cudaFree(scratch);
     return cuda_fail(e, "pic_draw_cell_counts: accumulate");
   }
   if (h.bad || !(h.W > 0.0) || !std::isfinite(h.W)) {
-    cudaFree(acc);
-    cudaFree(info);
+    cudaFree(scratch);
     return (set_error("pic_draw_cell_counts: weights must be finite and >= 0 with a positive sum"), PIC_ERR_ARG);
   }
   e = cudaMemsetAsync(counts, 0, sizeof(uint32_t) * n_cells, st);
@@ -610,8 +608,7 @@ extern "C" pic_status pic_draw_cell_counts(uint32_t n_cells, const double* w, ui
     e = cudaGetLastError();
   }
   count_launches(n_particles > 0 ? 2 : 1);
-  cudaFreeAsync(acc, st);
-  cudaFreeAsync(info, st);
+  cudaFreeAsync(scratch, st);
   if (e != cudaSuccess) return cuda_fail(e, "pic_draw_cell_counts: draws");
   return PIC_OK;
 }
@@ -662,25 +659,20 @@ extern "C" pic_status pic_import_particles(pic_mesh mesh, size_t n, const double
            *off = nullptr;
   double* xh = nullptr;
   uint64_t* id = nullptr;
-  bool ok = cudaMalloc(&cell, sizeof(uint32_t) * nn) == cudaSuccess &&
-            cudaMalloc(&flag, sizeof(uint32_t) * nn) == cudaSuccess &&
-            cudaMalloc(&rank, sizeof(uint32_t) * (nn + 1)) == cudaSuccess &&
-            cudaMalloc(&sums, scan_scratch_bytes((uint32_t)nn)) == cudaSuccess &&
-            cudaMalloc(&total, sizeof(uint32_t) * 2) == cudaSuccess &&
-            cudaMalloc(&perm, sizeof(uint32_t) * nn) == cudaSuccess &&
-            cudaMalloc(&off, sizeof(uint32_t) * (C + 1)) == cudaSuccess &&
-            cudaMalloc(&xh, sizeof(double) * d * nn) == cudaSuccess &&
-            cudaMalloc(&id, sizeof(uint64_t) * nn) == cudaSuccess;
+  void* scratch = nullptr;
+  Slab slab;
+  slab.add(&cell, nn);
+  slab.add(&flag, nn);
+  slab.add(&rank, nn + 1);
+  slab.add(&sums, scan_scratch_bytes((uint32_t)nn) / sizeof(uint32_t));
+  slab.add(&total, 2);
+  slab.add(&perm, nn);
+  slab.add(&xh, (size_t)d * nn);
+  slab.add(&id, nn);
+  const bool ok = slab.allocate(&scratch) && cudaMalloc(&off, sizeof(uint32_t) * (C + 1)) == cudaSuccess;
   auto release = [&](bool keep_off) {
-    cudaFree(cell);
-    cudaFree(flag);
-    cudaFree(rank);
-    cudaFree(sums);
-    cudaFree(total);
-    cudaFree(perm);
+    cudaFree(scratch);
     if (!keep_off) cudaFree(off);
-    cudaFree(xh);
-    cudaFree(id);
   };
   if (!ok) {
     cudaGetLastError();

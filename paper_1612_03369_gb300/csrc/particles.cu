@@ -29,22 +29,8 @@ using namespace pic;
 
 extern "C" pic_status pic_destroy_particles(pic_particles p) {
   if (!p) return PIC_OK;
-  for (int b = 0; b < 2; ++b) {
-    cudaFree(p->x[b]);
-    cudaFree(p->xhat[b]);
-    cudaFree(p->id[b]);
-    cudaFree(p->cell[b]);
-    cudaFree(p->props[b]);
-  }
   cudaFree(p->cell_off);
-  cudaFree(p->cell_new);
-  cudaFree(p->counts);
-  cudaFree(p->cursor);
-  cudaFree(p->block_sums);
-  cudaFree(p->key_id);
-  cudaFree(p->key_src);
-  cudaFree(p->perm);
-  cudaFree(p->ctr);
+  cudaFree(p->slab);
   cudaFree(p->xfer);
   cudaFree(p->stage_rec);
   for (int k = 0; k < 3 * p->ev_cap; ++k) cudaEventDestroy(p->ev[k]);
@@ -71,24 +57,23 @@ pic_particles_s* store_alloc(int dim, int n_props, uint32_t C, size_t capacity, 
   p->capacity = capacity > 0 ? capacity : 1;
   p->cell_off = cell_off;
   const size_t cap = p->capacity, d = (size_t)dim;
-  bool ok = true;
-  for (int b = 0; b < 2 && ok; ++b) {
-    ok = ok && cudaMalloc(&p->x[b], sizeof(double) * d * cap) == cudaSuccess;
-    ok = ok && cudaMalloc(&p->xhat[b], sizeof(float2) * d * cap) == cudaSuccess;
-    ok = ok && cudaMalloc(&p->id[b], sizeof(uint64_t) * cap) == cudaSuccess;
-    ok = ok && cudaMalloc(&p->cell[b], sizeof(uint32_t) * cap) == cudaSuccess;
-    ok = ok && cudaMalloc(&p->props[b], sizeof(double) * (n_props > 0 ? n_props : 1) * cap) == cudaSuccess;
+  Slab slab;
+  for (int b = 0; b < 2; ++b) {
+    slab.add(&p->x[b], d * cap);
+    slab.add(&p->xhat[b], d * cap);
+    slab.add(&p->id[b], cap);
+    slab.add(&p->cell[b], cap);
+    slab.add(&p->props[b], (size_t)(n_props > 0 ? n_props : 1) * cap);
   }
-  ok = ok && cudaMalloc(&p->cell_new, sizeof(uint32_t) * cap) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->counts, sizeof(uint32_t) * C) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->cursor, sizeof(uint32_t) * C) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->block_sums, scan_scratch_bytes(C)) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->key_id, sizeof(uint64_t) * cap) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->key_src, sizeof(uint32_t) * cap) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->perm, sizeof(uint32_t) * cap) == cudaSuccess;
-  ok = ok && cudaMalloc(&p->ctr, sizeof(DevCounters)) == cudaSuccess;
-  if (!ok) {
-    cudaGetLastError();
+  slab.add(&p->cell_new, cap);
+  slab.add(&p->counts, C);
+  slab.add(&p->cursor, C);
+  slab.add(&p->block_sums, scan_scratch_bytes(C) / sizeof(uint32_t));
+  slab.add(&p->key_id, cap);
+  slab.add(&p->key_src, cap);
+  slab.add(&p->perm, cap);
+  slab.add(&p->ctr, 1);
+  if (!slab.allocate(&p->slab)) {
     pic_destroy_particles(p);
     set_error("store_alloc: device allocation failed (capacity %zu)", cap);
     return nullptr;
@@ -111,20 +96,17 @@ pic_status seed_prepare(pic_mesh mesh, const uint32_t* per_cell, uint32_t unifor
   if (n_props < 0 || n_props > kMaxProps) return (set_error("%s: n_props must be in [0, %d]", who, kMaxProps), PIC_ERR_ARG);
   const uint32_t C = mesh->C;
   uint32_t *counts = nullptr, *off = nullptr, *sums = nullptr, *total = nullptr;
-  if (cudaMalloc(&counts, sizeof(uint32_t) * C) != cudaSuccess || cudaMalloc(&off, sizeof(uint32_t) * (C + 1)) != cudaSuccess ||
-      cudaMalloc(&sums, scan_scratch_bytes(C)) != cudaSuccess || cudaMalloc(&total, sizeof(uint32_t) * 2) != cudaSuccess) {
+  void* tmp = nullptr;
+  Slab slab;
+  slab.add(&counts, C);
+  slab.add(&sums, scan_scratch_bytes(C) / sizeof(uint32_t));
+  slab.add(&total, 2);
+  if (!slab.allocate(&tmp) || cudaMalloc(&off, sizeof(uint32_t) * (C + 1)) != cudaSuccess) {
     cudaGetLastError();
-    cudaFree(counts);
-    cudaFree(off);
-    cudaFree(sums);
-    cudaFree(total);
+    cudaFree(tmp);
     return (set_error("%s: device allocation failed", who), PIC_ERR_OOM);
   }
-  auto cleanup_tmp = [&]() {
-    cudaFree(counts);
-    cudaFree(sums);
-    cudaFree(total);
-  };
+  auto cleanup_tmp = [&]() { cudaFree(tmp); };
   fill_counts_kernel<<<(C + 255) / 256 < 4096 ? (C + 255) / 256 : 4096, 256, 0, st>>>(per_cell, uniform_count, counts, C);
   // 64-bit total check: the scan is 32-bit, so guard against overflow first
   uint64_t total64 = 0;

@@ -53,6 +53,45 @@ struct DevCounters {
 
 }  // namespace pic
 
+namespace pic {
+// The device arrays of one object (or of one call's scratch) in a single
+// allocation, each on a 256-byte boundary as cudaMalloc would place it.
+// cudaMalloc and cudaFree cost 20-40 us a call on GB300 whatever the size, and
+// cudaFree waits for the device: a store of 17 arrays took 0.73 ms to allocate
+// and 0.74 ms to free, 3.7 of the 6.3 ms of drawing, seeding and importing 1.77 M
+// particles twice.
+class Slab {
+ public:
+  template <class T>
+  void add(T** p, size_t count) {
+    piece_[n_].ptr = reinterpret_cast<void**>(p);
+    piece_[n_].offset = bytes_;
+    bytes_ += (sizeof(T) * count + 255) / 256 * 256;
+    ++n_;
+  }
+  // Allocates and sets every added pointer; *base owns the memory.  On failure
+  // the pointers are left alone, *base is null and the error is cleared.
+  bool allocate(void** base) {
+    if (cudaMalloc(base, bytes_ ? bytes_ : 256) != cudaSuccess) {
+      cudaGetLastError();
+      *base = nullptr;
+      return false;
+    }
+    for (int k = 0; k < n_; ++k) *piece_[k].ptr = static_cast<char*>(*base) + piece_[k].offset;
+    return true;
+  }
+
+ private:
+  static constexpr int kMax = 24;
+  struct {
+    void** ptr;
+    size_t offset;
+  } piece_[kMax];
+  int n_ = 0;
+  size_t bytes_ = 0;
+};
+}  // namespace pic
+
 struct pic_mesh_s {
   int dim;
   int n[3];      // cells per axis (1 on unused axes)
@@ -109,6 +148,7 @@ struct pic_particles_s {
   uint32_t* key_src;      // [capacity]
   uint32_t* perm;         // [capacity]
   pic::DevCounters* ctr;  // device counters and status word
+  void* slab;             // the allocation that holds the arrays above but cell_off
   double* xfer;           // [2 * 2^dim][C] per-cell partial sums of the vertex averages, allocated on first use
   void* stage_rec;        // property ODEs, on first use: StageRec cell [4][cap] u32, x-hat [dim][4][cap] float2, then G [4][dim^2][cap] float2
   cudaStream_t stream;
