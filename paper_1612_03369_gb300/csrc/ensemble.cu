@@ -293,20 +293,6 @@ __global__ void barrier_selftest_kernel(GridBarrier* b, unsigned long long timeo
   (void)grid_sync(b, gridDim.x + 1, timeout_ns);
 }
 
-__global__ void xhat_pairs_kernel(const float2* __restrict__ src, double* __restrict__ dst, size_t n, size_t cap,
-                                  size_t beg, int dim) {
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n * dim; q += (size_t)gridDim.x * blockDim.x) {
-    const size_t a = q / n, j = q % n;
-    const float2 v = src[a * cap + beg + j];
-    dst[q] = (double)v.x + (double)v.y;
-  }
-}
-
-__global__ void local_cells_kernel(const uint32_t* __restrict__ src, uint32_t* __restrict__ dst, uint32_t n,
-                                   uint32_t base) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i] - base;
-}
-
 }  // namespace pic
 
 using namespace pic;
@@ -840,27 +826,29 @@ extern "C" pic_status pic_ensemble_export(pic_ensemble e, int problem, double* x
   cudaStream_t st = (cudaStream_t)stream;
   pic_particles_s* s = e->store;
   PIC_CUDA(cudaDeviceSynchronize());
+  // the segment's two ends, as the rows of one strided copy where the stride is
+  // a pitch that the copy can take
   uint32_t r[2];
-  PIC_CUDA(cudaMemcpy(&r[0], s->cell_off + e->base_host[problem], sizeof(uint32_t), cudaMemcpyDeviceToHost));
-  PIC_CUDA(cudaMemcpy(&r[1], s->cell_off + e->base_host[problem + 1], sizeof(uint32_t), cudaMemcpyDeviceToHost));
+  const uint32_t* ends = s->cell_off + e->base_host[problem];
+  const size_t cells = e->base_host[problem + 1] - e->base_host[problem], pitch = sizeof(uint32_t) * cells;
+  if (pitch < (1u << 30)) {
+    PIC_CUDA(cudaMemcpy2D(r, sizeof(uint32_t), ends, pitch, sizeof(uint32_t), 2, cudaMemcpyDeviceToHost));
+  } else {
+    PIC_CUDA(cudaMemcpy(&r[0], ends, sizeof(uint32_t), cudaMemcpyDeviceToHost));
+    PIC_CUDA(cudaMemcpy(&r[1], ends + cells, sizeof(uint32_t), cudaMemcpyDeviceToHost));
+  }
   const size_t beg = r[0], n = r[1] - r[0], cap = s->capacity;
   if (n_out) *n_out = n;
-  if (n == 0) return PIC_OK;
+  if (n == 0 || (!x && !xhat && !id && !cell)) return PIC_OK;
   const int c = s->cur;
-  for (int a = 0; a < e->dim; ++a) {
-    if (x) PIC_CUDA(cudaMemcpyAsync(x + a * n, s->x[c] + a * cap + beg, sizeof(double) * n, cudaMemcpyDefault, st));
-  }
-  if (xhat) {
-    xhat_pairs_kernel<<<1024, 256, 0, st>>>(s->xhat[c], xhat, n, cap, beg, e->dim);
-    PIC_CUDA(cudaGetLastError());
-  }
-  if (id) PIC_CUDA(cudaMemcpyAsync(id, s->id[c] + beg, sizeof(uint64_t) * n, cudaMemcpyDefault, st));
-  if (cell) {
-    local_cells_kernel<<<(int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096), 256, 0, st>>>(s->cell[c] + beg, cell,
-                                                                                                (uint32_t)n,
-                                                                                                e->base_host[problem]);
-    PIC_CUDA(cudaGetLastError());
-  }
+  // device arrays in one kernel; x and id may also be host arrays, copied
+  const bool hx = x && !on_device(x), hid = id && !on_device(id);
+  for (int a = 0; a < e->dim && hx; ++a)
+    PIC_CUDA(cudaMemcpyAsync(x + a * n, s->x[c] + a * cap + beg, sizeof(double) * n, cudaMemcpyDefault, st));
+  if (hid) PIC_CUDA(cudaMemcpyAsync(id, s->id[c] + beg, sizeof(uint64_t) * n, cudaMemcpyDefault, st));
+  launch_pack(s, c, nullptr, beg, n, e->base_host[problem],
+              PackedOut{hx ? nullptr : x, xhat, hid ? nullptr : id, cell, nullptr}, st);
+  PIC_CUDA(cudaGetLastError());
   return PIC_OK;
 }
 

@@ -18,6 +18,71 @@ __global__ void xhat_to_double_kernel(const float2* __restrict__ src, double* __
   }
 }
 
+// Every field of the packed particles in one pass.  With perm the order that
+// pic_advect left pending is read through, not applied (cells are already in
+// the new order, in the other buffer).  At 64^3 x 20 with three properties, in
+// place of a gather, one copy per array and the x-hat conversion (150 + 120 +
+// 105 us; the conversion alone is FP64-pipe bound, and hides behind the copies'
+// memory time here): see pic_export.
+template <int D>
+__global__ void __launch_bounds__(256) pack_kernel(const __grid_constant__ StoreView s, const uint32_t* __restrict__ cell,
+                                                   const uint32_t* __restrict__ perm, size_t first, size_t n,
+                                                   uint32_t cell_base, const __grid_constant__ PackedOut o,
+                                                   unsigned int* __restrict__ status) {
+  for (size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x) {
+    size_t i = first + j;
+    if (perm) {
+      i = perm[j];
+      if (i >= s.cap) {
+        atomicOr(status, PIC_STATUS_BOUNDS);
+        continue;
+      }
+    }
+    double x[D];
+    float2 t[D];
+    uint64_t id = 0;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      if (o.x) x[a] = s.x[a * s.cap + i];
+      if (o.xhat) t[a] = s.xhat[a * s.cap + i];
+    }
+    if (o.id) id = s.id[i];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      if (o.x) o.x[a * n + j] = x[a];
+      if (o.xhat) o.xhat[a * n + j] = (double)t[a].x + (double)t[a].y;
+    }
+    if (o.id) o.id[j] = id;
+    if (o.cell) o.cell[j] = cell[first + j] - cell_base;
+    if (o.props)
+      for (int q = 0; q < s.n_props; ++q) o.props[q * n + j] = s.props[q * s.cap + i];
+  }
+}
+
+void launch_pack(pic_particles_s* p, int buf, const uint32_t* perm, size_t first, size_t n, uint32_t cell_base,
+                 const PackedOut& o, cudaStream_t s) {
+  if (n == 0) return;
+  const StoreView v = store_view(p, buf);
+  const uint32_t* cell = perm ? p->cell[1 - buf] : p->cell[buf];
+  const size_t want = (n + 255) / 256, most = (size_t)num_sms() * 32;
+  const int g = (int)(want < most ? want : most);
+  if (p->dim == 2)
+    pack_kernel<2><<<g, 256, 0, s>>>(v, cell, perm, first, n, cell_base, o, &p->ctr->status);
+  else
+    pack_kernel<3><<<g, 256, 0, s>>>(v, cell, perm, first, n, cell_base, o, &p->ctr->status);
+  count_launches(1);
+}
+
+// Device memory of the current device.
+bool on_device(const void* ptr) {
+  cudaPointerAttributes at;
+  int here = 0;
+  const bool dev = cudaGetDevice(&here) == cudaSuccess && cudaPointerGetAttributes(&at, ptr) == cudaSuccess &&
+                   at.type == cudaMemoryTypeDevice && at.device == here;
+  cudaGetLastError();
+  return dev;
+}
+
 __global__ void set_prop_kernel(double* __restrict__ dst, const double* __restrict__ src, const DevCounters* ctr) {
   const uint32_t n = ctr->n_alive;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
@@ -255,7 +320,12 @@ extern "C" pic_status pic_export(pic_particles p, double* x, double* xhat, uint6
                                  void* stream) {
   if (!p) return (set_error("pic_export: null handle"), PIC_ERR_ARG);
   cudaStream_t st = (cudaStream_t)stream;
-  {
+  // into device arrays: one kernel, through a pending order; with any host
+  // array: the order applied, then a copy per array
+  const void* dst[5] = {x, xhat, id, cell, props};
+  bool packed = true;
+  for (const void* q : dst) packed = packed && (!q || on_device(q));
+  if (!packed) {
     const pic_status r0 = settle_order(p, st);
     if (r0 != PIC_OK) return r0;
   }
@@ -265,13 +335,16 @@ extern "C" pic_status pic_export(pic_particles p, double* x, double* xhat, uint6
   const size_t N = h.n_alive, cap = p->capacity;
   const int c = p->cur;
   if (N == 0) return PIC_OK;
+  if (packed) {
+    launch_pack(p, c, p->pending_order ? p->perm : nullptr, 0, N, 0, PackedOut{x, xhat, id, cell, props}, st);
+    PIC_CUDA(cudaGetLastError());
+    return PIC_OK;
+  }
   for (int a = 0; a < p->dim; ++a) {
     if (x) PIC_CUDA(cudaMemcpyAsync(x + a * N, p->x[c] + a * cap, sizeof(double) * N, cudaMemcpyDefault, st));
   }
   if (xhat) {
-    cudaPointerAttributes at;
-    const bool dev = cudaPointerGetAttributes(&at, xhat) == cudaSuccess && at.type == cudaMemoryTypeDevice;
-    cudaGetLastError();
+    const bool dev = on_device(xhat);
     double* tmp = xhat;
     if (!dev) PIC_CUDA(cudaMallocAsync((void**)&tmp, sizeof(double) * p->dim * N, st));
     xhat_to_double_kernel<<<1024, 256, 0, st>>>(p->xhat[c], tmp, cap, N, p->dim);

@@ -429,6 +429,19 @@ __device__ __forceinline__ bool in_ref_cell(const double t[D]) {
 
 namespace pic {
 // ---------------------------------------------- host-side internal calls --
+bool on_device(const void* ptr);
+// Particles [first, first + n) of buffer `buf` (slot first + j is particle
+// perm[j] when perm is given), packed into device arrays of n (any may be
+// null), cells less cell_base.  Defined in particles.cu.
+struct PackedOut {
+  double* x;      // [dim][n]
+  double* xhat;   // [dim][n]
+  uint64_t* id;
+  uint32_t* cell;
+  double* props;  // [P][n]
+};
+void launch_pack(pic_particles_s* p, int buf, const uint32_t* perm, size_t first, size_t n, uint32_t cell_base,
+                 const PackedOut& o, cudaStream_t s);
 // Rebuild the sorted store from the cells found by the last locate
 // (cell_new, counts already filled).  Defined in rebin.cu.
 pic_status rebin_from_counts(pic_particles_s* p, cudaStream_t s);
