@@ -16,7 +16,7 @@
 //   dL/dU_i   += dt phi-hat_i(x-hat_s) lambda_k_s
 // G and lambda in double-float.  Each stage's contribution (stage cell,
 // x-hat_s, dt lambda_k_s) is a record keyed by (stage, slot); the records are
-// sorted by (cell, key), summed per cell in that order, and the cells' sums
+// sorted by (cell, stage, slot), summed per cell in that order, and the cells' sums
 // are added into the nodes in increasing cell order.  No floating-point
 // atomics, so the gradient is bit-for-bit reproducible.
 #include <cmath>
@@ -27,6 +27,7 @@
 #include "grad_df.cuh"
 #include "locate.cuh"
 #include "pic_internal.cuh"
+#include "rebin.cuh"
 
 struct pic_tape_s {
   pic_particles_s* parts;
@@ -48,12 +49,11 @@ struct pic_tape_s {
   uint32_t* n_dev;   // [n_steps + 1] particles at the start of each step (and at the end)
   // reverse-sweep work
   float2* lam[2];      // [dim][cap] double-float
-  uint32_t* rec_cell;  // [4 cap] stage cells of the step's survivors, PIC_LOST elsewhere (the sort's keys)
-  uint64_t* rec_key;   // [4 cap]
   float2* rec_w;       // [dim][4 cap] double-float dt lambda_k
-  uint32_t* rec_perm;  // [4 cap]
-  uint32_t* rec_off;   // [C + 1]
-  void* sort_scratch;
+  uint32_t* rec_perm;  // [4 cap] the step's records sorted by (cell, stage, slot)
+  uint32_t* rec_off;   // [4 C + 1] their offsets per (cell, stage)
+  uint32_t *rec_counts, *rec_cursor;  // [4 C] sort scratch
+  uint32_t *rec_scan, *rec_src;       // scan scratch, [4 cap]
   double* partial;     // [C][3^dim][dim]
   void* slab;          // the allocation that holds every device array above
 };
@@ -106,34 +106,38 @@ struct TapeStep {
 // recorded stage points, all in double-float on the FP32 pipe:
 //   lambda_k_s = b_s lambda' + a_{s+1} lambda_y_{s+1}
 //   lambda_y_s = dt G_s^T lambda_k_s,   lambda = lambda' + sum_s lambda_y_s
-// and record r = s cap + i gets its cell, key and weight dt lambda_k_s.  The
-// records of particles that did not survive the step stay PIC_LOST.
+// and record r = s cap + i gets its weight dt lambda_k_s and is counted at
+// (its cell, s).
 template <int D, int RK>
 __global__ void __launch_bounds__(128, PIC_REVERSE_MIN_BLOCKS) reverse_lambda_kernel(
     const __grid_constant__ MeshView m, const __grid_constant__ TapeStep tp, size_t cap, df dt, const float2* __restrict__ lam_in, float2* __restrict__ lam_out,
-    uint32_t* __restrict__ rec_cell, uint64_t* __restrict__ rec_key, float2* __restrict__ rec_w,
-    DevCounters* __restrict__ ctr) {
+    uint32_t* __restrict__ rec_counts, float2* __restrict__ rec_w, DevCounters* __restrict__ ctr) {
   using TB = AdjTableau<RK>;
   constexpr int S = TB::S;
   const uint32_t n = *tp.n_next;
   const size_t rcap = kRecPerParticle * cap;
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    const uint32_t i = tp.perm[j];
-    if (i >= cap) {
-      latch_status(ctr, PIC_STATUS_BOUNDS);
-      continue;
-    }
-    uint32_t Ks[S];
-    bool ok = true;
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t base = blockIdx.x * blockDim.x + threadIdx.x - lane; base < n; base += gridDim.x * blockDim.x) {
+    const uint32_t j = base + lane;
+    uint32_t i = 0, Ks[S];
+    bool ok = j < n;
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      Ks[s] = tp.rcell[(size_t)s * cap + i];
-      ok = ok && Ks[s] < m.C;
+    for (int s = 0; s < S; ++s) Ks[s] = PIC_LOST;
+    if (ok) {
+      i = tp.perm[j];
+      ok = i < cap;
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        if (ok) Ks[s] = tp.rcell[(size_t)s * cap + i];
+        ok = ok && Ks[s] < m.C;
+      }
+      if (!ok) latch_status(ctr, PIC_STATUS_BOUNDS);  // cannot happen for a particle that survived the step
     }
-    if (!ok) {  // cannot happen for a particle that survived the step
-      latch_status(ctr, PIC_STATUS_BOUNDS);
-      continue;
-    }
+    // the counts of the records' sort, one atomic per distinct (cell, stage) of
+    // the warp
+#pragma unroll
+    for (int s = 0; s < S; ++s) (void)aggregated_increment(rec_counts, Ks[s] * kRecPerParticle + s, ok);
+    if (!ok) continue;
     df lam[D], lam_x[D], lam_ynext[D];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
@@ -154,32 +158,77 @@ __global__ void __launch_bounds__(128, PIC_REVERSE_MIN_BLOCKS) reverse_lambda_ke
       uint32_t K = Ks[0];
 #pragma unroll
       for (int q = 1; q < S; ++q) K = (s == q) ? Ks[q] : K;
-      df G[D][D];
-      velocity_gradient_df<D>(m, K, t, G);
       const df bs = TB::b(s);
       const float an = s + 1 < S ? TB::a(s + 1) : 0.f;
       df lk[D];
 #pragma unroll
       for (int a = 0; a < D; ++a) lk[a] = df_add(df_mul(bs, lam[a]), df_scale2(lam_ynext[a], an));
-      rec_cell[r] = K;
-      rec_key[r] = r;
 #pragma unroll
       for (int a = 0; a < D; ++a) {
         const df w = df_mul(dt, lk[a]);
         rec_w[a * rcap + r] = make_float2(w.hi, w.lo);
       }
+      // G_s^T lambda_k = J^{-T} ((du/dx-hat)^T lambda_k)
+      df Gu[D][D], v[D], z[D];
+      q2_grad_mono_df<D>(m.Qc, K, t, Gu);
 #pragma unroll
       for (int q = 0; q < D; ++q) {
         df_acc acc = acc_zero();
 #pragma unroll
-        for (int c = 0; c < D; ++c) acc_mad(acc, G[c][q], lk[c]);
-        lam_ynext[q] = df_mul(dt, acc_result(acc));
+        for (int c = 0; c < D; ++c) acc_mad(acc, Gu[c][q], lk[c]);
+        v[q] = acc_result(acc);
+      }
+      solve_transposed_df<D>(m, K, t, v, z);
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        lam_ynext[q] = df_mul(dt, z[q]);
         lam_x[q] = df_add(lam_x[q], lam_ynext[q]);
       }
     }
 #pragma unroll
     for (int a = 0; a < D; ++a) lam_out[a * cap + i] = make_float2(lam_x[a].hi, lam_x[a].lo);
   }
+}
+
+// The records of the step's survivors into their (cell, stage) segments.  The
+// sums want them by (cell, stage, slot): with a segment per stage the rank that
+// follows only compares slots, over a quarter of the cell's records (128 of
+// them at 32 particles per cell: 160 us a step for 4.2 M records ranked by a
+// 64-bit key per cell; this and the rank over 4 C segments take 55).
+__global__ void __launch_bounds__(256) scatter_records_kernel(const __grid_constant__ TapeStep tp, int S, uint32_t C,
+                                                              size_t cap, uint32_t* __restrict__ cursor,
+                                                              uint32_t* __restrict__ src, DevCounters* __restrict__ ctr) {
+  const uint32_t n = *tp.n_next;
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t base = blockIdx.x * blockDim.x + threadIdx.x - lane; base < n; base += gridDim.x * blockDim.x) {
+    const uint32_t j = base + lane;
+    const uint32_t i = j < n ? tp.perm[j] : PIC_LOST;
+    // all stages or none, as the lambda sweep counted them
+    uint32_t K[kRecPerParticle];
+    bool ok = i < cap;
+#pragma unroll
+    for (int s = 0; s < kRecPerParticle; ++s) {
+      K[s] = ok && s < S ? tp.rcell[(size_t)s * cap + i] : 0u;
+      ok = ok && K[s] < C;
+    }
+#pragma unroll
+    for (int s = 0; s < kRecPerParticle; ++s) {
+      if (s >= S) break;
+      const uint32_t slot = aggregated_increment(cursor, K[s] * kRecPerParticle + s, ok);
+      if (!ok) continue;
+      if (slot < kRecPerParticle * cap)
+        src[slot] = (uint32_t)(s * cap + i);
+      else
+        latch_status(ctr, PIC_STATUS_BOUNDS);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) rank_records_kernel(const uint32_t* __restrict__ off, const uint32_t* __restrict__ src,
+                                                           uint32_t* __restrict__ perm, uint32_t segments, size_t rcap,
+                                                           DevCounters* __restrict__ ctr) {
+  rank_phase(off, src, src, perm, (uint32_t*)nullptr, segments, rcap, &ctr->status,
+             (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
 }
 
 // Checkpoint tapes: the step replayed from the store as it was at the start
@@ -194,12 +243,13 @@ __global__ void __launch_bounds__(128, PIC_ADVECT_MIN_BLOCKS) replay_step_kernel
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     int iters = 0;
     unsigned flags = 0;
-    RecordHook hook{rec, i};
-    advect_particle_to<D, RK, false, false>(m, s, i, sink, i, s.cell[i], dt, iters, flags, hook);
+    uint32_t full = 0;
+    (void)advect_particle_step<D, RK, false, false>(GlobalCells<D, false>{m}, m, s, i, sink, i, s.cell[i], dt, iters,
+                                                    flags, full, RecordHook{rec, i});
   }
 }
 
-// Warp per cell: the records of the cell, in (cell, key) order, summed into
+// Warp per cell: the records of the cell, in (cell, stage, slot) order, summed into
 // the cell's 3^D x D block of nodal gradient entries (lane e owns entries e,
 // e+32, ...), in double-float on the FP32 pipe; every cell is written (FP64),
 // empty ones with zeros.  The entry (node (a, b, c), comp) of a record is
@@ -233,7 +283,7 @@ __global__ void __launch_bounds__(256) cell_partial_kernel(uint32_t C, const uin
     df_acc acc[PER];
 #pragma unroll
     for (int q = 0; q < PER; ++q) acc[q] = acc_zero();
-    const uint32_t beg = rec_off[K], end = rec_off[K + 1];
+    const uint32_t beg = rec_off[K * kRecPerParticle], end = rec_off[(K + 1) * kRecPerParticle];
     for (uint32_t e0 = beg; e0 < end; e0 += 32) {
       const uint32_t e = e0 + lane;
       if (e < end) {
@@ -364,8 +414,8 @@ static void launch_reverse(pic_tape_s* tp, const MeshView& m, int step, const Ta
                                                                      StageRec{tp->rcell[0], tp->rt[0], tp->cap});
     count_launches(1);
   }
-  reverse_lambda_kernel<D, RK><<<grid_of(tp->cap, 128), 128, 0, st>>>(m, ts, tp->cap, dtd, lin, lout, tp->rec_cell,
-                                                                       tp->rec_key, tp->rec_w, tp->parts->ctr);
+  reverse_lambda_kernel<D, RK><<<grid_of(tp->cap, 128), 128, 0, st>>>(m, ts, tp->cap, dtd, lin, lout,
+                                                                       tp->rec_counts, tp->rec_w, tp->parts->ctr);
 }
 
 }  // namespace pic
@@ -401,11 +451,8 @@ extern "C" pic_status pic_advect_record_tape(pic_particles parts, pic_mesh mesh,
   if (mesh->has_next)
     return (set_error("pic_advect_record: the adjoint supports a steady field only (no U_next)"), PIC_ERR_ARG);
   cudaStream_t st = (cudaStream_t)stream;
-  {
-    const pic_status r0 = settle_order(parts, st);
-    if (r0 != PIC_OK) return r0;
-  }
   pic_tape_s* tp = (pic_tape_s*)calloc(1, sizeof(pic_tape_s));
+  if (!tp) return (set_error("pic_advect_record: host allocation failed"), PIC_ERR_OOM);
   tp->parts = parts;
   tp->mesh = mesh;
   tp->dim = mesh->dim;
@@ -450,12 +497,14 @@ extern "C" pic_status pic_advect_record_tape(pic_particles parts, pic_mesh mesh,
     slab.add(&tp->n_dev, steps + 1);
     slab.add(&tp->lam[0], d * cap);
     slab.add(&tp->lam[1], d * cap);
-    slab.add(&tp->rec_cell, rcap);
-    slab.add(&tp->rec_key, rcap);
     slab.add(&tp->rec_w, d * rcap);
     slab.add(&tp->rec_perm, rcap);
-    slab.add(&tp->rec_off, (size_t)tp->C + 1);
-    slab.add(reinterpret_cast<char**>(&tp->sort_scratch), sort_scratch_bytes(rcap, tp->C));
+    const uint32_t segments = kRecPerParticle * tp->C;
+    slab.add(&tp->rec_off, (size_t)segments + 1);
+    slab.add(&tp->rec_counts, segments);
+    slab.add(&tp->rec_cursor, segments);
+    slab.add(&tp->rec_scan, scan_scratch_bytes(segments) / sizeof(uint32_t));
+    slab.add(&tp->rec_src, rcap);
     slab.add(&tp->partial, (size_t)NE * tp->C);
     ok = slab.allocate(&tp->slab);
   }
@@ -479,8 +528,13 @@ extern "C" pic_status pic_advect_record_tape(pic_particles parts, pic_mesh mesh,
   const MeshView m = mesh_view(mesh);
   for (int s = 0; s < n_steps; ++s) {
     cudaError_t e = cudaMemcpyAsync(tp->n_dev + s, &parts->ctr->n_alive, sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(parts->counts, 0, sizeof(uint32_t) * parts->C, st);
     if (ckpt) {
+      // the checkpoint is the sorted store
+      const pic_status r0 = settle_order(parts, st);
+      if (r0 != PIC_OK) {
+        pic_destroy_tape(tp);
+        return r0;
+      }
       const int c = parts->cur;
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(tp->x[s], parts->x[c], sizeof(double) * d * cap, cudaMemcpyDeviceToDevice, st);
@@ -494,18 +548,14 @@ extern "C" pic_status pic_advect_record_tape(pic_particles parts, pic_mesh mesh,
       return cuda_fail(e, "pic_advect_record: checkpoint");
     }
     // a checkpoint tape keeps one record set, which the sweep's replay rewrites
-    launch_advect_record(parts, m, dt, (int)integrator, StageRec{tp->rcell[ckpt ? 0 : s], tp->rt[ckpt ? 0 : s], cap},
-                         st);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      pic_destroy_tape(tp);
-      return cuda_fail(e, "pic_advect_record: step");
-    }
-    pic_status r = rebin_from_counts(parts, st);
+    pic_status r = launch_advect_record(parts, m, dt, (int)integrator,
+                                        StageRec{tp->rcell[ckpt ? 0 : s], tp->rt[ckpt ? 0 : s], cap}, st);
+    if (r == PIC_OK) r = rebin_order_from_counts(parts, st);
     if (r != PIC_OK) {
       pic_destroy_tape(tp);
       return r;
     }
+    parts->pending_order = 1;  // applied by the next step, or by whoever needs the sorted arrays
     e = cudaMemcpyAsync(tp->perm[s], parts->perm, sizeof(uint32_t) * cap, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) {
       pic_destroy_tape(tp);
@@ -538,7 +588,7 @@ extern "C" pic_status pic_tape_adjoint(pic_tape tp, const double* dL_dxfinal, do
   copy_in_kernel<<<grid_of(d * cap, 256), 256, 0, st>>>(dL_dxfinal, tp->lam[0], tp->n_dev + tp->n_steps, tp->dim, cap);
   count_launches(1);
   int cur = 0;
-  const SortScratch sc = sort_scratch_layout(tp->sort_scratch, rcap, tp->C);
+  const uint32_t segments = kRecPerParticle * tp->C;
   for (int s = tp->n_steps - 1; s >= 0; --s) {
     TapeStep ts;
     ts.rcell = tp->rcell[tp->kind == PIC_TAPE_CHECKPOINTS ? 0 : s];
@@ -546,7 +596,7 @@ extern "C" pic_status pic_tape_adjoint(pic_tape tp, const double* dL_dxfinal, do
     ts.perm = tp->perm[s];
     ts.n_next = tp->n_dev + s + 1;
     PIC_CUDA(cudaMemsetAsync(tp->lam[1 - cur], 0, sizeof(float2) * d * cap, st));
-    PIC_CUDA(cudaMemsetAsync(tp->rec_cell, 0xFF, sizeof(uint32_t) * rcap, st));
+    PIC_CUDA(cudaMemsetAsync(tp->rec_counts, 0, sizeof(uint32_t) * segments, st));
     const float2* lin = tp->lam[cur];
     float2* lout = tp->lam[1 - cur];
     if (tp->dim == 2) {
@@ -560,8 +610,14 @@ extern "C" pic_status pic_tape_adjoint(pic_tape tp, const double* dL_dxfinal, do
     }
     count_launches(1);
     PIC_CUDA(cudaGetLastError());
-    pic_status r = sort_by_cell_run(rcap, tp->rec_cell, tp->rec_key, tp->C, tp->rec_perm, tp->rec_off, sc, st);
+    pic_status r = scan_u32(tp->rec_counts, tp->rec_off, segments, tp->rec_scan, nullptr, tp->rec_cursor, st,
+                            &tp->parts->ctr->status);
     if (r != PIC_OK) return r;
+    scatter_records_kernel<<<grid_of(cap, 256), 256, 0, st>>>(ts, tp->integrator, tp->C, cap, tp->rec_cursor, tp->rec_src,
+                                                              tp->parts->ctr);
+    rank_records_kernel<<<grid_of((size_t)segments * 32, 256), 256, 0, st>>>(tp->rec_off, tp->rec_src, tp->rec_perm,
+                                                                             segments, rcap, tp->parts->ctr);
+    count_launches(2);
     const int gp = grid_of((size_t)tp->C * 32, 256);
     const int gn = grid_of(d * (size_t)mesh->nnodes, 256);
     if (tp->dim == 2) {

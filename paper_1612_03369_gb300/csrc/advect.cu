@@ -58,10 +58,10 @@ struct StageLayout {
 // d.cell[j], its id and properties are carried over), else slot j of s in
 // place.  Returns the new cell (PIC_LOST if none); *full is set when the full
 // path redid it.
-template <int D, int RK, bool F32B, bool TWO, class Cells>
+template <int D, int RK, bool F32B, bool TWO, class Hook, class Cells>
 __device__ __forceinline__ uint32_t tile_particle(const Cells& cs, const MeshView& m, const StoreView& s,
                                                   const StoreView& d, const uint32_t* __restrict__ perm, df dt,
-                                                  uint32_t j, int& iters, unsigned& flags, uint32_t& full) {
+                                                  uint32_t j, int& iters, unsigned& flags, uint32_t& full, Hook hook) {
   uint32_t i = j, K;
   if (perm) {
     i = perm[j];
@@ -75,15 +75,17 @@ __device__ __forceinline__ uint32_t tile_particle(const Cells& cs, const MeshVie
   } else {
     K = s.cell[j];
   }
-  uint32_t Kn = advect_particle_cells<D, RK, F32B, TWO, NoHook, true>(cs, m, s, i, d, j, K, dt, iters, flags);
-  if (Kn == kDefer) {
-    const FullStep f = advect_particle_full<D, RK, F32B, TWO>(m, s, i, d, j, K, dt);
-    Kn = f.K;
-    iters = f.iters;
-    flags = f.flags;
-    full = 1;
-  }
-  return Kn;
+  return advect_particle_step<D, RK, F32B, TWO>(cs, m, s, i, d, j, K, dt, iters, flags, full, hook);
+}
+
+// What follows a tile's particles: counters, and the count of each new cell.
+__device__ __forceinline__ void finish_tile(DevCounters* __restrict__ ctr, uint32_t* __restrict__ counts, uint32_t Kc,
+                                            unsigned steps, int iters, unsigned flags, uint32_t full) {
+  const unsigned dc = __reduce_add_sync(0xffffffffu, full);
+  if (dc && (threadIdx.x & 31) == 0) atomicAdd(&ctr->deferred, (unsigned long long)dc);
+  (void)aggregated_increment(counts, Kc, Kc != PIC_LOST);
+  flush_counters(ctr, steps, iters, steps && Kc == PIC_LOST ? 1u : 0u, (flags & kFlagWalk) ? 1u : 0u,
+                 (flags & kFlagGlobal) ? 1u : 0u, flags);
 }
 
 // Resident blocks per SM of the step kernel, swept on the 128^3 x 20 step
@@ -182,27 +184,19 @@ __global__ void __launch_bounds__(kAdvectThreads, F32B ? PIC_ADVECT_MIN_BLOCKS_F
 
     const uint32_t j = t * 32 + lane;
     int iters = 0;
-    unsigned flags = 0, lost = 0, steps = 0;
+    unsigned flags = 0, steps = 0;
     uint32_t Kc = PIC_LOST, full = 0;  // the new cell to count
     if (j < n) {
       steps = 1;
-      uint32_t Kn;
       if constexpr (STAGE) {
         const StagedCells<D, F32B, kWarpStageCells> cs{m, wbuf + b * L::BUF, k0_cur, (need && ok) ? n_cur : 0u};
-        Kn = tile_particle<D, RK, F32B, TWO>(cs, m, s, d, perm, dt, j, iters, flags, full);
+        Kc = tile_particle<D, RK, F32B, TWO>(cs, m, s, d, perm, dt, j, iters, flags, full, NoHook());
       } else {
-        Kn = tile_particle<D, RK, F32B, TWO>(GlobalCells<D, F32B>{m}, m, s, d, perm, dt, j, iters, flags, full);
+        Kc = tile_particle<D, RK, F32B, TWO>(GlobalCells<D, F32B>{m}, m, s, d, perm, dt, j, iters, flags, full, NoHook());
       }
-      cell_new[j] = Kn;
-      Kc = Kn;
-      lost = Kn == PIC_LOST ? 1u : 0u;
+      cell_new[j] = Kc;
     }
-    {
-      const unsigned dc = __reduce_add_sync(0xffffffffu, full);
-      if (dc && lane == 0) atomicAdd(&ctr->deferred, (unsigned long long)dc);
-    }
-    (void)aggregated_increment(counts, Kc, Kc != PIC_LOST);
-    flush_counters(ctr, steps, iters, lost, (flags & kFlagWalk) ? 1u : 0u, (flags & kFlagGlobal) ? 1u : 0u, flags);
+    finish_tile(ctr, counts, Kc, steps, iters, flags, full);
     if constexpr (STAGE) __syncwarp();  // this buffer is free for the copy issued one tile on
     need = need_next;
     k0_cur = k0_nxt;
@@ -216,6 +210,41 @@ __global__ void __launch_bounds__(kAdvectThreads, F32B ? PIC_ADVECT_MIN_BLOCKS_F
   if (STAGE && lane == 0)
     for (int b = 0; b < 2; ++b)
       if ((stuck >> b) & 1u) (void)mbar_wait_bounded(&bar[b], (stuck_parity >> b) & 1u, kStageWaitNs);
+}
+
+// The step kernel that also leaves every stage's (cell, x-hat) behind, in slot
+// order of the store the step writes: the same particle step, so positions,
+// cells and order are pic_advect's bit for bit.  Like it, it runs the fast path
+// over dynamic tiles and applies a pending order on the way (as one grid-stride
+// kernel over the full step, with a gather per step, it took 367 + 26 us for
+// 1.05 M particles).
+template <int D, int RK>
+__global__ void __launch_bounds__(kAdvectThreads, PIC_ADVECT_MIN_BLOCKS_F64)
+    advect_record_kernel(const __grid_constant__ MeshView m, const __grid_constant__ StoreView s,
+                         const __grid_constant__ StoreView d, const uint32_t* __restrict__ perm, df dt,
+                         const __grid_constant__ StageRec rec, uint32_t* __restrict__ cell_new,
+                         uint32_t* __restrict__ counts, DevCounters* __restrict__ ctr) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t n = ctr->n_alive, ntiles = (n + 31) / 32;
+  auto grab = [&]() -> uint32_t {
+    uint32_t t = 0;
+    if (lane == 0) t = atomicAdd(&ctr->tile_next, 1u);
+    return __shfl_sync(0xffffffffu, t, 0);
+  };
+  for (uint32_t t = grab(); t < ntiles;) {
+    const uint32_t tn = grab(), j = t * 32 + lane;
+    int iters = 0;
+    unsigned flags = 0, steps = 0;
+    uint32_t Kc = PIC_LOST, full = 0;
+    if (j < n) {
+      steps = 1;
+      Kc = tile_particle<D, RK, false, false>(GlobalCells<D, false>{m}, m, s, d, perm, dt, j, iters, flags, full,
+                                              RecordHook{rec, j});
+      cell_new[j] = Kc;
+    }
+    finish_tile(ctr, counts, Kc, steps, iters, flags, full);
+    t = tn;
+  }
 }
 
 // Relocate every particle at its current x (hint: its current cell).
@@ -429,6 +458,38 @@ static void launch_advect(pic_particles_s* p, const MeshView& m, double dt, bool
   }
   count_launches(1);
   if (fused) p->cur = 1 - p->cur;
+}
+
+template <int D>
+static void launch_record_d(pic_particles_s* p, const MeshView& m, double dt, int rk, const StageRec& rec, bool fused,
+                            cudaStream_t st) {
+  const float hi = (float)dt;
+  const df dtd = {hi, (float)(dt - (double)hi)};
+  const StoreView s = store_view(p, p->cur), d = fused ? store_view(p, 1 - p->cur) : s;
+  const uint32_t* perm = fused ? p->perm : nullptr;
+  const int g = advect_grid(p->capacity, false);
+  if (rk == 1)
+    advect_record_kernel<D, 1><<<g, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, rec, p->cell_new, p->counts, p->ctr);
+  else if (rk == 2)
+    advect_record_kernel<D, 2><<<g, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, rec, p->cell_new, p->counts, p->ctr);
+  else
+    advect_record_kernel<D, 4><<<g, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, rec, p->cell_new, p->counts, p->ctr);
+  count_launches(1);
+}
+
+pic_status launch_advect_record(pic_particles_s* p, const MeshView& m, double dt, int rk, const StageRec& rec,
+                                cudaStream_t st) {
+  PIC_CUDA(cudaMemsetAsync(p->counts, 0, sizeof(uint32_t) * p->C, st));
+  PIC_CUDA(cudaMemsetAsync(&p->ctr->tile_next, 0, sizeof(unsigned int), st));
+  const bool fused = p->pending_order != 0;
+  if (p->dim == 2)
+    launch_record_d<2>(p, m, dt, rk, rec, fused, st);
+  else
+    launch_record_d<3>(p, m, dt, rk, rec, fused, st);
+  PIC_CUDA(cudaGetLastError());
+  if (fused) p->cur = 1 - p->cur;
+  p->pending_order = 0;
+  return PIC_OK;
 }
 
 // Three events per timed step (before advect, after advect, after rebin),

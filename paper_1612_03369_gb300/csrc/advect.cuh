@@ -262,14 +262,31 @@ struct FullStep {
   int iters;
   unsigned flags;
 };
-template <int D, int RK, bool F32B, bool TWO>
+template <int D, int RK, bool F32B, bool TWO, class Hook = NoHook>
 __device__ __noinline__ FullStep advect_particle_full(const MeshView& m, const StoreView& s, uint32_t i,
-                                                      const StoreView& d, uint32_t j, uint32_t K, df dt) {
+                                                      const StoreView& d, uint32_t j, uint32_t K, df dt,
+                                                      Hook hook = Hook()) {
   FullStep o;
   o.iters = 0;
   o.flags = 0;
-  o.K = advect_particle_to<D, RK, F32B, TWO>(m, s, i, d, j, K, dt, o.iters, o.flags);
+  o.K = advect_particle_to<D, RK, F32B, TWO>(m, s, i, d, j, K, dt, o.iters, o.flags, hook);
   return o;
+}
+
+// The fast path, then the full step where it defers (*full is set).
+template <int D, int RK, bool F32B, bool TWO, class Hook, class Cells>
+__device__ __forceinline__ uint32_t advect_particle_step(const Cells& cs, const MeshView& m, const StoreView& s,
+                                                         uint32_t i, const StoreView& d, uint32_t j, uint32_t K, df dt,
+                                                         int& iters, unsigned& flags, uint32_t& full, Hook hook) {
+  uint32_t Kn = advect_particle_cells<D, RK, F32B, TWO, Hook&, true>(cs, m, s, i, d, j, K, dt, iters, flags, hook);
+  if (Kn == kDefer) {
+    const FullStep f = advect_particle_full<D, RK, F32B, TWO, Hook>(m, s, i, d, j, K, dt, hook);
+    Kn = f.K;
+    iters = f.iters;
+    flags = f.flags;
+    full = 1;
+  }
+  return Kn;
 }
 
 }  // namespace pic

@@ -158,15 +158,8 @@ __device__ __forceinline__ uint32_t ensemble_particle(const EnsShared& sh, const
   const int p = problem_of(sh.base, P, g);
   const MeshView& m = views[p];
   const uint32_t K = g - sh.base[p];
-  uint32_t Kn = advect_particle_cells<D, RK, false, false, NoHook, true>(GlobalCells<D, false>{m}, m, s, i, d, j, K,
-                                                                         sh.dt[p], iters, flags);
-  if (Kn == kDefer) {
-    const FullStep f = advect_particle_full<D, RK, false, false>(m, s, i, d, j, K, sh.dt[p]);
-    Kn = f.K;
-    iters = f.iters;
-    flags = f.flags;
-    full = 1;
-  }
+  const uint32_t Kn = advect_particle_step<D, RK, false, false>(GlobalCells<D, false>{m}, m, s, i, d, j, K, sh.dt[p], iters,
+                                                                flags, full, NoHook());
   return Kn == PIC_LOST ? PIC_LOST : sh.base[p] + Kn;
 }
 

@@ -449,7 +449,7 @@ pic_status rebin_from_counts(pic_particles_s* p, cudaStream_t s);
 // cells in the other buffer), then the gather that applies it.
 pic_status rebin_order_from_counts(pic_particles_s* p, cudaStream_t s);
 // Stage records of one step (props.cu): for evaluation point p < 4 of the
-// particle in slot i (store order at the start of the step), the located
+// particle in slot i (the sorted order at the start of the step), the located
 // cell at cell[p cap + i] and component a of its double-float x-hat at
 // t[(4 a + p) cap + i], so that record r = p cap + i has its components at
 // t[a 4 cap + r].
@@ -458,10 +458,11 @@ struct StageRec {
   float2* t;
   size_t cap;
 };
-// One particle step of pic_advect (FP64 form, in place, counts and cell_new
-// for the rebin) that also writes the stage records.
-void launch_advect_record(pic_particles_s* p, const MeshView& m, double dt, int rk, const StageRec& rec,
-                          cudaStream_t st);
+// One particle step of pic_advect (FP64 form; a pending order is applied on the
+// way; cell_new and counts are left for the rebin) that also writes the stage
+// records, in the slots of the store after that order.  Defined in advect.cu.
+pic_status launch_advect_record(pic_particles_s* p, const MeshView& m, double dt, int rk, const StageRec& rec,
+                                cudaStream_t st);
 pic_status rebin_apply_order(pic_particles_s* p, cudaStream_t s);
 // pic_advect leaves its last rebin's order pending (the next pic_advect
 // applies it inside its advect, pic_interpolate_to_cells reads through it);

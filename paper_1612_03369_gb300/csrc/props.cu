@@ -5,9 +5,9 @@
 // with |.| the Frobenius norm.  The properties and the position form one
 // system z = (x, d, F) stepped by the same RK tableau over the same located
 // stage points.  Each time step runs in three kernels:
-//   1. the particle step of pic_advect (the same advect_particle, so
-//      positions, cells and order are those of pic_advect bit for bit),
-//      recording every stage's (cell, x-hat);
+//   1. the particle step of pic_advect (advect_record_kernel: positions,
+//      cells and order are those of pic_advect bit for bit), recording every
+//      stage's (cell, x-hat);
 //   2. G = grad u_h at every recorded stage point, thread per (stage,
 //      particle), in double-float on the FP32 pipe;
 //   3. the ODEs over the stages with those G, in double-float.
@@ -29,35 +29,6 @@ struct OdeArgs {
   int defgrad;  // first of D*D slots of F (row-major), or -1
   df alpha, beta;
 };
-
-// Phase 1: the particle step of pic_advect (the same advect_particle, so
-// positions, cells and order are bit for bit those of pic_advect), leaving
-// each stage's (cell, x-hat) behind.
-template <int D, int RK>
-__global__ void __launch_bounds__(128, PIC_ADVECT_MIN_BLOCKS) advect_record_kernel(const __grid_constant__ MeshView m, const __grid_constant__ StoreView s, df dt,
-                                                                                  const __grid_constant__ StageRec rec,
-                                                                                  uint32_t* __restrict__ cell_new,
-                                                                                  uint32_t* __restrict__ counts,
-                                                                                  DevCounters* __restrict__ ctr) {
-  const uint32_t n = ctr->n_alive;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t base = blockIdx.x * blockDim.x; base < n; base += stride) {
-    const uint32_t i = base + threadIdx.x;
-    int iters = 0;
-    unsigned flags = 0, lost = 0, steps = 0;
-    uint32_t Kc = PIC_LOST;  // the new cell to count
-    if (i < n) {
-      steps = 1;
-      RecordHook hook{rec, i};
-      const uint32_t Kn = advect_particle<D, RK, false, false>(m, s, i, s.cell[i], dt, iters, flags, hook);
-      cell_new[i] = Kn;
-      Kc = Kn;
-      lost = Kn == PIC_LOST ? 1u : 0u;
-    }
-    (void)aggregated_increment(counts, Kc, Kc != PIC_LOST);
-    flush_counters(ctr, steps, iters, lost, (flags & kFlagWalk) ? 1u : 0u, (flags & kFlagGlobal) ? 1u : 0u, flags);
-  }
-}
 
 // Phase 2, thread per (stage, surviving particle): G_p = grad u_h at the
 // recorded stage point, in double-float, stored as G[(p D^2 + e) cap + i].
@@ -192,53 +163,25 @@ static int props_grid(size_t n) {
 }
 
 template <int D, int RK>
-static void launch_props_rk(pic_particles_s* p, const MeshView& m, df dt, const OdeArgs& o, StageRec rec,
-                            cudaStream_t st) {
-  const StoreView s = store_view(p, p->cur);
-  const int g = props_grid(p->capacity);
+static void launch_odes_rk(pic_particles_s* p, const MeshView& m, df dt, const OdeArgs& o, StageRec rec, cudaStream_t st) {
   float2* Gs = stage_gradients(p);
-  advect_record_kernel<D, RK><<<g, 128, 0, st>>>(m, s, dt, rec, p->cell_new, p->counts, p->ctr);
   props_grad_kernel<D><<<props_grid((size_t)Tableau<RK>::S * p->capacity), 128, 0, st>>>(m, rec, Tableau<RK>::S,
                                                                                         p->cell_new, p->ctr, Gs);
-  props_ode_kernel<D, RK><<<g, 128, 0, st>>>(s, dt, o, Gs, p->cell_new, p->ctr);
-  count_launches(3);
+  props_ode_kernel<D, RK><<<props_grid(p->capacity), 128, 0, st>>>(store_view(p, p->cur), dt, o, Gs, p->cell_new, p->ctr);
+  count_launches(2);
 }
 
 template <int D>
-static void launch_props(pic_particles_s* p, const MeshView& m, double dt, int rk, const OdeArgs& o, StageRec rec,
-                         cudaStream_t st) {
+static void launch_odes(pic_particles_s* p, const MeshView& m, double dt, int rk, const OdeArgs& o, StageRec rec,
+                        cudaStream_t st) {
   const float hi = (float)dt;
   const df dtd = {hi, (float)(dt - (double)hi)};
   if (rk == 1)
-    launch_props_rk<D, 1>(p, m, dtd, o, rec, st);
+    launch_odes_rk<D, 1>(p, m, dtd, o, rec, st);
   else if (rk == 2)
-    launch_props_rk<D, 2>(p, m, dtd, o, rec, st);
+    launch_odes_rk<D, 2>(p, m, dtd, o, rec, st);
   else
-    launch_props_rk<D, 4>(p, m, dtd, o, rec, st);
-}
-
-template <int D>
-static void launch_record_d(pic_particles_s* p, const MeshView& m, df dt, int rk, const StageRec& rec,
-                            cudaStream_t st) {
-  const StoreView s = store_view(p, p->cur);
-  const int g = props_grid(p->capacity);
-  if (rk == 1)
-    advect_record_kernel<D, 1><<<g, 128, 0, st>>>(m, s, dt, rec, p->cell_new, p->counts, p->ctr);
-  else if (rk == 2)
-    advect_record_kernel<D, 2><<<g, 128, 0, st>>>(m, s, dt, rec, p->cell_new, p->counts, p->ctr);
-  else
-    advect_record_kernel<D, 4><<<g, 128, 0, st>>>(m, s, dt, rec, p->cell_new, p->counts, p->ctr);
-  count_launches(1);
-}
-
-void launch_advect_record(pic_particles_s* p, const MeshView& m, double dt, int rk, const StageRec& rec,
-                          cudaStream_t st) {
-  const float hi = (float)dt;
-  const df dtd = {hi, (float)(dt - (double)hi)};
-  if (p->dim == 2)
-    launch_record_d<2>(p, m, dtd, rk, rec, st);
-  else
-    launch_record_d<3>(p, m, dtd, rk, rec, st);
+    launch_odes_rk<D, 4>(p, m, dtd, o, rec, st);
 }
 
 }  // namespace pic
@@ -277,10 +220,6 @@ extern "C" pic_status pic_advect_properties(pic_particles parts, pic_mesh mesh, 
   };
   const OdeArgs o = {odes->damage, odes->deformation, split(odes->alpha), split(odes->beta)};
   cudaStream_t st = (cudaStream_t)stream;
-  {
-    const pic_status r0 = settle_order(parts, st);
-    if (r0 != PIC_OK) return r0;
-  }
   const MeshView m = mesh_view(mesh);
   if (!parts->stage_rec) {
     const size_t bytes = (size_t)4 * parts->capacity * (sizeof(uint32_t) + sizeof(float2) * d + sizeof(float2) * d * d);
@@ -294,15 +233,19 @@ extern "C" pic_status pic_advect_properties(pic_particles parts, pic_mesh mesh, 
   const StageRec rec = {(uint32_t*)parts->stage_rec,
                         (float2*)((char*)parts->stage_rec + (size_t)4 * parts->capacity * sizeof(uint32_t)),
                         parts->capacity};
+  // as in pic_advect, each rebin's order is applied by the next step's kernel
+  // and the last one stays pending
   for (int step = 0; step < n_steps; ++step) {
-    PIC_CUDA(cudaMemsetAsync(parts->counts, 0, sizeof(uint32_t) * parts->C, st));
-    if (d == 2)
-      launch_props<2>(parts, m, dt, (int)integrator, o, rec, st);
-    else
-      launch_props<3>(parts, m, dt, (int)integrator, o, rec, st);
-    PIC_CUDA(cudaGetLastError());
-    pic_status r = rebin_from_counts(parts, st);
+    pic_status r = launch_advect_record(parts, m, dt, (int)integrator, rec, st);
     if (r != PIC_OK) return r;
+    if (d == 2)
+      launch_odes<2>(parts, m, dt, (int)integrator, o, rec, st);
+    else
+      launch_odes<3>(parts, m, dt, (int)integrator, o, rec, st);
+    PIC_CUDA(cudaGetLastError());
+    r = rebin_order_from_counts(parts, st);
+    if (r != PIC_OK) return r;
+    parts->pending_order = 1;
   }
   return PIC_OK;
 }

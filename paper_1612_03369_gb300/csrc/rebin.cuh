@@ -185,7 +185,8 @@ __device__ __forceinline__ void scatter_phase(const uint32_t* __restrict__ cell_
 // and counting the smaller ids of that segment.  All lanes work whatever the
 // cells' sizes, where one warp per cell left most lanes idle at ~10-20
 // particles per cell.
-__device__ __forceinline__ void rank_phase(const uint32_t* __restrict__ cell_off, const uint64_t* __restrict__ key_id,
+template <class Key>
+__device__ __forceinline__ void rank_phase(const uint32_t* __restrict__ cell_off, const Key* __restrict__ key_id,
                                            const uint32_t* __restrict__ key_src, uint32_t* __restrict__ perm,
                                            uint32_t* __restrict__ cell_out, uint32_t C, size_t cap,
                                            unsigned int* __restrict__ status, uint32_t w, uint32_t nw) {
@@ -216,7 +217,7 @@ __device__ __forceinline__ void rank_phase(const uint32_t* __restrict__ cell_off
       continue;
     }
     // each chunk's key and source are loaded one chunk ahead
-    uint64_t my_n = 0;
+    Key my_n = 0;
     uint32_t src_n = 0;
     if (beg_all + lane < end_all) {
       my_n = key_id[beg_all + lane];
@@ -224,7 +225,7 @@ __device__ __forceinline__ void rank_phase(const uint32_t* __restrict__ cell_off
     }
     for (uint32_t j0 = beg_all; j0 < end_all; j0 += 32u) {
       const uint32_t j = j0 + lane;
-      const uint64_t my = my_n;
+      const Key my = my_n;
       const uint32_t src = src_n;
       if (j + 32u < end_all) {
         my_n = key_id[j + 32u];
