@@ -10,10 +10,46 @@ namespace pic {
 // a warp read neighbouring segments, so every sector fetched from HBM is used
 // by the following iterations through L1.  Kinds (Sec. 2.7 (ii)):
 //   0 arithmetic  sum v / n
-//   1 geometric   exp(sum log v / n)   (NaN if the cell holds a v <= 0)
+//   1 geometric   (product v)^(1/n)     (NaN if the cell holds a v <= 0)
 //   2 harmonic    n / sum (1 / v)      (NaN if the cell holds a v <= 0)
+// The geometric mean multiplies significands and adds exponents, so it takes
+// one logarithm per cell instead of one per particle: with v_i = m_i 2^e_i, P 2^E
+// their product and E = q n + r, it is 2^q exp((r log 2 + log P) / n).  The
+// product's relative rounding, sqrt(n) 2^-53, counts 1/n of itself in the mean.
+// (An FP64 logarithm per particle: 332 us at 64^3 x 20, FP64-pipe bound.)
 // PERM (an order left pending by pic_advect): slot i's value is
 // prop[perm[i]], the same values in the same order as after the gather.
+struct ProductAcc {
+  double P = 1.0;     // in [1, 2)
+  long long E = 0;
+  bool infinite = false;
+
+  __device__ __forceinline__ void mul(double v) {  // v > 0
+    int hi = __double2hiint(v);
+    int e = hi >> 20;
+    if (e == 0) {  // subnormal
+      v *= 0x1p54;
+      hi = __double2hiint(v);
+      e = (hi >> 20) - 54;
+    }
+    infinite = infinite || e == 0x7ff;
+    P *= __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(v));
+    const int top = __double2hiint(P);
+    const int carry = (top >> 20) - 1023;  // 0 or 1
+    P = __hiloint2double(top - (carry << 20), __double2loint(P));
+    E += e - 1023 + carry;
+  }
+  __device__ __forceinline__ double mean(uint32_t n) const {
+    if (infinite) return __longlong_as_double(0x7ff0000000000000ll);
+    long long q = E / (long long)n, r = E % (long long)n;
+    if (r < 0) {
+      r += n;
+      --q;
+    }
+    return ldexp(exp(((double)r * 0.6931471805599453094 + log(P)) / (double)n), (int)q);
+  }
+};
+
 template <int KIND, bool PERM>
 __global__ void __launch_bounds__(256) cell_average_kernel(const uint32_t* __restrict__ cell_off,
                                                            const double* __restrict__ prop,
@@ -28,6 +64,7 @@ __global__ void __launch_bounds__(256) cell_average_kernel(const uint32_t* __res
     }
     double s = 0.0;
     bool bad = false;
+    ProductAcc product;
     for (uint32_t i = beg; i < end; ++i) {
       uint32_t src = i;
       if constexpr (PERM) {
@@ -43,7 +80,11 @@ __global__ void __launch_bounds__(256) cell_average_kernel(const uint32_t* __res
         s += v;
       } else {
         bad = bad || !(v > 0.0);
-        s += (KIND == 1) ? log(v) : 1.0 / v;
+        if constexpr (KIND == 1) {
+          if (v > 0.0) product.mul(v);
+        } else {
+          s += 1.0 / v;
+        }
       }
     }
     const uint32_t n = end - beg;
@@ -54,7 +95,7 @@ __global__ void __launch_bounds__(256) cell_average_kernel(const uint32_t* __res
       else if (bad)
         r = __longlong_as_double(0x7ff8000000000000ll);
       else
-        r = (KIND == 1) ? exp(s / (double)n) : (double)n / s;
+        r = (KIND == 1) ? product.mean(n) : (double)n / s;
     }
     avg[K] = r;
     if (count) count[K] = n;

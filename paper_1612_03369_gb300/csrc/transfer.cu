@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(128) lsq_linear_kernel(const uint32_t* __restr
     }
     // the upper triangle of A^T A, A^T p and sum p, accumulated in
     // double-float (row a = (1, x-hat - 1/2)), then converted once
-    df_acc Ma[NB][NB + 1], sa = acc_zero();
+    df_acc Ma[NB][NB + 1];
 #pragma unroll
     for (int r = 0; r < NB; ++r)
 #pragma unroll
@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(128) lsq_linear_kernel(const uint32_t* __restr
       for (int r = 0; r < NB; ++r) {
 #pragma unroll
         for (int q = r; q < NB; ++q) {
+          if (r == 0 && q == 0) continue;  // the count
           if (r == 0)
             acc_add(Ma[r][q], a[q]);  // a[0] = 1
           else
@@ -169,14 +170,14 @@ __global__ void __launch_bounds__(128) lsq_linear_kernel(const uint32_t* __restr
         else
           acc_mad(Ma[r][NB], a[r], p);
       }
-      acc_add(sa, p);
     }
     double M[NB][NB + 1];
 #pragma unroll
     for (int r = 0; r < NB; ++r)
 #pragma unroll
       for (int q = r; q <= NB; ++q) M[r][q] = df_to_f64(acc_result(Ma[r][q]));
-    const double sum = df_to_f64(acc_result(sa));
+    M[0][0] = (double)(end - beg);
+    const double sum = M[0][NB];
 #pragma unroll
     for (int r = 1; r < NB; ++r)
 #pragma unroll
