@@ -65,25 +65,38 @@ __global__ void __launch_bounds__(256) cell_average_kernel(const uint32_t* __res
     double s = 0.0;
     bool bad = false;
     ProductAcc product;
-    for (uint32_t i = beg; i < end; ++i) {
-      uint32_t src = i;
-      if constexpr (PERM) {
-        src = perm[i];
-        if (src >= cap) {
+    // kBatch particles at a time: their loads (two dependent ones with PERM) are
+    // in flight together, then folded in store order: 14 -> 7 us for 16^3 cells
+    // and 42 -> 31 us for 64^3 through a pending order (settled, 4 at a time is
+    // enough for 20 particles a cell)
+    constexpr int kBatch = PERM ? 8 : 4;
+    for (uint32_t i0 = beg; i0 < end; i0 += kBatch) {
+      uint32_t src[kBatch];
+      double v[kBatch];
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        src[q] = i0 + q;
+        if constexpr (PERM) src[q] = i0 + q < end ? perm[i0 + q] : 0u;
+      }
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) v[q] = i0 + q < end && src[q] < cap ? prop[src[q]] : 0.0;
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        if (i0 + q >= end) break;
+        if (PERM && src[q] >= cap) {
           bad = true;
           latch_status(ctr, PIC_STATUS_BOUNDS);
           continue;
         }
-      }
-      const double v = prop[src];
-      if constexpr (KIND == 0) {
-        s += v;
-      } else {
-        bad = bad || !(v > 0.0);
-        if constexpr (KIND == 1) {
-          if (v > 0.0) product.mul(v);
+        if constexpr (KIND == 0) {
+          s += v[q];
         } else {
-          s += 1.0 / v;
+          bad = bad || !(v[q] > 0.0);
+          if constexpr (KIND == 1) {
+            if (v[q] > 0.0) product.mul(v[q]);
+          } else {
+            s += 1.0 / v[q];
+          }
         }
       }
     }

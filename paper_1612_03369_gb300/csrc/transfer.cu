@@ -32,6 +32,38 @@ __device__ __forceinline__ df minus_half(df t) {  // t - 1/2
 }
 __device__ __forceinline__ double df_to_f64(df a) { return (double)a.hi + (double)a.lo; }
 
+// An FP64 value as a double-float, as df_from_double rounds it, on the integer
+// and FP32 pipes: the high part is the value rounded to 24 bits in the bit
+// field, the low part the 29-bit signed remainder, converted and scaled.
+// (df_from_double's three conversions and a subtraction are 4 FP64-pipe
+// operations, 64 clocks of an SM each for a warp.)  Values outside the range
+// where both parts are normal floats take df_from_double.
+__device__ __forceinline__ df split_f64(double x) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff) - 896;  // the float's exponent field
+  if (e < 60 || e > 250) return df_from_double(x);
+  const long long r = b + (1ll << 28);  // round half up in the magnitude
+  const unsigned mag = ((unsigned)(r >> 29) ^ 0x40000000u) & 0x7fffffffu;
+  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+  const int rem = (int)(b & 0x1fffffff) - (int)(((unsigned)b & 0x10000000u) << 1);  // in [-2^28, 2^28)
+  const float scale = __int_as_float((int)(((unsigned)(e - 52) << 23) | sign));
+  return df_make(__uint_as_float(mag | sign), __fmul_rn((float)rem, scale));
+}
+
+// One particle's loads, issued an iteration ahead of their use.
+template <int D>
+struct ParticleLoads {
+  float2 t[D];
+  double p;
+  __device__ __forceinline__ void load(const float2* __restrict__ xh, const double* __restrict__ prop, size_t cap,
+                                       uint32_t i, uint32_t end) {
+    if (i >= end) return;
+#pragma unroll
+    for (int a = 0; a < D; ++a) t[a] = xh[a * cap + i];
+    p = prop[i];
+  }
+};
+
 // Two phases, both deterministic.
 // Phase 1, thread per cell: each particle of the cell is read once and its
 // 2^D corner weights (the tensor product of (1 - t_a, t_a), multiplied in
@@ -53,15 +85,18 @@ __global__ void __launch_bounds__(128) vertex_partial_kernel(const uint32_t* __r
     if (end > cap || beg > end) {
       latch_status(ctr, PIC_STATUS_BOUNDS);
     } else {
+      ParticleLoads<D> next;
+      next.load(xh, prop, cap, beg, end);
       for (uint32_t i = beg; i < end; ++i) {
+        const ParticleLoads<D> now = next;
+        next.load(xh, prop, cap, i + 1, end);
         df f[D][2];  // f[a][0] = 1 - t_a, f[a][1] = t_a
 #pragma unroll
         for (int a = 0; a < D; ++a) {
-          const float2 v = xh[a * cap + i];
-          f[a][1] = df_make(v.x, v.y);
+          f[a][1] = df_make(now.t[a].x, now.t[a].y);
           f[a][0] = one_minus(f[a][1]);
         }
-        const df p = df_from_double(prop[i]);
+        const df p = split_f64(now.p);
         df w01[4];  // the first two axes' products, corner bits 0 and 1
 #pragma unroll
         for (int c = 0; c < 4; ++c) w01[c] = df_mul(f[0][c & 1], f[1][(c >> 1) & 1]);
@@ -146,15 +181,16 @@ __global__ void __launch_bounds__(128) lsq_linear_kernel(const uint32_t* __restr
     for (int r = 0; r < NB; ++r)
 #pragma unroll
       for (int q = 0; q <= NB; ++q) Ma[r][q] = acc_zero();
+    ParticleLoads<D> next;
+    next.load(xh, prop, cap, beg, end);
     for (uint32_t i = beg; i < end; ++i) {
+      const ParticleLoads<D> now = next;
+      next.load(xh, prop, cap, i + 1, end);
       df a[NB];
       a[0] = df_make(1.0f, 0.f);
 #pragma unroll
-      for (int j = 0; j < D; ++j) {
-        const float2 v = xh[j * cap + i];
-        a[j + 1] = minus_half(df_make(v.x, v.y));
-      }
-      const df p = df_from_double(prop[i]);
+      for (int j = 0; j < D; ++j) a[j + 1] = minus_half(df_make(now.t[j].x, now.t[j].y));
+      const df p = split_f64(now.p);
 #pragma unroll
       for (int r = 0; r < NB; ++r) {
 #pragma unroll
