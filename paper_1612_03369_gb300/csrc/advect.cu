@@ -106,7 +106,8 @@ template <int D, int RK, bool F32B, bool TWO, bool STAGE>
 __global__ void __launch_bounds__(kAdvectThreads, F32B ? PIC_ADVECT_MIN_BLOCKS_F32 : PIC_ADVECT_MIN_BLOCKS_F64)
     advect_kernel(const __grid_constant__ MeshView m, const __grid_constant__ StoreView s,
                   const __grid_constant__ StoreView d, const uint32_t* __restrict__ perm, df dt,
-                  uint32_t* __restrict__ cell_new, uint32_t* __restrict__ counts, DevCounters* __restrict__ ctr) {
+                  uint32_t* __restrict__ cell_new, uint32_t* __restrict__ counts, uint32_t* __restrict__ tile_next,
+                  DevCounters* __restrict__ ctr) {
   using L = StageLayout<D, F32B>;
   extern __shared__ float4 stage_smem[];  // STAGE: [warp][2 buffers][BUF]
   __shared__ __align__(8) uint64_t bars[kAdvectWarps][2];
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(kAdvectThreads, F32B ? PIC_ADVECT_MIN_BLOCKS_F
   const uint32_t* __restrict__ start_cell = perm ? d.cell : s.cell;
   auto grab = [&]() -> uint32_t {
     uint32_t t = 0;
-    if (lane == 0) t = atomicAdd(&ctr->tile_next, 1u);
+    if (lane == 0) t = atomicAdd(tile_next, 1u);
     return __shfl_sync(0xffffffffu, t, 0);
   };
   auto start_of = [&](uint32_t t) -> uint32_t {
@@ -223,12 +224,13 @@ __global__ void __launch_bounds__(kAdvectThreads, PIC_ADVECT_MIN_BLOCKS_F64)
     advect_record_kernel(const __grid_constant__ MeshView m, const __grid_constant__ StoreView s,
                          const __grid_constant__ StoreView d, const uint32_t* __restrict__ perm, df dt,
                          const __grid_constant__ StageRec rec, uint32_t* __restrict__ cell_new,
-                         uint32_t* __restrict__ counts, DevCounters* __restrict__ ctr) {
+                         uint32_t* __restrict__ counts, uint32_t* __restrict__ tile_next,
+                         DevCounters* __restrict__ ctr) {
   const int lane = threadIdx.x & 31;
   const uint32_t n = ctr->n_alive, ntiles = (n + 31) / 32;
   auto grab = [&]() -> uint32_t {
     uint32_t t = 0;
-    if (lane == 0) t = atomicAdd(&ctr->tile_next, 1u);
+    if (lane == 0) t = atomicAdd(tile_next, 1u);
     return __shfl_sync(0xffffffffu, t, 0);
   };
   for (uint32_t t = grab(); t < ntiles;) {
@@ -448,13 +450,13 @@ static void launch_advect(pic_particles_s* p, const MeshView& m, double dt, bool
   const int grid = advect_grid(p->capacity, F32B);
   if (m.has_next) {
     advect_kernel<D, RK, F32B, true, false><<<grid, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, p->cell_new,
-                                                                             p->counts, p->ctr);
+                                                                             p->counts, p->tile_next, p->ctr);
   } else if (D == 3 && p->stage_cells) {
     advect_kernel<D, RK, F32B, false, D == 3><<<grid, kAdvectThreads, StageLayout<D, F32B>::bytes(), st>>>(
-        m, s, d, perm, dtd, p->cell_new, p->counts, p->ctr);
+        m, s, d, perm, dtd, p->cell_new, p->counts, p->tile_next, p->ctr);
   } else {
     advect_kernel<D, RK, F32B, false, false><<<grid, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, p->cell_new,
-                                                                              p->counts, p->ctr);
+                                                                              p->counts, p->tile_next, p->ctr);
   }
   count_launches(1);
   if (fused) p->cur = 1 - p->cur;
@@ -469,18 +471,20 @@ static void launch_record_d(pic_particles_s* p, const MeshView& m, double dt, in
   const uint32_t* perm = fused ? p->perm : nullptr;
   const int g = advect_grid(p->capacity, false);
   if (rk == 1)
-    advect_record_kernel<D, 1><<<g, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, rec, p->cell_new, p->counts, p->ctr);
+    advect_record_kernel<D, 1><<<g, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, rec, p->cell_new, p->counts, p->tile_next, p->ctr);
   else if (rk == 2)
-    advect_record_kernel<D, 2><<<g, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, rec, p->cell_new, p->counts, p->ctr);
+    advect_record_kernel<D, 2><<<g, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, rec, p->cell_new, p->counts, p->tile_next, p->ctr);
   else
-    advect_record_kernel<D, 4><<<g, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, rec, p->cell_new, p->counts, p->ctr);
+    advect_record_kernel<D, 4><<<g, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, rec, p->cell_new, p->counts, p->tile_next, p->ctr);
   count_launches(1);
 }
 
 pic_status launch_advect_record(pic_particles_s* p, const MeshView& m, double dt, int rk, const StageRec& rec,
                                 cudaStream_t st) {
-  PIC_CUDA(cudaMemsetAsync(p->counts, 0, sizeof(uint32_t) * p->C, st));
-  PIC_CUDA(cudaMemsetAsync(&p->ctr->tile_next, 0, sizeof(unsigned int), st));
+  {
+    const pic_status r0 = clear_step_scratch(p, st);
+    if (r0 != PIC_OK) return r0;
+  }
   const bool fused = p->pending_order != 0;
   if (p->dim == 2)
     launch_record_d<2>(p, m, dt, rk, rec, fused, st);
@@ -546,8 +550,10 @@ extern "C" pic_status pic_advect(pic_particles parts, pic_mesh mesh, double dt, 
   // call (see settle_order).
   bool pending = parts->pending_order != 0;
   for (int step = 0; step < n_steps; ++step) {
-    PIC_CUDA(cudaMemsetAsync(parts->counts, 0, sizeof(uint32_t) * parts->C, st));
-    PIC_CUDA(cudaMemsetAsync(&parts->ctr->tile_next, 0, sizeof(unsigned int), st));
+    {
+      const pic_status r0 = clear_step_scratch(parts, st);
+      if (r0 != PIC_OK) return r0;
+    }
     cudaEvent_t* ev = parts->timing ? timing_slot(parts) : nullptr;
     if (ev) PIC_CUDA(cudaEventRecord(ev[0], st));
     const bool f32 = precision != PIC_FP64;
@@ -583,7 +589,10 @@ extern "C" pic_status pic_locate(pic_particles parts, pic_mesh mesh, void* strea
     if (r0 != PIC_OK) return r0;
   }
   const MeshView m = mesh_view(mesh);
-  PIC_CUDA(cudaMemsetAsync(parts->counts, 0, sizeof(uint32_t) * parts->C, st));
+  {
+    const pic_status r0 = clear_step_scratch(parts, st);
+    if (r0 != PIC_OK) return r0;
+  }
   if (mesh->dim == 2)
     relocate_kernel<2><<<grid_for(parts->capacity, 128), 128, 0, st>>>(m, store_view(parts, parts->cur),
                                                                        parts->cell_new, parts->counts, parts->ctr);

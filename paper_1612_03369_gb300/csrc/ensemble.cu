@@ -213,10 +213,11 @@ template <int D, int RK>
 __global__ void __launch_bounds__(kEnsBlock, ens_min_blocks<D>()) ensemble_advect_kernel(
     const MeshView* __restrict__ views, const uint32_t* __restrict__ base, const df* __restrict__ dts, int P,
     const __grid_constant__ StoreView s, const __grid_constant__ StoreView d, const uint32_t* __restrict__ perm,
-    uint32_t tile, uint32_t* __restrict__ cell_new, uint32_t* __restrict__ counts, DevCounters* __restrict__ ctr) {
+    uint32_t tile, uint32_t* __restrict__ cell_new, uint32_t* __restrict__ counts, uint32_t* __restrict__ tile_next,
+    DevCounters* __restrict__ ctr) {
   __shared__ EnsShared sh;
   load_ensemble(sh, base, dts, P);
-  ensemble_advect_tiles<D, RK>(sh, views, P, s, d, perm, ctr->n_alive, tile, &ctr->tile_next, cell_new, counts, ctr);
+  ensemble_advect_tiles<D, RK>(sh, views, P, s, d, perm, ctr->n_alive, tile, tile_next, cell_new, counts, ctr);
 }
 
 struct PersistArgs {
@@ -522,21 +523,23 @@ static pic_status enqueue_run(pic_ensemble_s* e, int integrator, int n_steps, in
     const int grid = ensemble_advect_blocks_per_sm(e->dim, rk) * num_sms();
     const uint32_t tile = (uint32_t)e->tile;
     for (int step = 0; step < n_steps; ++step) {
-      PIC_CUDA(cudaMemsetAsync(s->counts, 0, sizeof(uint32_t) * s->C, st));
-      PIC_CUDA(cudaMemsetAsync(&s->ctr->tile_next, 0, sizeof(uint32_t), st));
+      {
+        const pic_status r0 = clear_step_scratch(s, st);
+        if (r0 != PIC_OK) return r0;
+      }
       // as in pic_advect: each step applies the previous step's order on the
       // way, and the last step's order is applied by one gather
       const bool fused = step > 0;
       const StoreView sv = store_view(s, s->cur), dv = fused ? store_view(s, 1 - s->cur) : sv;
       const uint32_t* pm = fused ? s->perm : nullptr;
       if (e->dim == 2) {
-        if (rk == 1) ensemble_advect_kernel<2, 1><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->ctr);
-        else if (rk == 2) ensemble_advect_kernel<2, 2><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->ctr);
-        else ensemble_advect_kernel<2, 4><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->ctr);
+        if (rk == 1) ensemble_advect_kernel<2, 1><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->tile_next, s->ctr);
+        else if (rk == 2) ensemble_advect_kernel<2, 2><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->tile_next, s->ctr);
+        else ensemble_advect_kernel<2, 4><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->tile_next, s->ctr);
       } else {
-        if (rk == 1) ensemble_advect_kernel<3, 1><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->ctr);
-        else if (rk == 2) ensemble_advect_kernel<3, 2><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->ctr);
-        else ensemble_advect_kernel<3, 4><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->ctr);
+        if (rk == 1) ensemble_advect_kernel<3, 1><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->tile_next, s->ctr);
+        else if (rk == 2) ensemble_advect_kernel<3, 2><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->tile_next, s->ctr);
+        else ensemble_advect_kernel<3, 4><<<grid, kEnsBlock, 0, st>>>(e->views_dev, e->base_dev, e->dt_dev, e->P, sv, dv, pm, tile, s->cell_new, s->counts, s->tile_next, s->ctr);
       }
       count_launches(1);
       PIC_CUDA(cudaGetLastError());

@@ -146,7 +146,10 @@ extern "C" pic_status pic_merge_particles(pic_particles p, uint32_t keep_lo, uin
     return (set_error("pic_merge_particles: %u + %zu particles exceed the capacity %zu", n_old, n_in, p->capacity),
             PIC_ERR_CAPACITY);
   const uint32_t total = n_old + (uint32_t)n_in;
-  PIC_CUDA(cudaMemsetAsync(p->counts, 0, sizeof(uint32_t) * p->C, st));
+  {
+    const pic_status r0 = clear_step_scratch(p, st);
+    if (r0 != PIC_OK) return r0;
+  }
   if (total) {
     const size_t want = ((size_t)total + 255) / 256, cap = (size_t)num_sms() * 16;
     const int g = (int)(want < cap ? want : cap);

@@ -132,8 +132,9 @@ pic_particles_s* store_alloc(int dim, int n_props, uint32_t C, size_t capacity, 
   }
   slab.add(&p->cell_new, cap);
   slab.add(&p->counts, C);
-  slab.add(&p->cursor, C);
   slab.add(&p->block_sums, scan_scratch_bytes(C) / sizeof(uint32_t));
+  slab.add(&p->tile_next, 1);
+  slab.add(&p->cursor, C);
   slab.add(&p->key_id, cap);
   slab.add(&p->key_src, cap);
   slab.add(&p->perm, cap);

@@ -47,8 +47,7 @@ struct DevCounters {
   unsigned int n_alive;  // particles in the store
   unsigned int n_next;   // particles after the pending rebin
   unsigned int fail_count;
-  unsigned int tile_next;  // work counter of the advect kernel's dynamic tiles (cleared before each launch)
-  unsigned int pad_;
+  unsigned int pad_[2];
 };
 
 }  // namespace pic
@@ -141,9 +140,12 @@ struct pic_particles_s {
   uint32_t* cell_off;     // [C+1]
   // scratch for the rebin
   uint32_t* cell_new;     // [capacity]
+  // counts, block_sums and tile_next lie one after another: a step clears the
+  // three with one memset (clear_step_scratch)
   uint32_t* counts;       // [C]
-  uint32_t* cursor;       // [C]
   uint32_t* block_sums;   // scan scratch (scan_scratch_bytes(C))
+  uint32_t* tile_next;    // work counter of the advect kernel's dynamic tiles
+  uint32_t* cursor;       // [C]
   uint64_t* key_id;       // [capacity]
   uint32_t* key_src;      // [capacity]
   uint32_t* perm;         // [capacity]
@@ -444,6 +446,7 @@ void launch_pack(pic_particles_s* p, int buf, const uint32_t* perm, size_t first
                  const PackedOut& o, cudaStream_t s);
 // Rebuild the sorted store from the cells found by the last locate
 // (cell_new, counts already filled).  Defined in rebin.cu.
+// A counting kernel preceded by clear_step_scratch comes first.
 pic_status rebin_from_counts(pic_particles_s* p, cudaStream_t s);
 // The two halves of rebin_from_counts: the new order (perm, offsets, sorted
 // cells in the other buffer), then the gather that applies it.
@@ -477,9 +480,12 @@ pic_status seed_prepare(pic_mesh mesh, const uint32_t* per_cell, uint32_t unifor
 // Exclusive scan of n u32 values into out[0..n] (out[n] = total); total also
 // written to *total_dev when non-null; cursor_init, when non-null, receives
 // out[0..n) too.  scratch: scan_scratch_bytes(n) bytes (cleared by the
-// call).  Defined in rebin.cu.
+// call unless the caller has).  Defined in rebin.cu.
 pic_status scan_u32(const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* scratch, uint32_t* total_dev,
-                    uint32_t* cursor_init, cudaStream_t s, unsigned int* status = nullptr);
+                    uint32_t* cursor_init, cudaStream_t s, unsigned int* status = nullptr, bool cleared = false);
+// Clears what a counting step starts from: the per-cell counts, the rebin
+// scan's state and the tile counter.
+pic_status clear_step_scratch(pic_particles_s* p, cudaStream_t s);
 int num_sms();
 // Allocate a store (particles.cu); takes ownership of cell_off.
 pic_particles_s* store_alloc(int dim, int n_props, uint32_t C, size_t capacity, uint32_t* cell_off);

@@ -125,11 +125,11 @@ __global__ void __launch_bounds__(kScanThreads) scan_single_pass_kernel(const ui
 // The scan's status word: the store's counters where there is one, else a
 // word of the scratch past the tile states (cleared with them).
 pic_status scan_u32(const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* scratch, uint32_t* total_dev,
-                    uint32_t* cursor_init, cudaStream_t s, unsigned int* status) {
+                    uint32_t* cursor_init, cudaStream_t s, unsigned int* status, bool cleared) {
   if (n == 0) return PIC_OK;
   const uint32_t nt = scan_tiles(n);
   uint64_t* state = reinterpret_cast<uint64_t*>(scratch);
-  PIC_CUDA(cudaMemsetAsync(state, 0, sizeof(uint64_t) * (nt + 1), s));
+  if (!cleared) PIC_CUDA(cudaMemsetAsync(state, 0, sizeof(uint64_t) * (nt + 1), s));
   unsigned int* st = status ? status : reinterpret_cast<unsigned int*>(state + nt) + 1;
   scan_single_pass_kernel<<<nt, kScanThreads, 0, s>>>(in, n, state, out, cursor_init, total_dev, st);
   count_launches(1);
@@ -184,11 +184,17 @@ static int grid_cap(size_t n, int block, int per_sm) {
   return (int)(g ? g : 1);
 }
 
+pic_status clear_step_scratch(pic_particles_s* p, cudaStream_t s) {
+  PIC_CUDA(cudaMemsetAsync(p->counts, 0, (size_t)((char*)(p->tile_next + 1) - (char*)p->counts), s));
+  return PIC_OK;
+}
+
 // The new order of the store after a step: cell offsets, perm (new slot ->
 // old slot) and the sorted cells written into the other buffer; n_alive
 // becomes the survivors' count.  The particles have not moved yet.
 pic_status rebin_order_from_counts(pic_particles_s* p, cudaStream_t s) {
-  pic_status r = scan_u32(p->counts, p->cell_off, p->C, p->block_sums, &p->ctr->n_next, p->cursor, s, &p->ctr->status);
+  pic_status r = scan_u32(p->counts, p->cell_off, p->C, p->block_sums, &p->ctr->n_next, p->cursor, s, &p->ctr->status,
+                          true);
   if (r != PIC_OK) return r;
   const StoreView a = store_view(p, p->cur), b = store_view(p, 1 - p->cur);
   scatter_keys_kernel<<<grid_cap(p->capacity, 256, 16), 256, 0, s>>>(p->cell_new, a.id, p->cursor, p->key_id, p->key_src,
@@ -334,7 +340,10 @@ extern "C" pic_status pic_rebin(pic_particles parts, void* stream) {
     const pic_status r0 = settle_order(parts, st);
     if (r0 != PIC_OK) return r0;
   }
-  PIC_CUDA(cudaMemsetAsync(parts->counts, 0, sizeof(uint32_t) * parts->C, st));
+  {
+    const pic_status r0 = clear_step_scratch(parts, st);
+    if (r0 != PIC_OK) return r0;
+  }
   identity_cells_kernel<<<grid_cap(parts->capacity, 256, 16), 256, 0, st>>>(parts->cell[parts->cur], parts->cell_new,
                                                                           parts->counts, parts->C, parts->ctr);
   count_launches(1);
