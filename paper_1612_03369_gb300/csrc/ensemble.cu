@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kEnsBlock, ens_min_blocks<D>()) ensemble_persi
     const uint32_t nn = *(volatile uint32_t*)&A.ctr->n_next;
     for (uint32_t c = gtid; c < A.C; c += gthreads) A.counts[c] = 0u;
     if (gtid == 0) A.ctr->n_alive = nn;
-    scatter_phase(A.cell_new, cur.id, A.cursor, A.key_id, A.key_src, A.C, A.cap, n, &A.ctr->status, gtid, gthreads);
+    scatter_phase(A.cell_new, cur.id, nullptr, A.cursor, A.key_id, A.key_src, A.C, A.cap, n, &A.ctr->status, gtid, gthreads);
     if (!grid_sync(A.bar, nb, A.timeout_ns)) return;
     rank_phase(A.cell_off, A.key_id, A.key_src, A.perm, nxt.cell, A.C, A.cap, &A.ctr->status, gtid >> 5,
                gthreads >> 5);
@@ -426,10 +426,7 @@ extern "C" pic_status pic_ensemble_create(int n_problems, const pic_mesh* meshes
   e->store = store_alloc(dim, n_props, C, N, off);
   if (!e->store) return fail(PIC_ERR_OOM);
   e->store->stream = st;
-  DevCounters h{};
-  h.n_alive = (uint32_t)N;
-  h.n_next = (uint32_t)N;
-  PIC_CUDA(cudaMemcpyAsync(e->store->ctr, &h, sizeof(h), cudaMemcpyHostToDevice, st));
+  PIC_CUDA(store_init(e->store, (uint32_t)N, st));
   for (int p = 0; p < n_problems; ++p) {
     const uint32_t Cp = meshes[p]->C;
     const int grid = (int)((Cp + 127) / 128 < 8192 ? (Cp + 127) / 128 : 8192);
@@ -519,6 +516,9 @@ static cudaError_t launch_persistent(const PersistArgs& A, int grid, cudaStream_
 static pic_status enqueue_run(pic_ensemble_s* e, int integrator, int n_steps, int mode, cudaStream_t st) {
   pic_particles_s* s = e->store;
   const int rk = integrator;
+  // a graph of the steps is replayed whatever ran before, so it clears the
+  // scratch itself; the persistent kernel leaves the cursors used
+  s->scratch_clear = 0;
   if (mode == 0) {
     const int grid = ensemble_advect_blocks_per_sm(e->dim, rk) * num_sms();
     const uint32_t tile = (uint32_t)e->tile;
@@ -670,6 +670,7 @@ extern "C" pic_status pic_ensemble_run(pic_ensemble e, pic_integrator integrator
     }
     PIC_CUDA(cudaGraphLaunch(e->cache[hit].exec, st));
     if (n_steps & 1) e->store->cur = 1 - e->store->cur;
+    e->store->scratch_clear = mode == 0;
     r = PIC_OK;
   }
   if (r != PIC_OK) return r;

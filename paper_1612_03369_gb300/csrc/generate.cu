@@ -715,10 +715,7 @@ extern "C" pic_status pic_import_particles(pic_mesh mesh, size_t n, const double
   }
   p->mesh = mesh;
   p->stream = st;
-  DevCounters h{};
-  h.n_alive = kept;
-  h.n_next = kept;
-  cudaError_t e = cudaMemcpyAsync(p->ctr, &h, sizeof(h), cudaMemcpyHostToDevice, st);
+  cudaError_t e = store_init(p, kept, st);
   if (e == cudaSuccess && kept > 0) {
     if (d == 2)
       import_gather_kernel<2><<<gen_grid(kept, 128), 128, 0, st>>>(store_view(p, 0), perm, off + C, n, x, xh, cell, id);

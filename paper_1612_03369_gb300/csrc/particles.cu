@@ -131,10 +131,10 @@ pic_particles_s* store_alloc(int dim, int n_props, uint32_t C, size_t capacity, 
     slab.add(&p->props[b], (size_t)(n_props > 0 ? n_props : 1) * cap);
   }
   slab.add(&p->cell_new, cap);
+  slab.add(&p->cursor, C);
   slab.add(&p->counts, C);
   slab.add(&p->block_sums, scan_scratch_bytes(C) / sizeof(uint32_t));
   slab.add(&p->tile_next, 1);
-  slab.add(&p->cursor, C);
   slab.add(&p->key_id, cap);
   slab.add(&p->key_src, cap);
   slab.add(&p->perm, cap);
@@ -145,6 +145,18 @@ pic_particles_s* store_alloc(int dim, int n_props, uint32_t C, size_t capacity, 
     return nullptr;
   }
   return p;
+}
+
+cudaError_t store_init(pic_particles_s* p, uint32_t n, cudaStream_t s) {
+  DevCounters h{};
+  h.n_alive = n;
+  h.n_next = n;
+  const cudaError_t e = cudaMemcpyAsync(p->ctr, &h, sizeof(h), cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return e;
+  p->scratch_clear = 0;
+  if (clear_step_scratch(p, s) != PIC_OK) return cudaErrorUnknown;
+  p->scratch_clear = 1;
+  return cudaSuccess;
 }
 
 }  // namespace pic
@@ -218,10 +230,7 @@ pic_status seed_prepare(pic_mesh mesh, const uint32_t* per_cell, uint32_t unifor
   if (!p) return PIC_ERR_OOM;
   p->mesh = mesh;
   p->stream = st;
-  DevCounters h{};
-  h.n_alive = (uint32_t)N;
-  h.n_next = (uint32_t)N;
-  cudaError_t e = cudaMemcpyAsync(p->ctr, &h, sizeof(h), cudaMemcpyHostToDevice, st);
+  const cudaError_t e = store_init(p, (uint32_t)N, st);
   if (e != cudaSuccess) {
     pic_destroy_particles(p);
     return cuda_fail(e, who);

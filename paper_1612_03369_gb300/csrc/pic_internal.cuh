@@ -140,12 +140,13 @@ struct pic_particles_s {
   uint32_t* cell_off;     // [C+1]
   // scratch for the rebin
   uint32_t* cell_new;     // [capacity]
-  // counts, block_sums and tile_next lie one after another: a step clears the
-  // three with one memset (clear_step_scratch)
+  // cursor, counts, block_sums and tile_next lie one after another: what a
+  // counting step starts from cleared (see clear_step_scratch)
+  uint32_t* cursor;       // [C]
   uint32_t* counts;       // [C]
   uint32_t* block_sums;   // scan scratch (scan_scratch_bytes(C))
   uint32_t* tile_next;    // work counter of the advect kernel's dynamic tiles
-  uint32_t* cursor;       // [C]
+  int scratch_clear;      // they are clear (or will be, in stream order)
   uint64_t* key_id;       // [capacity]
   uint32_t* key_src;      // [capacity]
   uint32_t* perm;         // [capacity]
@@ -483,9 +484,13 @@ pic_status seed_prepare(pic_mesh mesh, const uint32_t* per_cell, uint32_t unifor
 // call unless the caller has).  Defined in rebin.cu.
 pic_status scan_u32(const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* scratch, uint32_t* total_dev,
                     uint32_t* cursor_init, cudaStream_t s, unsigned int* status = nullptr, bool cleared = false);
-// Clears what a counting step starts from: the per-cell counts, the rebin
-// scan's state and the tile counter.
+// Clears what a counting step starts from (the per-cell counts, the rebin
+// scan's state, the tile counter; the cursors too where scatter_scan_kernel
+// counts in them), unless the last rebin's rank kernel has: it clears them for
+// the next step, so that a sequence of steps needs no memset.
 pic_status clear_step_scratch(pic_particles_s* p, cudaStream_t s);
+// A new store's counters (n particles) and cleared scratch, on its stream.
+cudaError_t store_init(pic_particles_s* p, uint32_t n, cudaStream_t s);
 int num_sms();
 // Allocate a store (particles.cu); takes ownership of cell_off.
 pic_particles_s* store_alloc(int dim, int n_props, uint32_t C, size_t capacity, uint32_t* cell_off);

@@ -144,17 +144,58 @@ __global__ void __launch_bounds__(256) scatter_keys_kernel(const uint32_t* __res
                                                            uint64_t* __restrict__ key_id, uint32_t* __restrict__ key_src,
                                                            uint32_t C, size_t cap, const uint32_t* __restrict__ n_dev,
                                                            unsigned int* __restrict__ status) {
-  scatter_phase(cell_new, id, cursor, key_id, key_src, C, cap, *n_dev, status, blockIdx.x * blockDim.x + threadIdx.x,
-                gridDim.x * blockDim.x);
+  scatter_phase(cell_new, id, nullptr, cursor, key_id, key_src, C, cap, *n_dev, status,
+                blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+// Scan and scatter in one launch for a mesh of at most kScanTileCells cells:
+// every block scans all the counts into its shared memory (one tile's scan,
+// ~1 us) and scatters its particles behind those offsets; block 0 also writes
+// the offsets and their total.  cursor starts from 0.  A scan kernel of its own
+// costs a small store's step 3.7 us and a launch gap of 2.
+__global__ void __launch_bounds__(256) scatter_scan_kernel(const uint32_t* __restrict__ cell_new,
+                                                           const uint64_t* __restrict__ id,
+                                                           const uint32_t* __restrict__ counts,
+                                                           uint32_t* __restrict__ cursor, uint32_t* __restrict__ cell_off,
+                                                           uint32_t* __restrict__ total_dev, uint64_t* __restrict__ key_id,
+                                                           uint32_t* __restrict__ key_src, uint32_t C, size_t cap,
+                                                           const uint32_t* __restrict__ n_dev,
+                                                           unsigned int* __restrict__ status) {
+  constexpr uint32_t kPer = kScanTileCells / 256;
+  __shared__ uint32_t s_off[kScanTileCells], s_total;
+  for (uint32_t k = threadIdx.x; k < kScanTileCells; k += 256) s_off[k] = k < C ? counts[k] : 0u;
+  __syncthreads();
+  uint32_t sum = 0;
+  for (uint32_t q = 0; q < kPer; ++q) sum += s_off[threadIdx.x * kPer + q];
+  uint32_t run = block_excl_scan(sum, &s_total);
+  for (uint32_t q = 0; q < kPer; ++q) {
+    const uint32_t k = threadIdx.x * kPer + q, c = s_off[k];
+    s_off[k] = run;
+    run += c;
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    for (uint32_t k = threadIdx.x; k < C; k += 256) cell_off[k] = s_off[k];
+    if (threadIdx.x == 0) {
+      cell_off[C] = s_total;
+      *total_dev = s_total;
+    }
+  }
+  scatter_phase(cell_new, id, s_off, cursor, key_id, key_src, C, cap, *n_dev, status,
+                blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // Rank by id within each cell.  cell_out may be NULL.  When publish_dst is
-// given, block 0 copies *publish_src there (the new particle count).
+// given, block 0 copies *publish_src there (the new particle count).  The
+// clear_words words at clear are set to 0 (the next step's scratch: nothing
+// here reads it).
 __global__ void __launch_bounds__(256) rank_by_id_kernel(const uint32_t* __restrict__ cell_off, const uint64_t* __restrict__ key_id,
                                                          const uint32_t* __restrict__ key_src, uint32_t* __restrict__ perm,
                                                          uint32_t* __restrict__ cell_out, uint32_t C, size_t cap,
                                                          unsigned int* __restrict__ status, uint32_t* publish_dst,
-                                                         const uint32_t* publish_src) {
+                                                         const uint32_t* publish_src, uint32_t* __restrict__ clear,
+                                                         uint32_t clear_words) {
+  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < clear_words; k += gridDim.x * blockDim.x) clear[k] = 0u;
   if (publish_dst && blockIdx.x == 0 && threadIdx.x == 0) *publish_dst = *publish_src;
   rank_phase(cell_off, key_id, key_src, perm, cell_out, C, cap, status, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
              (gridDim.x * blockDim.x) >> 5);
@@ -184,8 +225,13 @@ static int grid_cap(size_t n, int block, int per_sm) {
   return (int)(g ? g : 1);
 }
 
+static bool one_scan_tile(const pic_particles_s* p) { return p->C <= kScanTileCells; }
+static uint32_t* step_scratch(const pic_particles_s* p) { return one_scan_tile(p) ? p->cursor : p->counts; }
+static uint32_t step_scratch_words(const pic_particles_s* p) { return (uint32_t)(p->tile_next + 1 - step_scratch(p)); }
+
 pic_status clear_step_scratch(pic_particles_s* p, cudaStream_t s) {
-  PIC_CUDA(cudaMemsetAsync(p->counts, 0, (size_t)((char*)(p->tile_next + 1) - (char*)p->counts), s));
+  if (!p->scratch_clear) PIC_CUDA(cudaMemsetAsync(step_scratch(p), 0, sizeof(uint32_t) * step_scratch_words(p), s));
+  p->scratch_clear = 0;  // until a rebin has run to its end
   return PIC_OK;
 }
 
@@ -193,17 +239,24 @@ pic_status clear_step_scratch(pic_particles_s* p, cudaStream_t s) {
 // old slot) and the sorted cells written into the other buffer; n_alive
 // becomes the survivors' count.  The particles have not moved yet.
 pic_status rebin_order_from_counts(pic_particles_s* p, cudaStream_t s) {
-  pic_status r = scan_u32(p->counts, p->cell_off, p->C, p->block_sums, &p->ctr->n_next, p->cursor, s, &p->ctr->status,
-                          true);
-  if (r != PIC_OK) return r;
   const StoreView a = store_view(p, p->cur), b = store_view(p, 1 - p->cur);
-  scatter_keys_kernel<<<grid_cap(p->capacity, 256, 16), 256, 0, s>>>(p->cell_new, a.id, p->cursor, p->key_id, p->key_src,
-                                                                     p->C, p->capacity, &p->ctr->n_alive, &p->ctr->status);
-  rank_by_id_kernel<<<grid_cap((size_t)p->C * 32, 256, 16), 256, 0, s>>>(p->cell_off, p->key_id, p->key_src, p->perm,
-                                                                        b.cell, p->C, p->capacity, &p->ctr->status,
-                                                                        &p->ctr->n_alive, &p->ctr->n_next);
+  const int g = grid_cap(p->capacity, 256, 16);
+  if (one_scan_tile(p)) {
+    scatter_scan_kernel<<<g, 256, 0, s>>>(p->cell_new, a.id, p->counts, p->cursor, p->cell_off, &p->ctr->n_next, p->key_id,
+                                          p->key_src, p->C, p->capacity, &p->ctr->n_alive, &p->ctr->status);
+  } else {
+    pic_status r = scan_u32(p->counts, p->cell_off, p->C, p->block_sums, &p->ctr->n_next, p->cursor, s,
+                            &p->ctr->status, true);
+    if (r != PIC_OK) return r;
+    scatter_keys_kernel<<<g, 256, 0, s>>>(p->cell_new, a.id, p->cursor, p->key_id, p->key_src, p->C, p->capacity,
+                                          &p->ctr->n_alive, &p->ctr->status);
+  }
+  rank_by_id_kernel<<<grid_cap((size_t)p->C * 32, 256, 16), 256, 0, s>>>(
+      p->cell_off, p->key_id, p->key_src, p->perm, b.cell, p->C, p->capacity, &p->ctr->status, &p->ctr->n_alive,
+      &p->ctr->n_next, step_scratch(p), step_scratch_words(p));
   count_launches(2);
   PIC_CUDA(cudaGetLastError());
+  p->scratch_clear = 1;
   return PIC_OK;
 }
 
@@ -300,7 +353,7 @@ pic_status sort_by_cell_run(size_t n, const uint32_t* cell, const uint64_t* id, 
     scatter_keys_kernel<<<grid_cap(n, 256, 16), 256, 0, s>>>(cell, id, sc.cursor, sc.key_id, sc.key_src, C, n, sc.misc,
                                                              sc.misc + 1);
     rank_by_id_kernel<<<grid_cap((size_t)C * 32, 256, 16), 256, 0, s>>>(cell_off, sc.key_id, sc.key_src, perm, nullptr, C,
-                                                                        n, sc.misc + 1, nullptr, nullptr);
+                                                                        n, sc.misc + 1, nullptr, nullptr, nullptr, 0u);
   }
   count_launches(n ? 4 : 1);
   PIC_CUDA(cudaGetLastError());

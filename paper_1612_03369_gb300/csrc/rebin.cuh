@@ -127,13 +127,15 @@ __device__ __forceinline__ uint32_t aggregated_increment(uint32_t* __restrict__ 
 }
 
 // (id, old slot) of every located particle i < n into a free slot of its new
-// cell.  first - lane and stride must be multiples of 32 (whole warps), so
+// cell: cursor[K] counts from the cell's offset, or from 0 with the offsets in
+// off.  first - lane and stride must be multiples of 32 (whole warps), so
 // that every lane of a warp takes part in the aggregated increments.  Each
 // thread takes U particles per pass and issues their loads, then the U
 // warp-aggregated atomics, before it waits on any of them (memory-level
 // parallelism when the grid is small, as in a persistent kernel).
 __device__ __forceinline__ void scatter_phase(const uint32_t* __restrict__ cell_new, const uint64_t* __restrict__ id,
-                                              uint32_t* __restrict__ cursor, uint64_t* __restrict__ key_id,
+                                              const uint32_t* off, uint32_t* __restrict__ cursor,
+                                              uint64_t* __restrict__ key_id,
                                               uint32_t* __restrict__ key_src, uint32_t C, size_t cap, uint32_t n,
                                               unsigned int* __restrict__ status, uint32_t first, uint32_t stride) {
   constexpr int U = 4;
@@ -164,8 +166,9 @@ __device__ __forceinline__ void scatter_phase(const uint32_t* __restrict__ cell_
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const uint32_t slot = __shfl_sync(0xffffffffu, old[u], __ffs(peers[u]) - 1) + (uint32_t)__popc(peers[u] & below);
+      uint32_t slot = __shfl_sync(0xffffffffu, old[u], __ffs(peers[u]) - 1) + (uint32_t)__popc(peers[u] & below);
       if (K[u] >= C) continue;
+      if (off) slot += off[K[u]];
       if (slot >= cap) {
         atomicOr(status, PIC_STATUS_BOUNDS);
         continue;
