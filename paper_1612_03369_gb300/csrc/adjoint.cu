@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(128, PIC_ADVECT_MIN_BLOCKS) replay_step_kernel
     int iters = 0;
     unsigned flags = 0;
     uint32_t full = 0;
-    (void)advect_particle_step<D, RK, false, false>(GlobalCells<D, false>{m}, m, s, i, sink, i, s.cell[i], dt, iters,
+    (void)advect_particle_step<D, RK, false, kSteady>(GlobalCells<D, false>{m}, m, s, i, sink, i, s.cell[i], dt, iters,
                                                     flags, full, RecordHook{rec, i});
   }
 }

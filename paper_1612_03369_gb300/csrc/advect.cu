@@ -58,7 +58,7 @@ struct StageLayout {
 // d.cell[j], its id and properties are carried over), else slot j of s in
 // place.  Returns the new cell (PIC_LOST if none); *full is set when the full
 // path redid it.
-template <int D, int RK, bool F32B, bool TWO, class Hook, class Cells>
+template <int D, int RK, bool F32B, int TWO, class Hook, class Cells>
 __device__ __forceinline__ uint32_t tile_particle(const Cells& cs, const MeshView& m, const StoreView& s,
                                                   const StoreView& d, const uint32_t* __restrict__ perm, df dt,
                                                   uint32_t j, int& iters, unsigned& flags, uint32_t& full, Hook hook) {
@@ -102,7 +102,7 @@ __device__ __forceinline__ void finish_tile(DevCounters* __restrict__ ctr, uint3
 #ifndef PIC_ADVECT_MIN_BLOCKS_F32
 #define PIC_ADVECT_MIN_BLOCKS_F32 6
 #endif
-template <int D, int RK, bool F32B, bool TWO, bool STAGE>
+template <int D, int RK, bool F32B, int TWO, bool STAGE>
 __global__ void __launch_bounds__(kAdvectThreads, F32B ? PIC_ADVECT_MIN_BLOCKS_F32 : PIC_ADVECT_MIN_BLOCKS_F64)
     advect_kernel(const __grid_constant__ MeshView m, const __grid_constant__ StoreView s,
                   const __grid_constant__ StoreView d, const uint32_t* __restrict__ perm, df dt,
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kAdvectThreads, PIC_ADVECT_MIN_BLOCKS_F64)
     uint32_t Kc = PIC_LOST, full = 0;
     if (j < n) {
       steps = 1;
-      Kc = tile_particle<D, RK, false, false>(GlobalCells<D, false>{m}, m, s, d, perm, dt, j, iters, flags, full,
+      Kc = tile_particle<D, RK, false, kSteady>(GlobalCells<D, false>{m}, m, s, d, perm, dt, j, iters, flags, full,
                                               RecordHook{rec, j});
       cell_new[j] = Kc;
     }
@@ -449,13 +449,21 @@ static void launch_advect(pic_particles_s* p, const MeshView& m, double dt, bool
   const uint32_t* perm = fused ? p->perm : nullptr;
   const int grid = advect_grid(p->capacity, F32B);
   if (m.has_next) {
-    advect_kernel<D, RK, F32B, true, false><<<grid, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, p->cell_new,
-                                                                             p->counts, p->tile_next, p->ctr);
+    // the mean field's table where there is one (double-float form; it is left
+    // out when memory is short)
+    if constexpr (!F32B) {
+      if (m.Qch)
+        advect_kernel<D, RK, F32B, kMidTable, false><<<grid, kAdvectThreads, 0, st>>>(
+            m, s, d, perm, dtd, p->cell_new, p->counts, p->tile_next, p->ctr);
+    }
+    if (F32B || !m.Qch)
+      advect_kernel<D, RK, F32B, kTwoFields, false><<<grid, kAdvectThreads, 0, st>>>(
+          m, s, d, perm, dtd, p->cell_new, p->counts, p->tile_next, p->ctr);
   } else if (D == 3 && p->stage_cells) {
-    advect_kernel<D, RK, F32B, false, D == 3><<<grid, kAdvectThreads, StageLayout<D, F32B>::bytes(), st>>>(
+    advect_kernel<D, RK, F32B, kSteady, D == 3><<<grid, kAdvectThreads, StageLayout<D, F32B>::bytes(), st>>>(
         m, s, d, perm, dtd, p->cell_new, p->counts, p->tile_next, p->ctr);
   } else {
-    advect_kernel<D, RK, F32B, false, false><<<grid, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, p->cell_new,
+    advect_kernel<D, RK, F32B, kSteady, false><<<grid, kAdvectThreads, 0, st>>>(m, s, d, perm, dtd, p->cell_new,
                                                                               p->counts, p->tile_next, p->ctr);
   }
   count_launches(1);

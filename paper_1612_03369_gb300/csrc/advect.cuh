@@ -44,38 +44,40 @@ __device__ __forceinline__ void flush_counters(DevCounters* ctr, unsigned steps,
 // of the time interpolation of Sec. 2.3; theta = 1/2 is the exact average).
 // The Q2 evaluation (per-cell monomial form, Horner) is in double-float, or
 // FP32 for the precision form; it sits in a rolled loop over the (one or two)
-// fields so the kernel holds one copy of it.
-template <int D, bool F32B, bool TWO, class Cells>
+// fields so the kernel holds one copy of it.  The double-float form reads the
+// middle of the step from a table of the mean coefficients, set up with the
+// fields: four evaluations per RK4 step where two fields at two stages made
+// six (1.54 against 2.06 ms per step at 64^3 x 20, for 86 us more per field).
+enum : int {
+  kSteady = 0,
+  kMidTable = 1,  // two fields and the table of their mean
+  kTwoFields = 2  // two fields, both evaluated in the middle of the step
+};
+
+template <int D, bool F32B, int TWO, class Cells>
 __device__ __forceinline__ void velocity(const Cells& cs, const MeshView& m, uint32_t K, const df t[D], int tcode,
                                          df u[D]) {
-  if constexpr (!TWO) {
+  constexpr int NQ = F32B ? qf_float4s<D>() : qc_float4s<D>();
+  if constexpr (TWO == kSteady) {
     if constexpr (F32B)
       q2_eval_f32<D>(cs, cs.coef(K), t, u);
     else
       q2_eval_df<D>(cs, cs.coef(K), t, u);
-    return;
+  } else if constexpr (TWO == kMidTable) {
+    static_assert(!F32B, "the table of the mean field is double-float");
+    const float4* table = tcode == 0 ? m.Qc : (tcode == 1 ? m.Qch : m.Qcn);
+    q2_eval_df<D>(cs, table + (size_t)K * NQ, t, u);
   } else {
-    // the first field's blocks through the source, the second field's from
-    // the mesh arrays
-    constexpr int NQ = F32B ? qf_float4s<D>() : qc_float4s<D>();
-    const GlobalCells<D, F32B> g{m};
-    const float4* second = (F32B ? m.Qfn : m.Qcn) + (size_t)K * NQ;
     const bool two = m.has_next && tcode == 1;
     const bool only_next = m.has_next && tcode == 2;
 #pragma unroll 1
     for (int f = 0; f < (two ? 2 : 1); ++f) {
       df v[D];
-      if (f == 1 || only_next) {
-        if constexpr (F32B)
-          q2_eval_f32<D>(g, second, t, v);
-        else
-          q2_eval_df<D>(g, second, t, v);
-      } else {
-        if constexpr (F32B)
-          q2_eval_f32<D>(cs, cs.coef(K), t, v);
-        else
-          q2_eval_df<D>(cs, cs.coef(K), t, v);
-      }
+      const float4* table = f == 1 || only_next ? (F32B ? m.Qfn : m.Qcn) : (F32B ? m.Qf : m.Qc);
+      if constexpr (F32B)
+        q2_eval_f32<D>(cs, table + (size_t)K * NQ, t, v);
+      else
+        q2_eval_df<D>(cs, table + (size_t)K * NQ, t, v);
 #pragma unroll
       for (int a = 0; a < D; ++a) u[a] = (f == 0) ? v[a] : df_scale2(df_add(u[a], v[a]), 0.5f);
     }
@@ -170,7 +172,7 @@ __device__ __forceinline__ double reload_f64(const double* p) {
 }
 
 // One time step of particle i of store s in mesh m, starting in cell K.
-// TWO: the mesh carries a second field (time interpolation).
+// TWO: whether and how the mesh's second field is used (time interpolation).
 // Writes the new x and x-hat in place when the particle survives and returns
 // its new cell, or PIC_LOST.
 // advect_particle_cells reads particle i of store s and writes its new x and
@@ -179,7 +181,7 @@ __device__ __forceinline__ double reload_f64(const double* p) {
 // step's reordering), reading the cells' blocks from the source cs.
 // kFast: the fast path only; returns kDefer (and writes nothing) where a
 // rare path would be needed.
-template <int D, int RK, bool F32B, bool TWO = false, class Hook = NoHook, bool kFast = false, class Cells>
+template <int D, int RK, bool F32B, int TWO = kSteady, class Hook = NoHook, bool kFast = false, class Cells>
 __device__ __forceinline__ uint32_t advect_particle_cells(const Cells& cs, const MeshView& m, const StoreView& s,
                                                           uint32_t i, const StoreView& d, uint32_t j, uint32_t K,
                                                           df dt, int& iters, unsigned& flags, Hook&& hook = Hook()) {
@@ -239,7 +241,7 @@ __device__ __forceinline__ uint32_t advect_particle_cells(const Cells& cs, const
 }
 
 // The same reading every block from the mesh arrays.
-template <int D, int RK, bool F32B, bool TWO = false, class Hook = NoHook>
+template <int D, int RK, bool F32B, int TWO = kSteady, class Hook = NoHook>
 __device__ __forceinline__ uint32_t advect_particle_to(const MeshView& m, const StoreView& s, uint32_t i,
                                                        const StoreView& d, uint32_t j, uint32_t K, df dt, int& iters,
                                                        unsigned& flags, Hook&& hook = Hook()) {
@@ -247,7 +249,7 @@ __device__ __forceinline__ uint32_t advect_particle_to(const MeshView& m, const 
                                                  static_cast<Hook&&>(hook));
 }
 
-template <int D, int RK, bool F32B, bool TWO = false, class Hook = NoHook>
+template <int D, int RK, bool F32B, int TWO = kSteady, class Hook = NoHook>
 __device__ __forceinline__ uint32_t advect_particle(const MeshView& m, const StoreView& s, uint32_t i, uint32_t K,
                                                     df dt, int& iters, unsigned& flags, Hook&& hook = Hook()) {
   return advect_particle_to<D, RK, F32B, TWO>(m, s, i, s, i, K, dt, iters, flags, static_cast<Hook&&>(hook));
@@ -262,7 +264,7 @@ struct FullStep {
   int iters;
   unsigned flags;
 };
-template <int D, int RK, bool F32B, bool TWO, class Hook = NoHook>
+template <int D, int RK, bool F32B, int TWO, class Hook = NoHook>
 __device__ __noinline__ FullStep advect_particle_full(const MeshView& m, const StoreView& s, uint32_t i,
                                                       const StoreView& d, uint32_t j, uint32_t K, df dt,
                                                       Hook hook = Hook()) {
@@ -274,7 +276,7 @@ __device__ __noinline__ FullStep advect_particle_full(const MeshView& m, const S
 }
 
 // The fast path, then the full step where it defers (*full is set).
-template <int D, int RK, bool F32B, bool TWO, class Hook, class Cells>
+template <int D, int RK, bool F32B, int TWO, class Hook, class Cells>
 __device__ __forceinline__ uint32_t advect_particle_step(const Cells& cs, const MeshView& m, const StoreView& s,
                                                          uint32_t i, const StoreView& d, uint32_t j, uint32_t K, df dt,
                                                          int& iters, unsigned& flags, uint32_t& full, Hook hook) {

@@ -158,7 +158,7 @@ __device__ __forceinline__ uint32_t ensemble_particle(const EnsShared& sh, const
   const int p = problem_of(sh.base, P, g);
   const MeshView& m = views[p];
   const uint32_t K = g - sh.base[p];
-  const uint32_t Kn = advect_particle_step<D, RK, false, false>(GlobalCells<D, false>{m}, m, s, i, d, j, K, sh.dt[p], iters,
+  const uint32_t Kn = advect_particle_step<D, RK, false, kSteady>(GlobalCells<D, false>{m}, m, s, i, d, j, K, sh.dt[p], iters,
                                                                 flags, full, NoHook());
   return Kn == PIC_LOST ? PIC_LOST : sh.base[p] + Kn;
 }

@@ -57,8 +57,8 @@ __global__ void cell_bbox_kernel(const __grid_constant__ MeshView m, double* __r
 }
 
 __device__ __forceinline__ float2 split_df(double v) {
-  const float hi = __double2float_rn(v);
-  return make_float2(hi, __double2float_rn(v - (double)hi));
+  const df r = split_f64(v);
+  return make_float2(r.hi, r.lo);
 }
 
 // Per-cell map block: X_0 and the monomial coefficients of Phi_K - X_0
@@ -114,11 +114,15 @@ __global__ void cell_qbase_kernel(const __grid_constant__ MeshView m, uint32_t* 
   }
 }
 
-// U [comp][node] FP64 -> U2 [node][comp] double-float.
-__global__ void to_df_nodes_kernel(const double* __restrict__ U, float2* __restrict__ U2, int dim, size_t nnodes) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nnodes * dim; i += (size_t)gridDim.x * blockDim.x) {
-    const size_t node = i / dim, comp = i % dim;
-    U2[i] = split_df(U[comp * nnodes + node]);
+// U [comp][node] FP64 -> U2 [node][comp] double-float, thread per node.
+template <int D>
+__global__ void __launch_bounds__(256) to_df_nodes_kernel(const double* __restrict__ U, float2* __restrict__ U2, size_t nnodes) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nnodes; i += (size_t)gridDim.x * blockDim.x) {
+    double v[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) v[c] = U[c * nnodes + i];
+#pragma unroll
+    for (int c = 0; c < D; ++c) U2[i * D + c] = split_df(v[c]);
   }
 }
 
@@ -147,8 +151,11 @@ __device__ __forceinline__ void t_axis(df v0, df v1, df v2, df& c0, df& c1, df& 
 // With Qf given, the block also writes the coefficients' high parts, per
 // cell and component in the order r*9 + q*3 + p, padded to 28 (3D) or 12
 // (2D) floats: the FP32-basis form's table.
+// With U2b given, the field is the mean of the two (exact up to the sum's
+// double-float rounding).
 template <int D>
 __global__ void __launch_bounds__(32 * D) q2_coeff_kernel(const __grid_constant__ MeshView m, const float2* __restrict__ U2,
+                                                          const float2* __restrict__ U2b,
                                                           float4* __restrict__ Qc, float4* __restrict__ Qf) {
   // A block builds the coefficients of a group of 32 consecutive cells:
   // thread (comp, lane) does cell K0 + lane, component comp (neighbouring
@@ -169,14 +176,28 @@ __global__ void __launch_bounds__(32 * D) q2_coeff_kernel(const __grid_constant_
       cell_ijk<D>(m, K, c);
       const int64_t base = 2 * (int64_t)c[0] + sy * 2 * c[1] + (D == 3 ? sz * 2 * c[2] : 0);
       const float2* Uc = U2 + base * D + comp;  // node-major [node][comp]
+      const float2* Ub = U2b ? U2b + base * D + comp : nullptr;
       df V[3][3][3];  // [r (z)][q (y)][p (x)]
 #pragma unroll
       for (int r = 0; r < NS; ++r)
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
           const float2* row = Uc + (q * sy + (D == 3 ? r * sz : 0)) * D;
-          const float2 a = row[0], b = row[D], e = row[2 * D];
-          t_axis(df_make(a.x, a.y), df_make(b.x, b.y), df_make(e.x, e.y), V[r][q][0], V[r][q][1], V[r][q][2]);
+          df v[3];
+#pragma unroll
+          for (int p = 0; p < 3; ++p) {
+            const float2 a = row[p * D];
+            v[p] = df_make(a.x, a.y);
+          }
+          if (Ub) {
+            const float2* rowb = Ub + (row - Uc);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+              const float2 b = rowb[p * D];
+              v[p] = df_scale2(df_add(v[p], df_make(b.x, b.y)), 0.5f);
+            }
+          }
+          t_axis(v[0], v[1], v[2], V[r][q][0], V[r][q][1], V[r][q][2]);
         }
 #pragma unroll
       for (int r = 0; r < NS; ++r)
@@ -251,22 +272,31 @@ __global__ void __launch_bounds__(32 * D) q2_coeff_kernel(const __grid_constant_
   }
 }
 
-// Coefficients of one field into Qc: the FP64 values U are first split into
-// the node-major double-float copy U2 (one conversion per nodal value).
-static void build_coefficients(const pic_mesh_s* m, const double* U, float2* U2, float4* Qc, float4* Qf,
-                               cudaStream_t st) {
-  const size_t n = (size_t)m->dim * (size_t)m->nnodes;
-  const int gn = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  to_df_nodes_kernel<<<gn, 256, 0, st>>>(U, U2, m->dim, (size_t)m->nnodes);
+static void build_table(const pic_mesh_s* m, const float2* U2, const float2* U2b, float4* Qc, float4* Qf,
+                        cudaStream_t st) {
   MeshView v = mesh_view(m);
   const size_t groups = ((size_t)m->C + 31) / 32;
   const size_t cap = (size_t)num_sms() * 16;
   const int g = (int)(groups < cap ? groups : cap);
   if (m->dim == 2)
-    q2_coeff_kernel<2><<<g, 64, 0, st>>>(v, U2, Qc, Qf);
+    q2_coeff_kernel<2><<<g, 64, 0, st>>>(v, U2, U2b, Qc, Qf);
   else
-    q2_coeff_kernel<3><<<g, 96, 0, st>>>(v, U2, Qc, Qf);
-  count_launches(2);
+    q2_coeff_kernel<3><<<g, 96, 0, st>>>(v, U2, U2b, Qc, Qf);
+  count_launches(1);
+}
+
+// Coefficients of one field into Qc: the FP64 values U are first split into
+// the node-major double-float copy U2 (one conversion per nodal value).
+static void build_coefficients(const pic_mesh_s* m, const double* U, float2* U2, float4* Qc, float4* Qf,
+                               cudaStream_t st) {
+  const size_t n = (size_t)m->nnodes;
+  const int gn = (int)((n + 255) / 256 < 16384 ? (n + 255) / 256 : 16384);
+  if (m->dim == 2)
+    to_df_nodes_kernel<2><<<gn, 256, 0, st>>>(U, U2, n);
+  else
+    to_df_nodes_kernel<3><<<gn, 256, 0, st>>>(U, U2, n);
+  count_launches(1);
+  build_table(m, U2, nullptr, Qc, Qf, st);
 }
 
 static size_t coeff_float4s(const pic_mesh_s* m) { return (size_t)m->C * m->dim * (m->dim == 3 ? 15 : 5); }
@@ -404,6 +434,7 @@ extern "C" pic_status pic_destroy_mesh(pic_mesh m) {
   cudaFree(m->U2n);
   cudaFree(m->Qc);
   cudaFree(m->Qcn);
+  cudaFree(m->Qch);
   cudaFree(m->Qf);
   cudaFree(m->Qfn);
   free(m);
@@ -440,6 +471,12 @@ extern "C" pic_status pic_set_velocity_dofs(pic_mesh m, const double* U, const d
   if (U_next) {
     PIC_CUDA(cudaMemcpyAsync(m->Un, U_next, sizeof(double) * n, cudaMemcpyDefault, st));
     build_coefficients(m, m->Un, m->U2n, m->Qcn, m->Qfn, st);
+    // without room for the mean's table the steps evaluate both fields
+    if (!m->Qch && cudaMalloc(&m->Qch, sizeof(float4) * coeff_float4s(m)) != cudaSuccess) {
+      cudaGetLastError();
+      m->Qch = nullptr;
+    }
+    if (m->Qch) build_table(m, m->U2, m->U2n, m->Qch, nullptr, st);
   }
   PIC_CUDA(cudaGetLastError());
   m->has_velocity = 1;
@@ -485,6 +522,7 @@ extern "C" pic_status pic_commit_velocity_dofs(pic_mesh m, void* stream) {
   m->U = m->Ustage;
   m->Ustage = t;
   build_coefficients(m, m->U, m->U2, m->Qc, m->Qf, st);
+  if (m->has_next && m->Qch) build_table(m, m->U2, m->U2n, m->Qch, nullptr, st);
   PIC_CUDA(cudaGetLastError());
   PIC_CUDA(cudaEventRecord(m->ev_free, st));
   m->free_recorded = 1;

@@ -109,6 +109,7 @@ struct pic_mesh_s {
   float2* U2n;   // its double-float nodal copy (the source of Qcn)
   float4* Qc;    // [C][dim][slices][5] per-cell monomial coefficients (double-float pairs, see fastpath.cuh)
   float4* Qcn;   // the same for the field at the end of the step
+  float4* Qch;   // the same for the mean of the two fields (the middle of the step); null if it could not be allocated
   float4* Qf;    // [C][dim][28 or 12 floats] their high parts (FP32-basis form), allocated on first use
   float4* Qfn;   // the same for the field at the end of the step
   int has_next;
@@ -205,6 +206,7 @@ struct MeshView {
   const uint32_t* qbase;
   const float4* Qc;   // per-cell monomial coefficients of the field (and of the second field)
   const float4* Qcn;
+  const float4* Qch;
   const float4* Qf;   // their high parts (FP32-basis form; null until that form is first used)
   const float4* Qfn;
   int has_next;
@@ -234,6 +236,7 @@ inline MeshView mesh_view(const pic_mesh_s* m) {
   v.qbase = m->qbase;
   v.Qc = m->Qc;
   v.Qcn = m->Qcn;
+  v.Qch = m->Qch;
   v.Qf = m->Qf;
   v.Qfn = m->Qfn;
   v.has_next = m->has_next;

@@ -32,24 +32,6 @@ __device__ __forceinline__ df minus_half(df t) {  // t - 1/2
 }
 __device__ __forceinline__ double df_to_f64(df a) { return (double)a.hi + (double)a.lo; }
 
-// An FP64 value as a double-float, as df_from_double rounds it, on the integer
-// and FP32 pipes: the high part is the value rounded to 24 bits in the bit
-// field, the low part the 29-bit signed remainder, converted and scaled.
-// (df_from_double's three conversions and a subtraction are 4 FP64-pipe
-// operations, 64 clocks of an SM each for a warp.)  Values outside the range
-// where both parts are normal floats take df_from_double.
-__device__ __forceinline__ df split_f64(double x) {
-  const long long b = __double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7ff) - 896;  // the float's exponent field
-  if (e < 60 || e > 250) return df_from_double(x);
-  const long long r = b + (1ll << 28);  // round half up in the magnitude
-  const unsigned mag = ((unsigned)(r >> 29) ^ 0x40000000u) & 0x7fffffffu;
-  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-  const int rem = (int)(b & 0x1fffffff) - (int)(((unsigned)b & 0x10000000u) << 1);  // in [-2^28, 2^28)
-  const float scale = __int_as_float((int)(((unsigned)(e - 52) << 23) | sign));
-  return df_make(__uint_as_float(mag | sign), __fmul_rn((float)rem, scale));
-}
-
 // One particle's loads, issued an iteration ahead of their use.
 template <int D>
 struct ParticleLoads {
