@@ -24,20 +24,28 @@ struct ProductAcc {
   long long E = 0;
   bool infinite = false;
 
-  __device__ __forceinline__ void mul(double v) {  // v > 0
+  // Takes v in (0, inf]; false for anything else.  The tests are on the bits:
+  // an FP64 comparison would cost as much as the product.
+  __device__ __forceinline__ bool mul(double v) {
     int hi = __double2hiint(v);
+    const unsigned lo = (unsigned)__double2loint(v);
+    if (hi < 0 || ((unsigned)hi | lo) == 0u) return false;
+    if (hi >= 0x7ff00000) {
+      infinite = true;
+      return hi == 0x7ff00000 && lo == 0u;
+    }
     int e = hi >> 20;
     if (e == 0) {  // subnormal
       v *= 0x1p54;
       hi = __double2hiint(v);
       e = (hi >> 20) - 54;
     }
-    infinite = infinite || e == 0x7ff;
     P *= __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(v));
     const int top = __double2hiint(P);
     const int carry = (top >> 20) - 1023;  // 0 or 1
     P = __hiloint2double(top - (carry << 20), __double2loint(P));
     E += e - 1023 + carry;
+    return true;
   }
   __device__ __forceinline__ double mean(uint32_t n) const {
     if (infinite) return __longlong_as_double(0x7ff0000000000000ll);
@@ -91,10 +99,10 @@ __global__ void __launch_bounds__(256) cell_average_kernel(const uint32_t* __res
         if constexpr (KIND == 0) {
           s += v[q];
         } else {
-          bad = bad || !(v[q] > 0.0);
           if constexpr (KIND == 1) {
-            if (v[q] > 0.0) product.mul(v[q]);
+            if (!product.mul(v[q])) bad = true;
           } else {
+            bad = bad || !(v[q] > 0.0);
             s += 1.0 / v[q];
           }
         }

@@ -131,6 +131,10 @@ __device__ __forceinline__ df df_from_double(double x) {
   return df_make(hi, lo);
 }
 
+// Out of line, so that it stays behind a branch: inlined there it is predicated,
+// and its FP64 operations issue for every value.
+static __device__ __noinline__ df df_from_double_call(double x) { return df_from_double(x); }
+
 // An FP64 value as a double-float, as df_from_double rounds it, on the integer
 // and FP32 pipes: the high part is the value rounded to 24 bits in the bit
 // field, the low part the 29-bit signed remainder, converted and scaled.
@@ -140,7 +144,7 @@ __device__ __forceinline__ df df_from_double(double x) {
 __device__ __forceinline__ df split_f64(double x) {
   const long long b = __double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff) - 896;  // the float's exponent field
-  if (e < 60 || e > 250) return df_from_double(x);
+  if (e < 60 || e > 250) return df_from_double_call(x);
   const long long r = b + (1ll << 28);  // round half up in the magnitude
   const unsigned mag = ((unsigned)(r >> 29) ^ 0x40000000u) & 0x7fffffffu;
   const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;

@@ -32,6 +32,25 @@ __device__ __forceinline__ df minus_half(df t) {  // t - 1/2
 }
 __device__ __forceinline__ double df_to_f64(df a) { return (double)a.hi + (double)a.lo; }
 
+// kLanes neighbouring lanes share a cell, lane q folding its particles q, q +
+// kLanes, ..., and the lanes' compensated sums are then added in a fixed pattern
+// of exchanges.  The lanes' loads are consecutive, a 32-byte sector per cell and
+// array: with a thread per cell every load of a warp touched 32 sectors of as
+// many lines. With the property split off the FP64 pipe: vertex sums 92 -> 82 us,
+// linear fit 121 -> 107 us at 64^3 x 20 (FP32 issue 74 %; FP64 pipe 51 %).
+constexpr int kLanes = 4;
+
+// acc of every lane of the group becomes the group's sum (the same in each).
+__device__ __forceinline__ void group_sum(df_acc& acc) {
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) {
+    const float s = __shfl_xor_sync(0xffffffffu, acc.s, o), e = __shfl_xor_sync(0xffffffffu, acc.e, o);
+    const df r = two_sum(acc.s, s);
+    acc.s = r.hi;
+    acc.e = __fadd_rn(__fadd_rn(acc.e, e), r.lo);
+  }
+}
+
 // One particle's loads, issued an iteration ahead of their use.
 template <int D>
 struct ParticleLoads {
@@ -46,10 +65,23 @@ struct ParticleLoads {
   }
 };
 
+// The cell of a lane's group and its particles; a segment outside the store is
+// flagged and taken as empty.
+__device__ __forceinline__ void group_cell(const uint32_t* __restrict__ cell_off, uint32_t K, uint32_t C, size_t cap,
+                                           uint32_t& beg, uint32_t& end, bool& bad, DevCounters* __restrict__ ctr) {
+  beg = K < C ? cell_off[K] : 0u;
+  end = K < C ? cell_off[K + 1] : 0u;
+  bad = end > cap || beg > end;
+  if (bad) {
+    latch_status(ctr, PIC_STATUS_BOUNDS);
+    beg = end = 0;
+  }
+}
+
 // Two phases, both deterministic.
-// Phase 1, thread per cell: each particle of the cell is read once and its
-// 2^D corner weights (the tensor product of (1 - t_a, t_a), multiplied in
-// axis order) are folded, in store order, into the cell's partial sums
+// Phase 1, kLanes lanes per cell: each particle of the cell is read once and
+// its 2^D corner weights (the tensor product of (1 - t_a, t_a), multiplied in
+// axis order) are folded into the cell's partial sums
 //   num[c][K] = sum w_c(x-hat_i) p_i,   den[c][K] = sum w_c(x-hat_i)
 // stored as double-float pairs, corner-major ([c][C]) so that the phase-2
 // reads of a warp coalesce.
@@ -59,42 +91,47 @@ __global__ void __launch_bounds__(128) vertex_partial_kernel(const uint32_t* __r
                                                              uint32_t C, size_t cap, float2* __restrict__ part,
                                                              DevCounters* __restrict__ ctr) {
   constexpr int NC = 1 << D;
-  for (uint32_t K = blockIdx.x * blockDim.x + threadIdx.x; K < C; K += gridDim.x * blockDim.x) {
-    const uint32_t beg = cell_off[K], end = cell_off[K + 1];
+  constexpr uint32_t kCells = 128 / kLanes;  // per block and pass
+  const uint32_t q = threadIdx.x % kLanes;
+  for (uint32_t K0 = blockIdx.x * kCells; K0 < C; K0 += gridDim.x * kCells) {
+    const uint32_t K = K0 + threadIdx.x / kLanes;
+    uint32_t beg, end;
+    bool bad;
+    group_cell(cell_off, K, C, cap, beg, end, bad, ctr);
     df_acc num[NC], den[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) num[c] = den[c] = acc_zero();
-    if (end > cap || beg > end) {
-      latch_status(ctr, PIC_STATUS_BOUNDS);
-    } else {
-      ParticleLoads<D> next;
-      next.load(xh, prop, cap, beg, end);
-      for (uint32_t i = beg; i < end; ++i) {
-        const ParticleLoads<D> now = next;
-        next.load(xh, prop, cap, i + 1, end);
-        df f[D][2];  // f[a][0] = 1 - t_a, f[a][1] = t_a
+    ParticleLoads<D> next;
+    next.load(xh, prop, cap, beg + q, end);
+    for (uint32_t i = beg + q; i < end; i += kLanes) {
+      const ParticleLoads<D> now = next;
+      next.load(xh, prop, cap, i + kLanes, end);
+      df f[D][2];  // f[a][0] = 1 - t_a, f[a][1] = t_a
 #pragma unroll
-        for (int a = 0; a < D; ++a) {
-          f[a][1] = df_make(now.t[a].x, now.t[a].y);
-          f[a][0] = one_minus(f[a][1]);
-        }
-        const df p = split_f64(now.p);
-        df w01[4];  // the first two axes' products, corner bits 0 and 1
+      for (int a = 0; a < D; ++a) {
+        f[a][1] = df_make(now.t[a].x, now.t[a].y);
+        f[a][0] = one_minus(f[a][1]);
+      }
+      const df p = split_f64(now.p);
+      df w01[4];  // the first two axes' products, corner bits 0 and 1
 #pragma unroll
-        for (int c = 0; c < 4; ++c) w01[c] = df_mul(f[0][c & 1], f[1][(c >> 1) & 1]);
+      for (int c = 0; c < 4; ++c) w01[c] = df_mul(f[0][c & 1], f[1][(c >> 1) & 1]);
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const df w = D == 3 ? df_mul(w01[c & 3], f[D - 1][(c >> 2) & 1]) : w01[c];
-          acc_mad(num[c], w, p);
-          acc_add(den[c], w);
-        }
+      for (int c = 0; c < NC; ++c) {
+        const df w = D == 3 ? df_mul(w01[c & 3], f[D - 1][(c >> 2) & 1]) : w01[c];
+        acc_mad(num[c], w, p);
+        acc_add(den[c], w);
       }
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      const df a = acc_result(num[c]), b = acc_result(den[c]);
-      part[(size_t)c * C + K] = make_float2(a.hi, a.lo);
-      part[(size_t)(NC + c) * C + K] = make_float2(b.hi, b.lo);
+      group_sum(num[c]);
+      group_sum(den[c]);
+      if (K < C && (uint32_t)c % kLanes == q) {
+        const df a = acc_result(num[c]), b = acc_result(den[c]);
+        part[(size_t)c * C + K] = make_float2(a.hi, a.lo);
+        part[(size_t)(NC + c) * C + K] = make_float2(b.hi, b.lo);
+      }
     }
   }
 }
@@ -139,10 +176,13 @@ __global__ void __launch_bounds__(256) vertex_gather_kernel(const __grid_constan
   }
 }
 
-// Thread per cell: normal equations (A^T A) c = A^T p of the cell's design
-// matrix, rows (1, x-hat_i - 1/2), folded in store order; Gaussian
-// elimination with partial pivoting; the mean where the cell has at most D
-// particles or a pivot is <= 1e-12 of the largest diagonal entry.
+// The normal equations (A^T A) c = A^T p of the cell's design matrix, rows
+// (1, x-hat_i - 1/2), kLanes lanes per cell; Gaussian elimination with partial
+// pivoting; the mean where the cell has at most D particles or a pivot is <=
+// 1e-12 of the largest diagonal entry.  The sums are left in shared memory and
+// solved by one warp of the block, a cell per lane (an FP64 warp instruction
+// takes the FP64 pipe as long for 8 lanes as for 32), the block's warps in turn
+// while the others go on to the next cells.
 template <int D>
 __global__ void __launch_bounds__(128) lsq_linear_kernel(const uint32_t* __restrict__ cell_off,
                                                          const float2* __restrict__ xh, const double* __restrict__ prop,
@@ -150,57 +190,80 @@ __global__ void __launch_bounds__(128) lsq_linear_kernel(const uint32_t* __restr
                                                          double* __restrict__ coef, uint32_t* __restrict__ count,
                                                          DevCounters* __restrict__ ctr) {
   constexpr int NB = D + 1;
-  for (uint32_t K = blockIdx.x * blockDim.x + threadIdx.x; K < C; K += gridDim.x * blockDim.x) {
-    const uint32_t beg = cell_off[K], end = cell_off[K + 1];
-    if (end > cap || beg > end) {
-      latch_status(ctr, PIC_STATUS_BOUNDS);
-      continue;
-    }
-    // the upper triangle of A^T A, A^T p and sum p, accumulated in
-    // double-float (row a = (1, x-hat - 1/2)), then converted once
-    df_acc Ma[NB][NB + 1];
+  constexpr int NE = NB * (NB + 3) / 2 - 1;  // upper triangle of A^T A but the count, and A^T p
+  constexpr uint32_t kCells = 128 / kLanes;
+  static_assert(kCells == 32, "one cell per lane of the solving warp");
+  __shared__ float2 s_sum[2][NE][kCells];
+  __shared__ uint32_t s_n[2][kCells];
+  const uint32_t q = threadIdx.x % kLanes, g = threadIdx.x / kLanes, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  uint32_t pass = 0;
+  for (uint32_t K0 = blockIdx.x * kCells; K0 < C; K0 += gridDim.x * kCells, ++pass) {
+    const uint32_t buf = pass & 1u;
+    {
+      uint32_t beg, end;
+      bool bad;
+      group_cell(cell_off, K0 + g, C, cap, beg, end, bad, ctr);
+      // accumulated in double-float (row a = (1, x-hat - 1/2))
+      df_acc acc[NE];
 #pragma unroll
-    for (int r = 0; r < NB; ++r)
+      for (int e = 0; e < NE; ++e) acc[e] = acc_zero();
+      ParticleLoads<D> next;
+      next.load(xh, prop, cap, beg + q, end);
+      for (uint32_t i = beg + q; i < end; i += kLanes) {
+        const ParticleLoads<D> now = next;
+        next.load(xh, prop, cap, i + kLanes, end);
+        df a[NB];
 #pragma unroll
-      for (int q = 0; q <= NB; ++q) Ma[r][q] = acc_zero();
-    ParticleLoads<D> next;
-    next.load(xh, prop, cap, beg, end);
-    for (uint32_t i = beg; i < end; ++i) {
-      const ParticleLoads<D> now = next;
-      next.load(xh, prop, cap, i + 1, end);
-      df a[NB];
-      a[0] = df_make(1.0f, 0.f);
+        for (int j = 0; j < D; ++j) a[j + 1] = minus_half(df_make(now.t[j].x, now.t[j].y));
+        const df p = split_f64(now.p);
+        int e = 0;
 #pragma unroll
-      for (int j = 0; j < D; ++j) a[j + 1] = minus_half(df_make(now.t[j].x, now.t[j].y));
-      const df p = split_f64(now.p);
+        for (int r = 0; r < NB; ++r) {
 #pragma unroll
-      for (int r = 0; r < NB; ++r) {
-#pragma unroll
-        for (int q = r; q < NB; ++q) {
-          if (r == 0 && q == 0) continue;  // the count
-          if (r == 0)
-            acc_add(Ma[r][q], a[q]);  // a[0] = 1
-          else
-            acc_mad(Ma[r][q], a[r], a[q]);
+          for (int k = r; k <= NB; ++k) {
+            if (r == 0 && k == 0) continue;  // the count
+            const df b = k == NB ? p : a[k];
+            if (r == 0)
+              acc_add(acc[e++], b);
+            else
+              acc_mad(acc[e++], a[r], b);
+          }
         }
-        if (r == 0)
-          acc_add(Ma[r][NB], p);
-        else
-          acc_mad(Ma[r][NB], a[r], p);
       }
+#pragma unroll
+      for (int e = 0; e < NE; ++e) {
+        group_sum(acc[e]);
+        if ((uint32_t)e % kLanes == q) {
+          const df r = acc_result(acc[e]);
+          s_sum[buf][e][g] = make_float2(r.hi, r.lo);
+        }
+      }
+      if (q == 0) s_n[buf][g] = bad ? PIC_LOST : end - beg;
     }
+    // one barrier a pass: the buffer is written again two passes on, after the
+    // barrier that its solving warp passes when it is done
+    __syncthreads();
+    if (warp != (pass & 3u)) continue;
+    const uint32_t K = K0 + lane, n = s_n[buf][lane];
+    if (K >= C || n == PIC_LOST) continue;
     double M[NB][NB + 1];
+    int e = 0;
 #pragma unroll
     for (int r = 0; r < NB; ++r)
 #pragma unroll
-      for (int q = r; q <= NB; ++q) M[r][q] = df_to_f64(acc_result(Ma[r][q]));
-    M[0][0] = (double)(end - beg);
+      for (int k = r; k <= NB; ++k) {
+        if (r == 0 && k == 0) {
+          M[0][0] = (double)n;
+          continue;
+        }
+        const float2 v = s_sum[buf][e++][lane];
+        M[r][k] = (double)v.x + (double)v.y;
+      }
     const double sum = M[0][NB];
 #pragma unroll
     for (int r = 1; r < NB; ++r)
 #pragma unroll
-      for (int q = 0; q < r; ++q) M[r][q] = M[q][r];
-    const uint32_t n = end - beg;
+      for (int k = 0; k < r; ++k) M[r][k] = M[k][r];
     double c[NB];
 #pragma unroll
     for (int r = 0; r < NB; ++r) c[r] = 0.0;
@@ -298,7 +361,7 @@ extern "C" pic_status pic_interpolate_to_vertices(pic_particles p, pic_mesh mesh
     }
   }
   const double* pv = p->props[p->cur] + (size_t)prop * p->capacity;
-  const int g1 = transfer_grid(p->C, 128), g2 = transfer_grid((size_t)m.nverts, 256);
+  const int g1 = transfer_grid((size_t)p->C * kLanes, 128), g2 = transfer_grid((size_t)m.nverts, 256);
   float2* part = reinterpret_cast<float2*>(p->xfer);  // [2 * 2^dim][C] double-float pairs
   if (mesh->dim == 2) {
     vertex_partial_kernel<2><<<g1, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, part, p->ctr);
@@ -324,7 +387,7 @@ extern "C" pic_status pic_project_linear(pic_particles p, pic_mesh mesh, int pro
     if (r0 != PIC_OK) return r0;
   }
   const double* pv = p->props[p->cur] + (size_t)prop * p->capacity;
-  const int g = transfer_grid(p->C, 128);
+  const int g = transfer_grid((size_t)p->C * kLanes, 128);
   if (mesh->dim == 2)
     lsq_linear_kernel<2><<<g, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, empty_fill, coef,
                                             count, p->ctr);
