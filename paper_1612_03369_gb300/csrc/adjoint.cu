@@ -249,14 +249,16 @@ __global__ void __launch_bounds__(128, PIC_ADVECT_MIN_BLOCKS) replay_step_kernel
   }
 }
 
-// Warp per cell: the records of the cell, in (cell, stage, slot) order, summed into
-// the cell's 3^D x D block of nodal gradient entries (lane e owns entries e,
-// e+32, ...), in double-float on the FP32 pipe; every cell is written (FP64),
-// empty ones with zeros.  The entry (node (a, b, c), comp) of a record is
-// (w_comp l_a(t0)) (l_b(t1) l_c(t2)): records are taken 32 at a time, lane i
-// forms record i's D x 3 left factors and 3^(D-1) right factors once and
-// leaves them in shared memory, then every lane adds its entries' products
-// over those records in record order.
+// Warp per cell: the records of the cell, in (cell, stage, slot) order, summed
+// into the cell's 3^D x D block of nodal gradient entries, in double-float on
+// the FP32 pipe; every cell is written (FP64), empty ones with zeros.  The entry
+// (node (a, b, c), comp) of a record is (w_comp l_a(t0)) (l_b(t1) l_c(t2)):
+// records are taken 32 at a time, lane i forms record i's D x 3 left factors and
+// 3^(D-1) right factors once and leaves them in shared memory, then every lane
+// adds its entries' products over those records in record order.  Lane (left
+// factor, c) owns the entries of that left factor with the three right factors
+// of c (2D: of one right factor): 27 lanes (18) and four loads a record, where
+// entries dealt out evenly took six.
 template <int D>
 __global__ void __launch_bounds__(256) cell_partial_kernel(uint32_t C, const uint32_t* __restrict__ rec_off,
                                                            const uint32_t* __restrict__ rec_perm,
@@ -265,20 +267,14 @@ __global__ void __launch_bounds__(256) cell_partial_kernel(uint32_t C, const uin
                                                            double* __restrict__ partial) {
   constexpr int NN = (D == 3 ? 27 : 9);
   constexpr int NE = NN * D;
-  constexpr int PER = (NE + 31) / 32;
   constexpr int NA = 3 * D;             // w_comp l_a(t0), index comp * 3 + a
   constexpr int NB = (D == 3 ? 9 : 3);  // l_b(t1) l_c(t2), index c * 3 + b (2D: l_b(t1))
+  constexpr int PER = D == 3 ? 3 : 1;   // right factors per lane
   __shared__ float2 fac[256 / 32][32][NA + NB];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  int ia[PER], ib[PER];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int ent = lane + 32 * q;
-    const int node = ent / D, comp = ent % D;
-    ia[q] = comp * 3 + node % 3;
-    ib[q] = NA + (D == 3 ? (node / 9) * 3 + (node / 3) % 3 : (node / 3) % 3);
-  }
+  const bool mine = lane < 3 * NA;
+  const int left = lane % NA, group = mine ? lane / NA : 0;
   for (uint32_t K = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; K < C; K += warps) {
     df_acc acc[PER];
 #pragma unroll
@@ -312,23 +308,25 @@ __global__ void __launch_bounds__(256) cell_partial_kernel(uint32_t C, const uin
       }
       __syncwarp();
       const int cnt = (end - e0) < 32u ? (int)(end - e0) : 32;
-      for (int j = 0; j < cnt; ++j) {
+      if (mine) {
+#pragma unroll 2
+        for (int j = 0; j < cnt; ++j) {
+          const float2 A = fac[wib][j][left];
 #pragma unroll
-        for (int q = 0; q < PER; ++q) {
-          if (lane + 32 * q < NE) {
-            const float2 A = fac[wib][j][ia[q]], B = fac[wib][j][ib[q]];
+          for (int q = 0; q < PER; ++q) {
+            const float2 B = fac[wib][j][NA + group * PER + q];
             acc_mad(acc[q], df_make(A.x, A.y), df_make(B.x, B.y));
           }
         }
       }
       __syncwarp();
     }
+    if (mine) {
+      const int comp = left / 3, a = left % 3;
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      const int ent = lane + 32 * q;
-      if (ent < NE) {
-        const df v = acc_result(acc[q]);
-        partial[(size_t)K * NE + ent] = df_to_double(v);
+      for (int q = 0; q < PER; ++q) {
+        const int node = a + 3 * (group * PER + q);
+        partial[(size_t)K * NE + node * D + comp] = df_to_double(acc_result(acc[q]));
       }
     }
   }
