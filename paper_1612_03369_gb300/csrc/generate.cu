@@ -29,6 +29,7 @@
 #include <cstdlib>
 
 #include "fastpath.cuh"
+#include "grad_df.cuh"
 #include "pic_internal.cuh"
 #include "seed.cuh"
 
@@ -53,6 +54,20 @@ __device__ __forceinline__ double vweight_rn(int v, const double t[D], int skip 
 }
 
 template <int D>
+__device__ __forceinline__ double det_rn(const double J[D][D]) {
+  double det;
+  if constexpr (D == 2) {
+    det = __dsub_rn(__dmul_rn(J[0][0], J[1][1]), __dmul_rn(J[0][1], J[1][0]));
+  } else {
+    const double c0 = __dsub_rn(__dmul_rn(J[1][1], J[2][2]), __dmul_rn(J[1][2], J[2][1]));
+    const double c1 = __dsub_rn(__dmul_rn(J[1][2], J[2][0]), __dmul_rn(J[1][0], J[2][2]));
+    const double c2 = __dsub_rn(__dmul_rn(J[1][0], J[2][1]), __dmul_rn(J[1][1], J[2][0]));
+    det = __dadd_rn(__dadd_rn(__dmul_rn(J[0][0], c0), __dmul_rn(J[0][1], c1)), __dmul_rn(J[0][2], c2));
+  }
+  return det;
+}
+
+template <int D>
 __device__ double rho_hat_rn(const MeshView& m, uint32_t K, const double* __restrict__ rho, const double t[D]) {
   int c[3];
   cell_ijk<D>(m, K, c);
@@ -70,16 +85,7 @@ __device__ double rho_hat_rn(const MeshView& m, uint32_t K, const double* __rest
         s = __dadd_rn(s, __dmul_rn(__ldg(m.X + i * m.nverts + local_vertex<D>(m, c, v)), vweight_rn<D>(v, t, j)));
       J[i][j] = s;
     }
-  double det;
-  if constexpr (D == 2) {
-    det = __dsub_rn(__dmul_rn(J[0][0], J[1][1]), __dmul_rn(J[0][1], J[1][0]));
-  } else {
-    const double c0 = __dsub_rn(__dmul_rn(J[1][1], J[2][2]), __dmul_rn(J[1][2], J[2][1]));
-    const double c1 = __dsub_rn(__dmul_rn(J[1][2], J[2][0]), __dmul_rn(J[1][0], J[2][2]));
-    const double c2 = __dsub_rn(__dmul_rn(J[1][0], J[2][1]), __dmul_rn(J[1][1], J[2][0]));
-    det = __dadd_rn(__dadd_rn(__dmul_rn(J[0][0], c0), __dmul_rn(J[0][1], c1)), __dmul_rn(J[0][2], c2));
-  }
-  return __dmul_rn(r, fabs(det));
+  return __dmul_rn(r, fabs(det_rn<D>(J)));
 }
 
 // x = Phi_K(t) = sum_v X_v w_v(t), in the same rounded sequence.
@@ -101,22 +107,54 @@ __device__ __forceinline__ double unit53(uint64_t r) { return (double)(r >> 11) 
 
 // ------------------------------------------------------------ cell weights
 
+// The Gauss points are the same in every cell, and so are the weights w_v and
+// dw_v/dt_j there: each block forms them once, by the sequence's own operations,
+// and a cell only takes the products with its vertices (the full sequence per
+// cell, 1815 FP64 operations: 0.40 ms for 110,592 cells, FP64-pipe bound).
 template <int D>
 __global__ void __launch_bounds__(128) cell_weights_kernel(const __grid_constant__ MeshView m, const double* __restrict__ rho,
                                                            double* __restrict__ w) {
-  const double g0 = __dsub_rn(0.5, __ddiv_rn(0.5, __dsqrt_rn(3.0)));
-  const double g1 = __dadd_rn(0.5, __ddiv_rn(0.5, __dsqrt_rn(3.0)));
+  constexpr int NV = 1 << D;
+  __shared__ double s_w[NV][D + 1][NV];  // [point][j; D: the weight itself][vertex]
+  for (int e = threadIdx.x; e < NV * (D + 1) * NV; e += blockDim.x) {
+    const double g0 = __dsub_rn(0.5, __ddiv_rn(0.5, __dsqrt_rn(3.0)));
+    const double g1 = __dadd_rn(0.5, __ddiv_rn(0.5, __dsqrt_rn(3.0)));
+    const int v = e % NV, j = (e / NV) % (D + 1), q = e / (NV * (D + 1));
+    double t[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) t[a] = ((q >> a) & 1) ? g1 : g0;
+    s_w[q][j][v] = vweight_rn<D>(v, t, j == D ? -1 : j);
+  }
+  __syncthreads();
   for (uint32_t K = blockIdx.x * blockDim.x + threadIdx.x; K < m.C; K += gridDim.x * blockDim.x) {
+    int c[3];
+    cell_ijk<D>(m, K, c);
+    double X[D][NV], r[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int64_t lv = local_vertex<D>(m, c, v);
+      r[v] = __ldg(rho + lv);
+#pragma unroll
+      for (int i = 0; i < D; ++i) X[i][v] = __ldg(m.X + i * m.nverts + lv);
+    }
     double s = 0.0;
 #pragma unroll 1
-    for (int q = 0; q < (1 << D); ++q) {
-      double t[D];
+    for (int q = 0; q < NV; ++q) {
+      double rh = 0.0, J[D][D], wq = 1.0;
 #pragma unroll
-      for (int a = 0; a < D; ++a) t[a] = ((q >> a) & 1) ? g1 : g0;
-      double wq = 1.0;
+      for (int v = 0; v < NV; ++v) rh = __dadd_rn(rh, __dmul_rn(r[v], s_w[q][D][v]));
+#pragma unroll
+      for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          double e = 0.0;
+#pragma unroll
+          for (int v = 0; v < NV; ++v) e = __dadd_rn(e, __dmul_rn(X[i][v], s_w[q][j][v]));
+          J[i][j] = e;
+        }
 #pragma unroll
       for (int a = 0; a < D; ++a) wq = __dmul_rn(wq, 0.5);
-      s = __dadd_rn(s, __dmul_rn(wq, rho_hat_rn<D>(m, K, rho, t)));
+      s = __dadd_rn(s, __dmul_rn(wq, __dmul_rn(rh, fabs(det_rn<D>(J)))));
     }
     w[K] = s;
   }
@@ -142,7 +180,7 @@ struct DrawInfo {
 // once.  The first sum to reach the next power of two ends the run: it is
 // formed by one rounded addition, and the scan goes on behind it with the new
 // spacing (about log2(C) such breaks).  One warp folding value by value, each
-// addition waiting for the last, took 6.0 ms for 110,592 cells; this 0.33.
+// addition waiting for the last, took 6.0 ms for 110,592 cells; this 0.24.
 struct FoldInc {
   unsigned long long d[2];  // increment of n when n is even / odd, at most kFoldCap
 };
@@ -225,7 +263,30 @@ __global__ void __launch_bounds__(kFoldThreads) accumulate_weights_kernel(const 
     s_last = 0;
   }
   __syncthreads();
-  for (uint64_t base = 0; base < C;) {
+  // the first sums double within a few values, each a break of the scan: one
+  // warp folds them value by value (256 values: 0.01 ms for eight breaks)
+  constexpr uint32_t kPrologue = 256;
+  const uint32_t pro = C < kPrologue ? C : kPrologue;
+  if (warp == 0) {
+    double sum = 0.0;
+    for (uint32_t k0 = 0; k0 < pro; k0 += 32) {
+      const uint32_t k = k0 + lane;
+      double v = k < pro ? w[k] : 0.0, mine = 0.0;
+      if (!(v >= 0.0) || !isfinite(v)) {
+        s_bad = 1;
+        v = 0.0;
+      }
+      if (v > 0.0) atomicMax(&s_last, k + 1u);
+      for (int q = 0; q < 32; ++q) {
+        sum = __dadd_rn(sum, __shfl_sync(0xffffffffu, v, q));
+        if ((int)lane == q) mine = sum;
+      }
+      if (k < pro) acc[k] = mine;
+    }
+    if (lane == 0) s_sum = (unsigned long long)__double_as_longlong(sum);
+  }
+  __syncthreads();
+  for (uint64_t base = pro; base < C;) {
     const unsigned long long sum = s_sum;
     unsigned long long n0;
     int exp;
@@ -237,20 +298,26 @@ __global__ void __launch_bounds__(kFoldThreads) accumulate_weights_kernel(const 
     FoldInc inc[kFoldItems], mine;
     uint32_t pos = 0xffffffffu;  // this thread's first positive weight
     mine.d[0] = mine.d[1] = 0;
+    uint32_t last = 0;
 #pragma unroll
     for (int q = 0; q < kFoldItems; ++q) {
       const uint64_t k = base + (uint64_t)tid * kFoldItems + q;
-      const double v = k < C ? w[k] : 0.0;
-      const bool good = v >= 0.0 && isfinite(v);
+      // on the bits (an FP64 comparison holds the SM's FP64 pipe 16 clocks a
+      // warp): -0 counts as 0
+      const unsigned long long b = k < C ? (unsigned long long)__double_as_longlong(w[k]) : 0ull;
+      const bool minus_zero = b == 1ull << 63;
+      const bool good = (b >> 52) < 0x7ffu || minus_zero;
       if (!good) s_bad = 1;
-      wb[q] = good && v > 0.0 ? (unsigned long long)__double_as_longlong(v) : 0ull;
+      wb[q] = good && !minus_zero ? b : 0ull;
       if (wb[q]) {
         if (pos == 0xffffffffu) pos = tid * kFoldItems + q;
-        atomicMax(&s_last, (uint32_t)k + 1u);
+        last = (uint32_t)k + 1u;
       }
       inc[q] = fold_inc(wb[q], exp);
       mine = fold_compose(mine, inc[q]);
     }
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0 && last) atomicMax(&s_last, last);
     // exclusive composition over the threads before this one
     FoldInc inc_warp = mine;
 #pragma unroll
@@ -350,17 +417,68 @@ __device__ __forceinline__ void raw_coordinates(RawPoint<D> p, double t[D]) {
   for (int a = 0; a < D; ++a) t[a] = unit53(p.r[a]);
 }
 
-// The acceptance test as defined: u rho-hat(current) < rho-hat(proposal) in
-// the written sequence of IEEE operations.
+// rho-hat in double-float.
+template <int D>
+__device__ df rho_hat_df(const MeshView& m, uint32_t K, const double* __restrict__ rho, const df t[D]) {
+  int c[3];
+  cell_ijk<D>(m, K, c);
+  df_acc r = acc_zero();
+  df w[1 << D];
+  w[0] = df_make(1.0f, 0.f);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const df u = df_sub(df_make(1.0f, 0.f), t[a]);
+#pragma unroll
+    for (int v = 0; v < (1 << a); ++v) {
+      w[v + (1 << a)] = df_mul(w[v], t[a]);
+      w[v] = df_mul(w[v], u);
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < (1 << D); ++v) acc_mad(r, w[v], df_from_double(__ldg(rho + local_vertex<D>(m, c, v))));
+  df J[D][D], det;
+  map_jacobian_df<D>(LdgLoader(), m.blk + (size_t)K * block_float4s<D>(), t, J);
+  if constexpr (D == 2) {
+    det = df_det2(J[0][0], J[1][1], J[0][1], J[1][0]);
+  } else {
+    df_acc s = acc_zero();
+    acc_mad(s, J[0][0], df_det2(J[1][1], J[2][2], J[1][2], J[2][1]));
+    acc_mad(s, J[0][1], df_det2(J[1][2], J[2][0], J[1][0], J[2][2]));
+    acc_mad(s, J[0][2], df_det2(J[1][0], J[2][1], J[1][1], J[2][0]));
+    det = acc_result(s);
+  }
+  const df p = df_mul(acc_result(r), det);
+  return det.hi < 0.f ? df_make(-p.hi, -p.lo) : p;
+}
+
+// The acceptance test that FP32 values left open: by double-float ones where
+// they differ by more than their own bound (tau is FP32's, 2^-20 of it theirs:
+// they keep ~2^-46 where FP32 keeps 2^-24), and by the definition otherwise,
+// u rho-hat(current) < rho-hat(proposal) in the written sequence of IEEE
+// operations (two evaluations are 2000 FP64 operations, 33 k clocks of an SM's
+// FP64 pipe, and came 1.6 times per warp with FP32 alone before them).
 template <int D>
 __device__ __noinline__ bool mh_accept_rn(const MeshView& m, uint32_t K, const double* __restrict__ rho, RawPoint<D> cur,
-                                          RawPoint<D> prop, bool at_centre, double u) {
+                                          RawPoint<D> prop, bool at_centre, double u, float tau) {
   double t[D], y[D];
   raw_coordinates<D>(cur, t);
   if (at_centre)
 #pragma unroll
     for (int a = 0; a < D; ++a) t[a] = 0.5;
   raw_coordinates<D>(prop, y);
+  if (tau > 0x1p-90f && tau < 0x1p90f) {  // no double-float term below the normal floats
+    df td[D], yd[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      td[a] = df_from_double(t[a]);
+      yd[a] = df_from_double(y[a]);
+    }
+    const df lhs = df_mul(df_from_double(u), rho_hat_df<D>(m, K, rho, td));
+    const df diff = df_sub(rho_hat_df<D>(m, K, rho, yd), lhs);
+    const float sure = 0x1p-18f * tau;  // four times the bound
+    if (diff.hi > sure) return true;
+    if (diff.hi < -sure) return false;
+  }
   const double rc = rho_hat_rn<D>(m, K, rho, t), ry = rho_hat_rn<D>(m, K, rho, y);
   return __dmul_rn(u, rc) < ry;
 }
@@ -421,16 +539,20 @@ struct RhoHat32 {
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       row[a] = load_row<D>(cs, B, 0, a);
-      float r = 0.f;  // bounds every entry of the row
+      // bounds every entry of the row: its largest linear coefficient and the
+      // mixed ones
+      float r = 0.f, mixed = 0.f;
 #pragma unroll
-      for (int k = 0; k < (1 << D) - 1; ++k) r += fabsf(row[a].a[k]);
-      S *= r;
+      for (int k = 0; k < D; ++k) r = fmaxf(r, fabsf(row[a].a[k]));
+#pragma unroll
+      for (int k = D; k < (1 << D) - 1; ++k) mixed += fabsf(row[a].a[k]);
+      S *= r + mixed;
     }
     // With s_i the bound of row i and e = 2^-24: every entry of J is off by at
     // most 7 e s_i (coefficient, coordinate and FMA roundings), the determinant,
     // a sum of D! products, by 26 e D! s_0..s_(D-1), rho_h by 11 e R; the product
-    // by less than 256 e R S.  Doubled.
-    tau = 0x1p-15f * R * S;
+    // by less than 256 e R S.
+    tau = 0x1p-16f * R * S;
   }
 
   __device__ __forceinline__ float at(const float t[D]) const {
@@ -460,8 +582,8 @@ struct RhoHat32 {
 //
 // A step only needs the sign of u rho-hat(current) - rho-hat(proposal).  It is
 // taken from FP32 values where they differ by more than their error bound, and
-// from the written IEEE sequence otherwise (about one step in 10^4), so the
-// decisions are those of the sequence.  Evaluating the sequence at every
+// in double-float or by the written IEEE sequence otherwise (mh_accept_rn), so
+// the decisions are those of the sequence.  Evaluating the sequence at every
 // proposal, 239 FP64 operations, held the FP64 pipe 83 % busy: 12.8 ms for
 // 1.77 M particles at J = 8.
 template <int D>
@@ -499,7 +621,7 @@ __global__ void __launch_bounds__(128, 5) mh_seed_kernel(const __grid_constant__
       const float ry = f.at(t32);
       const float diff = ry - (float)(uint32_t)(ur >> 40) * 0x1p-24f * rc;
       bool accept = diff > sure;
-      if (!(fabsf(diff) > sure)) accept = mh_accept_rn<D>(m, K, rho, cur, y, at_centre, unit53(ur));
+      if (!(fabsf(diff) > sure)) accept = mh_accept_rn<D>(m, K, rho, cur, y, at_centre, unit53(ur), f.tau);
       if (accept) {
         cur = y;
         rc = ry;
