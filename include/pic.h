@@ -203,10 +203,10 @@ pic_status pic_set_properties(pic_particles parts, int prop, const double *value
  * The particle data move to their sorted slots inside the next step's
  * advect.  After the last step of a call the new order is computed but left
  * pending: the next pic_advect applies it inside its first advect, and
- * pic_interpolate_to_cells reads through it; every other call on the store
- * applies it first (one gather on that call's stream).  Every call thus sees
- * the store sorted by (cell, id); pic_get_state and pic_cell_offsets already
- * describe the new order.
+ * pic_interpolate_to_cells and pic_export into device arrays read through it;
+ * every other call on the store applies it first (one gather on that call's
+ * stream).  Every call thus sees the store sorted by (cell, id); pic_get_state
+ * and pic_cell_offsets already describe the new order.
  * Integrators (classical forms, reading of the garbled printed formulas):
  *   PIC_EULER x + dt u(x);  PIC_RK2 midpoint x + dt u(x + dt/2 u(x));
  *   PIC_RK4 x + (k1 + 2 k2 + 2 k3 + k4)/6, k1 = dt u(x), k2 = dt u(x + k1/2),
@@ -450,7 +450,7 @@ pic_status pic_interpolate_to_vertices(pic_particles parts, pic_mesh mesh, int p
  * least-squares fit in reference coordinates,
  *   f(x-hat) = c_0 + sum_j c_{j+1} (x-hat_j - 1/2)
  * minimising sum over the cell's particles of (f(x-hat_i) - p_i)^2.  Solved
- * from the normal equations (folded in store order) by Gaussian elimination
+ * from the normal equations (folded in a fixed order) by Gaussian elimination
  * with partial pivoting.  A cell with at most dim particles, or a pivot
  * <= 1e-12 times the largest diagonal entry, gets the mean (c_0 = mean,
  * slopes 0); an empty cell gets c_0 = empty_fill.

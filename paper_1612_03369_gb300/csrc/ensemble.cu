@@ -839,7 +839,7 @@ extern "C" pic_status pic_ensemble_export(pic_ensemble e, int problem, double* x
   if (n == 0 || (!x && !xhat && !id && !cell)) return PIC_OK;
   const int c = s->cur;
   // device arrays in one kernel; x and id may also be host arrays, copied
-  const bool hx = x && !on_device(x), hid = id && !on_device(id);
+  const bool hx = x && !on_device(x, sizeof(double)), hid = id && !on_device(id, sizeof(uint64_t));
   for (int a = 0; a < e->dim && hx; ++a)
     PIC_CUDA(cudaMemcpyAsync(x + a * n, s->x[c] + a * cap + beg, sizeof(double) * n, cudaMemcpyDefault, st));
   if (hid) PIC_CUDA(cudaMemcpyAsync(id, s->id[c] + beg, sizeof(uint64_t) * n, cudaMemcpyDefault, st));

@@ -73,8 +73,10 @@ void launch_pack(pic_particles_s* p, int buf, const uint32_t* perm, size_t first
   count_launches(1);
 }
 
-// Device memory of the current device.
-bool on_device(const void* ptr) {
+// Device memory of the current device that a kernel may write as elements of
+// `align` bytes (a copy takes any address).
+bool on_device(const void* ptr, size_t align) {
+  if ((uintptr_t)ptr % align) return false;
   cudaPointerAttributes at;
   int here = 0;
   const bool dev = cudaGetDevice(&here) == cudaSuccess && cudaPointerGetAttributes(&at, ptr) == cudaSuccess &&
@@ -332,9 +334,9 @@ extern "C" pic_status pic_export(pic_particles p, double* x, double* xhat, uint6
   cudaStream_t st = (cudaStream_t)stream;
   // into device arrays: one kernel, through a pending order; with any host
   // array: the order applied, then a copy per array
-  const void* dst[5] = {x, xhat, id, cell, props};
-  bool packed = true;
-  for (const void* q : dst) packed = packed && (!q || on_device(q));
+  const bool packed = (!x || on_device(x, sizeof(double))) && (!xhat || on_device(xhat, sizeof(double))) &&
+                      (!id || on_device(id, sizeof(uint64_t))) && (!cell || on_device(cell, sizeof(uint32_t))) &&
+                      (!props || on_device(props, sizeof(double)));
   if (!packed) {
     const pic_status r0 = settle_order(p, st);
     if (r0 != PIC_OK) return r0;
@@ -354,7 +356,7 @@ extern "C" pic_status pic_export(pic_particles p, double* x, double* xhat, uint6
     if (x) PIC_CUDA(cudaMemcpyAsync(x + a * N, p->x[c] + a * cap, sizeof(double) * N, cudaMemcpyDefault, st));
   }
   if (xhat) {
-    const bool dev = on_device(xhat);
+    const bool dev = on_device(xhat, sizeof(double));
     double* tmp = xhat;
     if (!dev) PIC_CUDA(cudaMallocAsync((void**)&tmp, sizeof(double) * p->dim * N, st));
     xhat_to_double_kernel<<<1024, 256, 0, st>>>(p->xhat[c], tmp, cap, N, p->dim);

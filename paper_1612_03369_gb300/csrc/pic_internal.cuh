@@ -435,7 +435,7 @@ __device__ __forceinline__ bool in_ref_cell(const double t[D]) {
 
 namespace pic {
 // ---------------------------------------------- host-side internal calls --
-bool on_device(const void* ptr);
+bool on_device(const void* ptr, size_t align);
 // Particles [first, first + n) of buffer `buf` (slot first + j is particle
 // perm[j] when perm is given), packed into device arrays of n (any may be
 // null), cells less cell_base.  Defined in particles.cu.
@@ -472,7 +472,8 @@ pic_status launch_advect_record(pic_particles_s* p, const MeshView& m, double dt
                                 cudaStream_t st);
 pic_status rebin_apply_order(pic_particles_s* p, cudaStream_t s);
 // pic_advect leaves its last rebin's order pending (the next pic_advect
-// applies it inside its advect, pic_interpolate_to_cells reads through it);
+// applies it inside its advect, pic_interpolate_to_cells and pic_export into
+// device arrays read through it);
 // every other call that reads or writes the particle arrays in slot order
 // applies it first with this (a gather on stream s; nothing when none is
 // pending).  Defined in rebin.cu.

@@ -132,6 +132,26 @@ def test_export_destinations_agree(P, settled):
         assert torch.equal(a[k], b[k]), k
 
 
+@pytest.mark.parametrize("field", ["x", "xhat", "id", "cell", "props"])
+def test_export_to_an_address_no_kernel_can_write(P, field):
+    """A device array off its element's alignment takes the copies, bit for bit."""
+    import torch
+
+    wl = W.curl_cube(4, 7, 2, 3)
+    mesh, parts = H.gpu_seed(wl)
+    parts.advect(wl.dt, 4, 1)
+    ref = parts.export()
+    out = {k: torch.zeros_like(v) for k, v in ref.items()}
+    size = ref[field].numel() * ref[field].element_size()
+    raw = torch.zeros(size + 16, dtype=torch.uint8, device="cuda")
+    shifted = raw[2:2 + size]
+    P.pic_export(parts.h, **{**out, field: shifted})
+    torch.cuda.synchronize()
+    out[field] = shifted.clone().view(ref[field].dtype).reshape(ref[field].shape)
+    for k in ref:
+        assert torch.equal(out[k], ref[k]), k
+
+
 @pytest.mark.parametrize("n", [(3, 3), (4, 3, 3)])
 def test_points_close_to_facets(P, oracle_mod, n):
     """Points within 1e-11 to 2e-6 of facets, inside and across: the fast path's
