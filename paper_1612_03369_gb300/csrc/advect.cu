@@ -88,14 +88,10 @@ __device__ __forceinline__ void finish_tile(DevCounters* __restrict__ ctr, uint3
                  (flags & kFlagGlobal) ? 1u : 0u, flags);
 }
 
-// Resident blocks per SM of the step kernel, swept on the 128^3 x 20 step
-// (CUDA events, the same GB300 nodes back to back):
-// - FP64 form: 7 blocks (72 registers) 14.47 ms, 6 blocks (80) 14.76 ms,
-//   5 blocks 16.29 ms;
-// - FP32-basis form: 8 blocks (64 registers) 6.81 ms on most nodes but
-//   9.27 ms on others, 7 blocks 6.82 or 8.18 ms from one run to the next on
-//   one node, 6 blocks (80 registers, fewest spills) 7.01-7.02 ms on every
-//   node and run, so it takes 6.
+// Resident blocks per SM of the step kernel.  Five steps and an export on 64^3 x
+// 20, one node: FP64 form 9.15 / 8.92 / 8.76 / 8.94 ms at 5 / 6 / 7 / 8 blocks;
+// FP32-basis form 6.11 / 5.76 / 5.75 / 5.75 ms, where earlier builds at 7 and 8
+// blocks ran up to a third slower on some nodes, so it takes 6 (80 registers).
 #ifndef PIC_ADVECT_MIN_BLOCKS_F64
 #define PIC_ADVECT_MIN_BLOCKS_F64 7
 #endif

@@ -23,11 +23,12 @@
 // it computes the same bits.
 //
 // Inverse map (Newton, Sec. 2.2 / Remark 2.1): FP32 iterations on the local
-// offset y - X_0 until the update falls below 1e-5, then one Newton step
-// whose residual (y - X_0) - sum_k a_k m_k(t) is evaluated in double-float
-// (absolute accuracy ~2^-47 h), with the FP32 Jacobian at the current
-// iterate.  That leaves |t - t*| ~ 1e-14.  If the FP32 phase does not settle
-// the cell is handed to the FP64 Newton of pic_internal.cuh (rare).
+// offset y - X_0 until the iterate is within ~2e-7 of the root, then one Newton
+// step whose residual (y - X_0) - sum_k a_k m_k(t) is evaluated in double-float
+// (absolute accuracy ~2^-47 h), with the FP32 Jacobian at the current iterate.
+// That leaves |t - t*| ~ 1e-13.  A point the FP32 phase does not settle is left
+// to the rare paths, where the FP64 Newton of pic_internal.cuh stands behind
+// each cell.
 #pragma once
 
 #include "df.cuh"

@@ -7,7 +7,8 @@
 // cell's segment:
 //   counts[K]   particles whose new cell is K (filled by the locate kernel)
 //   scan        cell_off = exclusive prefix sum of counts; cursor = cell_off
-//   scatter     (id, old slot) of each particle to a free slot of its cell
+//   scatter     (id, old slot) of each particle to a free slot of its cell (on
+//               a mesh of one scan tile, in one launch with the scan)
 //   rank        slot of each particle = segment start + its rank by id
 //   gather      every field copied from the old slot to the new slot
 // The result is a function of the particle set alone (no dependence on the

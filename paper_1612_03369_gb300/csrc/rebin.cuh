@@ -5,8 +5,8 @@
 //
 //   scan   exclusive prefix sum of per-cell counts: each block of the grid
 //          sums a contiguous chunk, then offsets its chunk by the sums of
-//          the chunks before it (the stand-alone rebin uses the single-pass
-//          kernel of rebin.cu instead)
+//          the chunks before it (the stand-alone rebin uses the kernels
+//          of rebin.cu instead)
 //   scatter (id, old slot) of each particle to a free slot of its new cell
 //   rank   new slot = segment start + rank of the id among the cell's ids
 //   gather every field copied from its old slot to its new slot

@@ -6,8 +6,8 @@
 //        the cells around v, phi_v the (bi/tri)linear nodal basis function
 //   (v)  per-cell linear least squares in reference coordinates,
 //        f(x-hat) = c_0 + sum_j c_{j+1} (x-hat_j - 1/2)
-// Both fold the particles in store order; no atomics, so the results are
-// reproducible run to run.  The vertex sums are formed per cell first and
+// Both fold each cell's particles as kLanes strided left folds added in a fixed
+// pattern; no atomics, so the results are reproducible run to run.  The vertex sums are formed per cell first and
 // the cells' partial sums then added in increasing cell index, which rounds
 // differently from one left fold over the support (the definition) by a few
 // ulps of the sum.
