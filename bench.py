@@ -72,16 +72,16 @@ def advect_bytes(dim: int, ppc: float, n_props: int, xhat_bytes: int = 8, dof_by
 # multi-step call; traffic grows with the particle count, so a launch at
 # another size is scaled by its particles.  Keyed by precision (0 FP64
 # form, 1 FP32-basis form).
-ADVECT_DRAM_BYTES_PER_PARTICLE = {0: 1342.109e6 / 5242880, 1: 1017.072e6 / 5242880}
+ADVECT_DRAM_BYTES_PER_PARTICLE = {0: 1209.017e6 / 5242880, 1: 1012.980e6 / 5242880}
 # Warp instructions per 32 particle-steps and pipe utilisation of the same
 # captures: the advect kernel is bound by instruction issue (double-float
 # arithmetic on the FP32 pipe) in the FP64 form, and by issue and load
 # latency in the FP32-basis form, not by HBM.
 ADVECT_ISSUE = {
-    0: {"warp_instructions_per_32_particle_steps": 10758, "issue_active_pct": 76.3, "fma_pipe_active_pct": 61.2,
-        "top_stall": "not_selected 3.12 per issue (issue-bound)"},
-    1: {"warp_instructions_per_32_particle_steps": 4343, "issue_active_pct": 64.5, "fma_pipe_active_pct": 41.1,
-        "top_stall": "long_scoreboard 3.83 per issue"},
+    0: {"warp_instructions_per_32_particle_steps": 8052, "issue_active_pct": 74.2, "fma_pipe_active_pct": 56.6,
+        "top_stall": "long_scoreboard 3.10 per issue, not_selected 2.45"},
+    1: {"warp_instructions_per_32_particle_steps": 4234, "issue_active_pct": 64.2, "fma_pipe_active_pct": 39.4,
+        "top_stall": "long_scoreboard 3.68 per issue"},
 }
 
 
@@ -593,9 +593,9 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # (1,048,576 particles, RK4), counted by an ncu capture of these kernels:
 # reverse_lambda_kernel (G and lambda at 4.19M stage points, double-float)
 # and cell_partial_kernel (the per-cell sums, double-float).
-ADJOINT_C4_FP32_FLOPS_PER_REVERSE_STEP = 1.572e10 + 6.538e9
+ADJOINT_C4_FP32_FLOPS_PER_REVERSE_STEP = 1.186e10 + 6.538e9
 # DRAM bytes (read + write) of the same two kernels per reverse step, same capture.
-ADJOINT_C4_DRAM_BYTES_PER_REVERSE_STEP = (204.5e6 + 148.8e6) + (220.1e6 + 15.9e6)
+ADJOINT_C4_DRAM_BYTES_PER_REVERSE_STEP = (195.3e6 + 97.2e6) + (220.8e6 + 15.3e6)
 
 
 def run_adjoint(args):
@@ -792,16 +792,17 @@ def run_props(args):
 
 
 # FP32 flops (FADD + FMUL + 2 FFMA) per particle-step of the property-ODE
-# work beyond the plain step: the stage-gradient kernel (13,768) and the ODE
+# work beyond the plain step: the stage-gradient kernel (12,016) and the ODE
 # kernel (4,480), both in double-float, counted by ncu on the 64^3 x 20
 # workload (an ncu capture of these kernels).
-PROPS_ODE_FP32_FLOPS_PER_PARTICLE_STEP = 18248.0
+PROPS_ODE_FP32_FLOPS_PER_PARTICLE_STEP = 16496.0
 
 # FP64 operations per unit of the FP64-bound kernels (dadd + dmul + 2 dfma,
-# counted by an ncu capture on the 64^3 x 20 workload).
+# counted by ncu captures on 48^3 x 16, J = 8).  The chains decide most of their
+# steps in FP32 and emit in FP64; the FP64 pipe also carries their conversions.
 FP64_FLOPS = {
-    "mh_seed_kernel<3>": 238.96,           # per chain step
-    "cell_weights_kernel<3>": 1815.0,      # per cell
+    "mh_seed_kernel<3>": 8.97,             # per chain step
+    "cell_weights_kernel<3>": 1455.5,      # per cell
 }
 # FP64 peak: the GB300's nominal FP64 rate, 1.25 TFLOP/s (FMA = 2 flops).
 FP64_PEAK_TFLOPS = 1.25
