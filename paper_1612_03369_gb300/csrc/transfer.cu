@@ -6,11 +6,11 @@
 //        the cells around v, phi_v the (bi/tri)linear nodal basis function
 //   (v)  per-cell linear least squares in reference coordinates,
 //        f(x-hat) = c_0 + sum_j c_{j+1} (x-hat_j - 1/2)
-// Both fold each cell's particles as kLanes strided left folds added in a fixed
-// pattern; no atomics, so the results are reproducible run to run.  The vertex sums are formed per cell first and
-// the cells' partial sums then added in increasing cell index, which rounds
-// differently from one left fold over the support (the definition) by a few
-// ulps of the sum.
+// No atomics, so the results are reproducible run to run.  The linear fit folds a
+// cell's particles in store order.  The vertex sums are formed per cell first (one
+// left fold, or four strided ones added in a fixed pattern) and the cells' partial
+// sums then added in increasing cell index, which rounds differently from one left
+// fold over the support (the definition) by a few ulps of the sum.
 #include "df.cuh"
 #include "pic_internal.cuh"
 
@@ -32,23 +32,38 @@ __device__ __forceinline__ df minus_half(df t) {  // t - 1/2
 }
 __device__ __forceinline__ double df_to_f64(df a) { return (double)a.hi + (double)a.lo; }
 
-// kLanes neighbouring lanes share a cell, lane q folding its particles q, q +
-// kLanes, ..., and the lanes' compensated sums are then added in a fixed pattern
-// of exchanges.  The lanes' loads are consecutive, a 32-byte sector per cell and
-// array: with a thread per cell every load of a warp touched 32 sectors of as
-// many lines. With the property split off the FP64 pipe: vertex sums 92 -> 82 us,
-// linear fit 121 -> 107 us at 64^3 x 20 (FP32 issue 74 %; FP64 pipe 51 %).
+// In the vertex sums kLanes neighbouring lanes share a cell, lane q folding its
+// particles q, q + kLanes, ..., and the lanes' compensated sums are then added in a
+// fixed pattern of exchanges.  The lanes' loads are consecutive, a 32-byte sector
+// per cell and array: with a thread per cell every load of a warp touches 32 sectors
+// of as many lines.  The call (with the vertices' pass and the launches) takes 92 us
+// for 113 at 64^3 x 20, 141 for 180 at 36 per cell, 175 for 283 at 8 per cell unevenly
+// filled, 623 for 686 at 128^3.  At 4 per cell the exchanges cost more than the
+// loads (43 us for 32), so below kSharedFrom particles of capacity per cell a
+// thread takes a cell.
 constexpr int kLanes = 4;
+constexpr size_t kSharedFrom = 6;
 
-// acc of every lane of the group becomes the group's sum (the same in each).
-__device__ __forceinline__ void group_sum(df_acc& acc) {
+// The group's sums, dealt to its lanes: own[j] of lane q becomes the sum over the
+// group of acc[kLanes j + q].  Each round halves what a lane holds, so an entry
+// costs a lane 3/4 of an exchange and addition, 2 if every lane took every sum.
+__device__ __forceinline__ df_acc exchange_add(const df_acc& even, const df_acc& odd, uint32_t bit, int mask) {
+  const float s = __shfl_xor_sync(0xffffffffu, bit ? even.s : odd.s, mask);
+  const float e = __shfl_xor_sync(0xffffffffu, bit ? even.e : odd.e, mask);
+  df_acc r = bit ? odd : even;
+  const df t = two_sum(r.s, s);
+  r.s = t.hi;
+  r.e = __fadd_rn(__fadd_rn(r.e, e), t.lo);
+  return r;
+}
+template <int N>
+__device__ __forceinline__ void group_sums(const df_acc (&acc)[N], df_acc (&own)[N / kLanes], uint32_t q) {
+  static_assert(kLanes == 4 && N % 4 == 0, "two rounds");
+  df_acc half[N / 2];
 #pragma unroll
-  for (int o = 1; o < kLanes; o <<= 1) {
-    const float s = __shfl_xor_sync(0xffffffffu, acc.s, o), e = __shfl_xor_sync(0xffffffffu, acc.e, o);
-    const df r = two_sum(acc.s, s);
-    acc.s = r.hi;
-    acc.e = __fadd_rn(__fadd_rn(acc.e, e), r.lo);
-  }
+  for (int k = 0; k < N / 2; ++k) half[k] = exchange_add(acc[2 * k], acc[2 * k + 1], q & 1u, 1);
+#pragma unroll
+  for (int j = 0; j < N / 4; ++j) own[j] = exchange_add(half[2 * j], half[2 * j + 1], q >> 1, 2);
 }
 
 // One particle's loads, issued an iteration ahead of their use.
@@ -79,22 +94,22 @@ __device__ __forceinline__ void group_cell(const uint32_t* __restrict__ cell_off
 }
 
 // Two phases, both deterministic.
-// Phase 1, kLanes lanes per cell: each particle of the cell is read once and
+// Phase 1, L lanes (kLanes or 1) per cell: each particle of the cell is read once and
 // its 2^D corner weights (the tensor product of (1 - t_a, t_a), multiplied in
 // axis order) are folded into the cell's partial sums
 //   num[c][K] = sum w_c(x-hat_i) p_i,   den[c][K] = sum w_c(x-hat_i)
 // stored as double-float pairs, corner-major ([c][C]) so that the phase-2
 // reads of a warp coalesce.
-template <int D>
+template <int D, int L>
 __global__ void __launch_bounds__(128) vertex_partial_kernel(const uint32_t* __restrict__ cell_off,
                                                              const float2* __restrict__ xh, const double* __restrict__ prop,
                                                              uint32_t C, size_t cap, float2* __restrict__ part,
                                                              DevCounters* __restrict__ ctr) {
   constexpr int NC = 1 << D;
-  constexpr uint32_t kCells = 128 / kLanes;  // per block and pass
-  const uint32_t q = threadIdx.x % kLanes;
+  constexpr uint32_t kCells = 128 / L;  // per block and pass
+  const uint32_t q = threadIdx.x % L;
   for (uint32_t K0 = blockIdx.x * kCells; K0 < C; K0 += gridDim.x * kCells) {
-    const uint32_t K = K0 + threadIdx.x / kLanes;
+    const uint32_t K = K0 + threadIdx.x / L;
     uint32_t beg, end;
     bool bad;
     group_cell(cell_off, K, C, cap, beg, end, bad, ctr);
@@ -103,9 +118,9 @@ __global__ void __launch_bounds__(128) vertex_partial_kernel(const uint32_t* __r
     for (int c = 0; c < NC; ++c) num[c] = den[c] = acc_zero();
     ParticleLoads<D> next;
     next.load(xh, prop, cap, beg + q, end);
-    for (uint32_t i = beg + q; i < end; i += kLanes) {
+    for (uint32_t i = beg + q; i < end; i += L) {
       const ParticleLoads<D> now = next;
-      next.load(xh, prop, cap, i + kLanes, end);
+      next.load(xh, prop, cap, i + L, end);
       df f[D][2];  // f[a][0] = 1 - t_a, f[a][1] = t_a
 #pragma unroll
       for (int a = 0; a < D; ++a) {
@@ -123,16 +138,25 @@ __global__ void __launch_bounds__(128) vertex_partial_kernel(const uint32_t* __r
         acc_add(den[c], w);
       }
     }
+    df_acc num_q[NC / L], den_q[NC / L];
+    if constexpr (L == 1) {
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      group_sum(num[c]);
-      group_sum(den[c]);
-      if (K < C && (uint32_t)c % kLanes == q) {
-        const df a = acc_result(num[c]), b = acc_result(den[c]);
-        part[(size_t)c * C + K] = make_float2(a.hi, a.lo);
-        part[(size_t)(NC + c) * C + K] = make_float2(b.hi, b.lo);
+      for (int c = 0; c < NC; ++c) {
+        num_q[c] = num[c];
+        den_q[c] = den[c];
       }
+    } else {
+      group_sums(num, num_q, q);
+      group_sums(den, den_q, q);
     }
+    if (K < C)
+#pragma unroll
+      for (int j = 0; j < NC / L; ++j) {
+        const size_t c = (size_t)(L * j) + q;
+        const df a = acc_result(num_q[j]), b = acc_result(den_q[j]);
+        part[c * C + K] = make_float2(a.hi, a.lo);
+        part[(NC + c) * C + K] = make_float2(b.hi, b.lo);
+      }
   }
 }
 
@@ -176,13 +200,13 @@ __global__ void __launch_bounds__(256) vertex_gather_kernel(const __grid_constan
   }
 }
 
-// The normal equations (A^T A) c = A^T p of the cell's design matrix, rows
-// (1, x-hat_i - 1/2), kLanes lanes per cell; Gaussian elimination with partial
-// pivoting; the mean where the cell has at most D particles or a pivot is <=
-// 1e-12 of the largest diagonal entry.  The sums are left in shared memory and
-// solved by one warp of the block, a cell per lane (an FP64 warp instruction
-// takes the FP64 pipe as long for 8 lanes as for 32), the block's warps in turn
-// while the others go on to the next cells.
+// Thread per cell: normal equations (A^T A) c = A^T p of the cell's design
+// matrix, rows (1, x-hat_i - 1/2), folded in store order; Gaussian
+// elimination with partial pivoting; the mean where the cell has at most D
+// particles or a pivot is <= 1e-12 of the largest diagonal entry.
+// The fold stays one left fold per sum: a pivot may be 1e-12 of the diagonal, and a
+// sum folded in another order (four lanes a cell: 115 -> 104 us a call at 64^3 x 20) would
+// move such a cell's coefficients by 1e12 times its rounding.
 template <int D>
 __global__ void __launch_bounds__(128) lsq_linear_kernel(const uint32_t* __restrict__ cell_off,
                                                          const float2* __restrict__ xh, const double* __restrict__ prop,
@@ -190,80 +214,57 @@ __global__ void __launch_bounds__(128) lsq_linear_kernel(const uint32_t* __restr
                                                          double* __restrict__ coef, uint32_t* __restrict__ count,
                                                          DevCounters* __restrict__ ctr) {
   constexpr int NB = D + 1;
-  constexpr int NE = NB * (NB + 3) / 2 - 1;  // upper triangle of A^T A but the count, and A^T p
-  constexpr uint32_t kCells = 128 / kLanes;
-  static_assert(kCells == 32, "one cell per lane of the solving warp");
-  __shared__ float2 s_sum[2][NE][kCells];
-  __shared__ uint32_t s_n[2][kCells];
-  const uint32_t q = threadIdx.x % kLanes, g = threadIdx.x / kLanes, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  uint32_t pass = 0;
-  for (uint32_t K0 = blockIdx.x * kCells; K0 < C; K0 += gridDim.x * kCells, ++pass) {
-    const uint32_t buf = pass & 1u;
-    {
-      uint32_t beg, end;
-      bool bad;
-      group_cell(cell_off, K0 + g, C, cap, beg, end, bad, ctr);
-      // accumulated in double-float (row a = (1, x-hat - 1/2))
-      df_acc acc[NE];
-#pragma unroll
-      for (int e = 0; e < NE; ++e) acc[e] = acc_zero();
-      ParticleLoads<D> next;
-      next.load(xh, prop, cap, beg + q, end);
-      for (uint32_t i = beg + q; i < end; i += kLanes) {
-        const ParticleLoads<D> now = next;
-        next.load(xh, prop, cap, i + kLanes, end);
-        df a[NB];
-#pragma unroll
-        for (int j = 0; j < D; ++j) a[j + 1] = minus_half(df_make(now.t[j].x, now.t[j].y));
-        const df p = split_f64(now.p);
-        int e = 0;
-#pragma unroll
-        for (int r = 0; r < NB; ++r) {
-#pragma unroll
-          for (int k = r; k <= NB; ++k) {
-            if (r == 0 && k == 0) continue;  // the count
-            const df b = k == NB ? p : a[k];
-            if (r == 0)
-              acc_add(acc[e++], b);
-            else
-              acc_mad(acc[e++], a[r], b);
-          }
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < NE; ++e) {
-        group_sum(acc[e]);
-        if ((uint32_t)e % kLanes == q) {
-          const df r = acc_result(acc[e]);
-          s_sum[buf][e][g] = make_float2(r.hi, r.lo);
-        }
-      }
-      if (q == 0) s_n[buf][g] = bad ? PIC_LOST : end - beg;
+  for (uint32_t K = blockIdx.x * blockDim.x + threadIdx.x; K < C; K += gridDim.x * blockDim.x) {
+    const uint32_t beg = cell_off[K], end = cell_off[K + 1];
+    if (end > cap || beg > end) {
+      latch_status(ctr, PIC_STATUS_BOUNDS);
+      continue;
     }
-    // one barrier a pass: the buffer is written again two passes on, after the
-    // barrier that its solving warp passes when it is done
-    __syncthreads();
-    if (warp != (pass & 3u)) continue;
-    const uint32_t K = K0 + lane, n = s_n[buf][lane];
-    if (K >= C || n == PIC_LOST) continue;
-    double M[NB][NB + 1];
-    int e = 0;
+    // the upper triangle of A^T A, A^T p and sum p, accumulated in
+    // double-float (row a = (1, x-hat - 1/2)), then converted once
+    df_acc Ma[NB][NB + 1];
 #pragma unroll
     for (int r = 0; r < NB; ++r)
 #pragma unroll
-      for (int k = r; k <= NB; ++k) {
-        if (r == 0 && k == 0) {
-          M[0][0] = (double)n;
-          continue;
+      for (int q = 0; q <= NB; ++q) Ma[r][q] = acc_zero();
+    ParticleLoads<D> next;
+    next.load(xh, prop, cap, beg, end);
+    for (uint32_t i = beg; i < end; ++i) {
+      const ParticleLoads<D> now = next;
+      next.load(xh, prop, cap, i + 1, end);
+      df a[NB];
+      a[0] = df_make(1.0f, 0.f);
+#pragma unroll
+      for (int j = 0; j < D; ++j) a[j + 1] = minus_half(df_make(now.t[j].x, now.t[j].y));
+      const df p = split_f64(now.p);
+#pragma unroll
+      for (int r = 0; r < NB; ++r) {
+#pragma unroll
+        for (int q = r; q < NB; ++q) {
+          if (r == 0 && q == 0) continue;  // the count
+          if (r == 0)
+            acc_add(Ma[r][q], a[q]);  // a[0] = 1
+          else
+            acc_mad(Ma[r][q], a[r], a[q]);
         }
-        const float2 v = s_sum[buf][e++][lane];
-        M[r][k] = (double)v.x + (double)v.y;
+        if (r == 0)
+          acc_add(Ma[r][NB], p);
+        else
+          acc_mad(Ma[r][NB], a[r], p);
       }
+    }
+    double M[NB][NB + 1];
+#pragma unroll
+    for (int r = 0; r < NB; ++r)
+#pragma unroll
+      for (int q = r; q <= NB; ++q) M[r][q] = df_to_f64(acc_result(Ma[r][q]));
+    M[0][0] = (double)(end - beg);
     const double sum = M[0][NB];
 #pragma unroll
     for (int r = 1; r < NB; ++r)
 #pragma unroll
-      for (int k = 0; k < r; ++k) M[r][k] = M[k][r];
+      for (int q = 0; q < r; ++q) M[r][q] = M[q][r];
+    const uint32_t n = end - beg;
     double c[NB];
 #pragma unroll
     for (int r = 0; r < NB; ++r) c[r] = 0.0;
@@ -361,13 +362,16 @@ extern "C" pic_status pic_interpolate_to_vertices(pic_particles p, pic_mesh mesh
     }
   }
   const double* pv = p->props[p->cur] + (size_t)prop * p->capacity;
-  const int g1 = transfer_grid((size_t)p->C * kLanes, 128), g2 = transfer_grid((size_t)m.nverts, 256);
+  const bool shared = p->capacity >= kSharedFrom * p->C;
+  const int g1 = transfer_grid((size_t)p->C * (shared ? kLanes : 1), 128), g2 = transfer_grid((size_t)m.nverts, 256);
   float2* part = reinterpret_cast<float2*>(p->xfer);  // [2 * 2^dim][C] double-float pairs
   if (mesh->dim == 2) {
-    vertex_partial_kernel<2><<<g1, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, part, p->ctr);
+    auto partial = shared ? vertex_partial_kernel<2, kLanes> : vertex_partial_kernel<2, 1>;
+    partial<<<g1, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, part, p->ctr);
     vertex_gather_kernel<2><<<g2, 256, 0, st>>>(m, part, empty_fill, avg, weight);
   } else {
-    vertex_partial_kernel<3><<<g1, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, part, p->ctr);
+    auto partial = shared ? vertex_partial_kernel<3, kLanes> : vertex_partial_kernel<3, 1>;
+    partial<<<g1, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, part, p->ctr);
     vertex_gather_kernel<3><<<g2, 256, 0, st>>>(m, part, empty_fill, avg, weight);
   }
   count_launches(2);
@@ -387,7 +391,7 @@ extern "C" pic_status pic_project_linear(pic_particles p, pic_mesh mesh, int pro
     if (r0 != PIC_OK) return r0;
   }
   const double* pv = p->props[p->cur] + (size_t)prop * p->capacity;
-  const int g = transfer_grid((size_t)p->C * kLanes, 128);
+  const int g = transfer_grid((size_t)p->C, 128);
   if (mesh->dim == 2)
     lsq_linear_kernel<2><<<g, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, empty_fill, coef,
                                             count, p->ctr);

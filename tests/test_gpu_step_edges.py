@@ -63,8 +63,8 @@ def test_rough_and_scaled_fields(P, oracle_mod, n, scale):
     H.assert_same_store(H.gpu_state(parts), op, wl)
 
 
-# cells of 0 to 9 particles: partial batches of the averages, partial groups of
-# four lanes in the transfers
+# cells of 0 to 9 particles: partial batches of the averages, empty cells and
+# ragged ones in the transfers
 @pytest.mark.parametrize("n", [(7, 5), (33, 9), (5, 4, 3)])
 def test_transfers_of_short_cells(P, oracle_mod, n):
     C = int(np.prod(n))
@@ -76,6 +76,16 @@ def test_transfers_of_short_cells(P, oracle_mod, n):
     oa, oc = oracle_mod.cell_average(C, op.cell, vals, empty_fill=-3.0)
     np.testing.assert_array_equal(gc.cpu().numpy(), oc)
     np.testing.assert_array_equal(ga.cpu().numpy(), oa)  # the same left fold
+
+
+# four lanes share a cell from six particles of capacity per cell on
+@pytest.mark.parametrize("n", [(9, 7), (5, 4, 3)])
+@pytest.mark.parametrize("low, span", [(5, 1), (6, 1), (0, 13), (3, 10)])
+def test_vertex_sums_either_side_of_shared_cells(P, oracle_mod, n, low, span):
+    C = int(np.prod(n))
+    per = (low + np.arange(C) % span).astype(np.uint32)
+    mesh, parts, om, op, vals = T._pair(P, oracle_mod, n, per_cell=per)
+    T._check_vertex(oracle_mod, parts, om, op, vals)
 
 
 def test_geometric_mean_of_extreme_values(P, oracle_mod):
