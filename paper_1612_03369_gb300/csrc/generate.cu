@@ -452,21 +452,20 @@ __device__ df rho_hat_df(const MeshView& m, uint32_t K, const double* __restrict
 }
 
 // The acceptance test that FP32 values left open: by double-float ones where
-// they differ by more than their own bound (tau is FP32's, 2^-20 of it theirs:
-// they keep ~2^-46 where FP32 keeps 2^-24), and by the definition otherwise,
+// they differ by more than `sure`, and by the definition otherwise,
 // u rho-hat(current) < rho-hat(proposal) in the written sequence of IEEE
 // operations (two evaluations are 2000 FP64 operations, 33 k clocks of an SM's
 // FP64 pipe, and came 1.6 times per warp with FP32 alone before them).
 template <int D>
 __device__ __noinline__ bool mh_accept_rn(const MeshView& m, uint32_t K, const double* __restrict__ rho, RawPoint<D> cur,
-                                          RawPoint<D> prop, bool at_centre, double u, float tau) {
+                                          RawPoint<D> prop, bool at_centre, double u, float sure) {
   double t[D], y[D];
   raw_coordinates<D>(cur, t);
   if (at_centre)
 #pragma unroll
     for (int a = 0; a < D; ++a) t[a] = 0.5;
   raw_coordinates<D>(prop, y);
-  if (tau > 0x1p-90f && tau < 0x1p90f) {  // no double-float term below the normal floats
+  if (sure < INFINITY) {
     df td[D], yd[D];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
@@ -475,7 +474,6 @@ __device__ __noinline__ bool mh_accept_rn(const MeshView& m, uint32_t K, const d
     }
     const df lhs = df_mul(df_from_double(u), rho_hat_df<D>(m, K, rho, td));
     const df diff = df_sub(rho_hat_df<D>(m, K, rho, yd), lhs);
-    const float sure = 0x1p-18f * tau;  // four times the bound
     if (diff.hi > sure) return true;
     if (diff.hi < -sure) return false;
   }
@@ -505,13 +503,15 @@ __device__ __noinline__ void mh_emit(const MeshView& m, const StoreView& s, uint
   for (int p = 0; p < s.n_props; ++p) s.props[(size_t)p * s.cap + q] = 0.0;
 }
 
-// rho-hat in FP32, with a bound of its error: the density's monomial
-// coefficients in the cell and the rows of the map's Jacobian.
+// rho-hat in FP32: the density's monomial coefficients in the cell and the rows
+// of the map's Jacobian; and how far u rho-hat(current) - rho-hat(proposal) has
+// to be from 0 for its FP32 and its double-float value to have the right sign
+// (infinite where they cannot decide).
 template <int D>
 struct RhoHat32 {
   float c[1 << D];      // 1, t0, t1, (t2,) mixed ones
   MapRow<D> row[D];
-  float tau;            // |rho-hat in FP32 - rho-hat| for t within 2^-24 of the given one
+  float sure32, sure_df;
 
   __device__ __forceinline__ void load(const MeshView& m, uint32_t K, const double* __restrict__ rho) {
     int ijk[3];
@@ -535,7 +535,7 @@ struct RhoHat32 {
     }
     const GlobalCells<D, false> cs{m};
     const float4* B = cs.block(K);
-    float S = 1.f;
+    float s[D];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       row[a] = load_row<D>(cs, B, 0, a);
@@ -546,13 +546,31 @@ struct RhoHat32 {
       for (int k = 0; k < D; ++k) r = fmaxf(r, fabsf(row[a].a[k]));
 #pragma unroll
       for (int k = D; k < (1 << D) - 1; ++k) mixed += fabsf(row[a].a[k]);
-      S *= r + mixed;
+      s[a] = r + mixed;
     }
     // With s_i the bound of row i and e = 2^-24: every entry of J is off by at
     // most 7 e s_i (coefficient, coordinate and FMA roundings), the determinant,
     // a sum of D! products, by 26 e D! s_0..s_(D-1), rho_h by 11 e R; the product
-    // by less than 256 e R S.
-    tau = 0x1p-16f * R * S;
+    // by less than 256 e R S = tau.  The double-float form keeps ~2^-46 where FP32
+    // keeps 2^-24, so its bound is 2^-20 tau.  Two evaluations and u's own rounding
+    // make 2.5 tau, and four times the bound in double-float.
+    const float minor = D == 3 ? s[1] * s[D - 1] : s[1];
+    const float S = s[0] * minor, tau = 0x1p-16f * R * S;
+    // These are relative roundings, true while every product of the evaluation,
+    // and in double-float its part of 2^-48 too, is a normal float: R, the rows
+    // and the products of rows that the determinant forms lie far enough inside
+    // that range, or the filter declines (2D, uniform cells, density 1e-42: an
+    // FP32 product is a few of the smallest float there, and 3 in 1,000 of the
+    // decisions taken from it were wrong).
+    float least = fminf(fminf(R, S), fminf(minor, R * S)), most = fmaxf(fmaxf(R, S), fmaxf(minor, R * S));
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      least = fminf(least, s[a]);
+      most = fmaxf(most, s[a]);
+    }
+    const bool normal32 = least > 0x1p-100f && most < 0x1p100f, normal_df = least > 0x1p-74f && normal32;
+    sure32 = normal32 ? 2.5f * tau : INFINITY;
+    sure_df = normal_df ? 0x1p-18f * tau : INFINITY;
   }
 
   __device__ __forceinline__ float at(const float t[D]) const {
@@ -596,7 +614,6 @@ __global__ void __launch_bounds__(128, 5) mh_seed_kernel(const __grid_constant__
     if (end > s.cap || beg >= end) continue;
     RhoHat32<D> f;
     f.load(m, K, rho);
-    const float sure = 2.5f * f.tau;
     RawPoint<D> cur;
     float t32[D];
 #pragma unroll
@@ -620,8 +637,8 @@ __global__ void __launch_bounds__(128, 5) mh_seed_kernel(const __grid_constant__
       const uint64_t ur = splitmix64_mix(z += kGamma);
       const float ry = f.at(t32);
       const float diff = ry - (float)(uint32_t)(ur >> 40) * 0x1p-24f * rc;
-      bool accept = diff > sure;
-      if (!(fabsf(diff) > sure)) accept = mh_accept_rn<D>(m, K, rho, cur, y, at_centre, unit53(ur), f.tau);
+      bool accept = diff > f.sure32;
+      if (!(fabsf(diff) > f.sure32)) accept = mh_accept_rn<D>(m, K, rho, cur, y, at_centre, unit53(ur), f.sure_df);
       if (accept) {
         cur = y;
         rc = ry;
