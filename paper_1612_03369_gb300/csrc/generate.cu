@@ -554,6 +554,17 @@ struct RhoHat32 {
     // by less than 256 e R S = tau.  The double-float form keeps ~2^-46 where FP32
     // keeps 2^-24, so its bound is 2^-20 tau.  Two evaluations and u's own rounding
     // make 2.5 tau, and four times the bound in double-float.
+    //
+    // The written sequence has an error of its own, since it sums whole
+    // coordinates: with f = 2^-53 and A_i the largest |x_i| of the mesh, an entry of
+    // row i is off by at most 22 f A_i (the derivative weights' magnitudes sum to
+    // 2; 11 roundings), the determinant by D! S f (22 sum A_i / s_i + 20), rho_h by
+    // 11 f R; the product by less than 2^-29 tau (2 + sum A_i / s_i).  A decision has
+    // to be clear of that too, twice, to be the sequence's (at |x| / h = 1e10 one in
+    // 2e5 was not).
+    float far = 2.f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) far += __double2float_ru(fmax(fabs(m.dlo[a]), fabs(m.dhi[a]))) / s[a];
     const float minor = D == 3 ? s[1] * s[D - 1] : s[1];
     const float S = s[0] * minor, tau = 0x1p-16f * R * S;
     // These are relative roundings, true while every product of the evaluation,
@@ -569,8 +580,9 @@ struct RhoHat32 {
       most = fmaxf(most, s[a]);
     }
     const bool normal32 = least > 0x1p-100f && most < 0x1p100f, normal_df = least > 0x1p-74f && normal32;
-    sure32 = normal32 ? 2.5f * tau : INFINITY;
-    sure_df = normal_df ? 0x1p-18f * tau : INFINITY;
+    const float sequence = 0x1.4p-28f * far * tau;
+    sure32 = normal32 ? 2.5f * tau + sequence : INFINITY;
+    sure_df = normal_df ? 0x1p-18f * tau + sequence : INFINITY;
   }
 
   __device__ __forceinline__ float at(const float t[D]) const {

@@ -45,3 +45,13 @@ def test_chains_of_cells_in_small_units(P, oracle_mod, h):
     X = W.jittered_vertices(n, 8) * (np.array(h) * np.array(n))[:, None]
     rho = np.random.default_rng(9).uniform(0.5, 2.0, X.shape[1])
     _chains_equal(P, oracle_mod, n, X, rho, 40, 25)
+
+
+# the sequence sums whole coordinates: its own error grows with |x| / h, to 2e-6 of
+# rho-hat at 1e10 and 2e-4, past FP32's, at 1e12; among 1.4 M steps some fall into it
+@pytest.mark.parametrize("offset", [1e6, 1e9, 1e10, 1e11, 1e12])
+@pytest.mark.parametrize("n", [(9, 8), (5, 4, 3)])
+def test_chains_of_meshes_far_from_the_origin(P, oracle_mod, n, offset):
+    X = W.jittered_vertices(n, 8) + offset / max(n)
+    rho = np.random.default_rng(9).uniform(0.5, 2.0, X.shape[1])
+    _chains_equal(P, oracle_mod, n, X, rho, 200, 100)
