@@ -183,8 +183,9 @@ __device__ __forceinline__ void jacobian_row32(const MapRow<D>& w, const float t
 // instruction, within 2 ulp; the IEEE division took a dozen): it scales a
 // Newton update whose last, double-float-residual step is ~1e-7, so it moves
 // the root by ~3e-14, the size of the FP32 Jacobian's own error.  A zero or
-// non-finite determinant fails; one so small that its reciprocal overflows
-// gives an update the caller rejects (|d| > 1e3).
+// non-finite determinant fails; so does one of 2^126 and more, for which that
+// reciprocal is 0 and the update with it; one so small that its reciprocal
+// overflows gives an update the caller rejects (|d| > 1e3).
 template <int D>
 struct Adjugate32 {
   float c[D][D];  // cofactors: (J^{-1})_ij = c[j][i] inv
@@ -196,7 +197,7 @@ __device__ __forceinline__ bool adjugate32(const float J[D][D], Adjugate32<D>& A
   auto det2 = [](float a, float b, float c, float e) { return __fmaf_rn(a, b, -__fmul_rn(c, e)); };  // a b - c e
   if constexpr (D == 2) {
     const float det = det2(J[0][0], J[1][1], J[0][1], J[1][0]);
-    if (!(fabsf(det) > 0.f) || !isfinite(det)) return false;
+    if (!(fabsf(det) > 0.f && fabsf(det) < 0x1p126f)) return false;
     A.inv = __fdividef(1.0f, det);
     A.c[0][0] = J[1][1];
     A.c[0][1] = -J[1][0];
@@ -207,7 +208,7 @@ __device__ __forceinline__ bool adjugate32(const float J[D][D], Adjugate32<D>& A
     A.c[0][1] = det2(J[1][2], J[2][0], J[1][0], J[2][2]);
     A.c[0][2] = det2(J[1][0], J[2][1], J[1][1], J[2][0]);
     const float det = __fmaf_rn(J[0][2], A.c[0][2], __fmaf_rn(J[0][1], A.c[0][1], __fmul_rn(J[0][0], A.c[0][0])));
-    if (!(fabsf(det) > 0.f) || !isfinite(det)) return false;
+    if (!(fabsf(det) > 0.f && fabsf(det) < 0x1p126f)) return false;
     A.inv = __fdividef(1.0f, det);
     A.c[1][0] = det2(J[0][2], J[2][1], J[0][1], J[2][2]);
     A.c[1][1] = det2(J[0][0], J[2][2], J[0][2], J[2][0]);

@@ -55,3 +55,21 @@ def test_chains_of_meshes_far_from_the_origin(P, oracle_mod, n, offset):
     X = W.jittered_vertices(n, 8) + offset / max(n)
     rho = np.random.default_rng(9).uniform(0.5, 2.0, X.shape[1])
     _chains_equal(P, oracle_mod, n, X, rho, 200, 100)
+
+
+# cells whose determinant lies where the FP32 reciprocal of it is 0 (2^126 to 2^128),
+# and on either side
+@pytest.mark.parametrize("n, h", [((5, 4), 2.0**58), ((5, 4), 2.0**63.5), ((5, 4), 2.0**66),
+                                  ((5, 4, 3), 2.0**38), ((5, 4, 3), 2.0**42.3), ((5, 4, 3), 2.0**45)])
+def test_steps_in_cells_of_large_units(P, oracle_mod, n, h):
+    d = len(n)
+    X = W.jittered_vertices(n, 4)
+    U = W.zero_wall_normal(n, W.normalise_max(np.random.default_rng(6).standard_normal((d, W.q2_node_coords(n, X).shape[1]))))
+    unit = h * np.array(n, dtype=float)[:, None]
+    wl = W.Workload("units", d, n, X * unit, U * unit, 9, None, 1, 4, W.cfl_dt(n, X, U, 0.5), 3, 4, W.particle_seed(4))
+    mesh, parts = H.gpu_seed(wl, n_props=0)
+    om = oracle_mod.Mesh(n, wl.X, wl.U)
+    op = oracle_mod.seed_particles(om, uniform_count=9, seed=wl.pseed, n_props=0)
+    parts.advect(wl.dt, 4, 3)
+    op = oracle_mod.advect(om, op, wl.dt, 4, 3)
+    H.assert_same_store(H.gpu_state(parts), op, wl, tol_x=H.TOL_X * unit.max())
