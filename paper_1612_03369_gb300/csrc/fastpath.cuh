@@ -859,20 +859,11 @@ __device__ __forceinline__ void lagrange2_df(df t, df l[3]) {
 // evaluated by nested Horner steps, 26 per component in 3D (8 in 2D),
 // each a double-float multiply-add.  For smooth fields |C_pqr| falls
 // with p + q + r (C_000 is the centre node's value), so the evaluation is
-// well conditioned.
-//
-// Two kinds of step.  The steps that bring in the constant and the linear
-// coefficients, and every step of the 2D form, are plain double-float ones
-// (df_horner, 12 operations).  The partial sums of the remaining ones, all of
-// order >= 2 in the cell size, stay below a bound M that the field set-up knows
-// per cell and component, so their high parts are kept on one fixed grid, the
-// multiples of ulp(B) for a bias B > 3 M: sums of high parts are then exact,
-// which takes the place of the two_sum (7 operations, 6 where the sum is only
-// added on, see grid_step).  The grid costs the low parts two or three bits
-// against a normalised pair, relative to M and not to u: error of dt u against
-// 128-bit arithmetic, CFL 0.5, curl field: the same to two digits as with plain
-// steps throughout on 16^3 cells and finer, 3.9e-17 against 3.1e-17 on 12^3.
-// 224 operations per component against 312.
+// well conditioned.  (Sums of order two and above with their high parts on one
+// fixed grid take 7 operations a step for 12, and 8.02 ms for 8.85 in five 64^3 x
+// 20 RK4 steps; but their low parts lose two or three bits of the largest sum,
+// which made positions up to 1.4 times and gradients 2 to 10 times less exact on
+// meshes below 16 cells a side.)
 
 // c + a s in double-float, the result left unnormalised (its low part may
 // exceed half an ulp of the high part slightly; the next step multiplies it
@@ -885,48 +876,13 @@ __device__ __forceinline__ df df_horner(df a, df s, df c) {
   return df_make(q.hi, __fadd_rn(q.lo, __fadd_rn(e, c.lo)));
 }
 
-// A pair whose high part carries the bias B: the value is (b - B) + lo, b - B
-// a multiple of ulp(B).
-struct biased {
-  float b, lo;
-};
-
-// c + a s on the grid of B: b = RN(c.b + a.hi s.hi) rounds to the grid (b and
-// c.b lie in B's binade), z = b - c.b is exact, and the fused remainder
-// a.hi s.hi - z is below half a grid step.
-__device__ __forceinline__ biased grid_step(df a, df s, biased c) {
-  biased r;
-  r.b = __fmaf_rn(a.hi, s.hi, c.b);
-  const float z = __fsub_rn(r.b, c.b);
-  float e = __fmaf_rn(a.lo, s.hi, c.lo);
-  e = __fmaf_rn(a.hi, s.lo, e);
-  r.lo = __fadd_rn(__fmaf_rn(a.hi, s.hi, -z), e);
-  return r;
-}
-
-__device__ __forceinline__ df unbias(biased a, float B) { return df_make(__fsub_rn(a.b, B), a.lo); }
-
-// The grid's bias for partial sums up to M: 1.5 times a power of two, above
-// 3 M and at most 6 M, so that B +- M stays in one binade.
-__device__ __forceinline__ float grid_bias(float M) {
-  const int e = __float_as_int(fminf(M, 0x1p124f)) & 0x7f800000;
-  return 3.0f * __int_as_float(e + 0x00800000);  // 2^floor(log2 M) * 2 * 3
-}
-
-// Whether coefficient (p, q, r) of the 3D table is stored on the grid
-// (B + high part rounded to the grid, remainder): the addends of grid steps.
-// The constant and linear ones are added by plain steps and the p = 2 ones
-// only multiply; those are plain pairs.
-__host__ __device__ constexpr bool qc_on_grid(int p, int q, int r) { return p < 2 && p + q + r >= 2; }
-
 // s = t - 1/2 in double-float.
 __device__ __forceinline__ df centred(df t) {
   const df d = two_sum(t.hi, -0.5f);
   return fast_two_sum(d.hi, __fadd_rn(d.lo, t.lo));
 }
 
-// One slice of Qc (five float4: ten high parts, then ten low parts; in 3D the
-// tenth high part is the component's grid bias).
+// One slice of Qc (five float4: ten high parts, then ten low parts).
 template <class Ld>
 __device__ __forceinline__ void load_slice(const Ld& ld, const float4* p, float hi[10], float lo[10]) {
   float f[20];
@@ -956,39 +912,18 @@ __device__ __forceinline__ void q2_eval_df(const Ld& ld, const float4* cell, con
   for (int comp = 0; comp < D; ++comp) {
     const float4* cq = cell + comp * (5 * NS);
     df rr;
-    float hi[10], lo[10];
-    auto plain = [&](int k) { return df_make(hi[k], lo[k]); };
-    if constexpr (D == 2) {
-      load_slice(ld, cq, hi, lo);
+#pragma unroll
+    for (int r = NS - 1; r >= 0; --r) {
+      float hi[10], lo[10];
+      load_slice(ld, cq + 5 * r, hi, lo);
+      auto c = [&](int k) { return df_make(hi[k], lo[k]); };
       df h[3];
 #pragma unroll
-      for (int q = 0; q < 3; ++q) h[q] = df_horner(df_horner(plain(3 * q + 2), s[0], plain(3 * q + 1)), s[0], plain(3 * q));
-      rr = df_norm(df_horner(df_horner(h[2], s[1], h[1]), s[1], h[0]));
-    } else {
-      // row(q): the slice's row q, all on the grid
-      auto grid = [&](int k) { return biased{hi[k], lo[k]}; };
-      auto inner = [&](int q) { return unbias(grid_step(plain(3 * q + 2), s[0], grid(3 * q + 1)), hi[9]); };
-      auto row = [&](int q) { return grid_step(inner(q), s[0], grid(3 * q)); };
-      load_slice(ld, cq + 10, hi, lo);  // r = 2
-      df g2;
-      {
-        const df v = unbias(grid_step(unbias(row(2), hi[9]), s[1], row(1)), hi[9]);
-        g2 = unbias(grid_step(v, s[1], row(0)), hi[9]);
-      }
-      load_slice(ld, cq + 5, hi, lo);  // r = 1: the linear coefficient leads row 0
-      {
-        const df v = unbias(grid_step(unbias(row(2), hi[9]), s[1], row(1)), hi[9]);
-        const df g1 = df_horner(v, s[1], df_horner(inner(0), s[0], plain(0)));
-        g2 = df_horner(g2, s[2], g1);
-      }
-      load_slice(ld, cq, hi, lo);  // r = 0: constant, and linear ones in rows 0 and 1
-      {
-        const df h1 = df_horner(inner(1), s[0], plain(3));
-        const df v = df_horner(unbias(row(2), hi[9]), s[1], h1);
-        const df h0 = df_horner(df_horner(plain(2), s[0], plain(1)), s[0], plain(0));
-        rr = df_norm(df_horner(g2, s[2], df_horner(v, s[1], h0)));
-      }
+      for (int q = 0; q < 3; ++q) h[q] = df_horner(df_horner(c(3 * q + 2), s[0], c(3 * q + 1)), s[0], c(3 * q));
+      const df g = df_horner(df_horner(h[2], s[1], h[1]), s[1], h[0]);
+      rr = r == NS - 1 ? g : df_horner(rr, s[D - 1], g);
     }
+    rr = df_norm(rr);
     // constant indices keep u in registers under the rolled loop
 #pragma unroll
     for (int a = 0; a < D; ++a)

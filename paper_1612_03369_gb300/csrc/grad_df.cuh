@@ -7,7 +7,7 @@
 //               (u_c = sum c_pqr s0^p s1^q s2^r, s = x-hat - 1/2, so
 //               d/dx-hat = d/ds): Horner steps that carry each partial
 //               sum's value and its derivatives along the axes already
-//               passed, in 3D mostly on the field's fixed grid
+//               passed
 //   J           from the cell's monomial block (the map about vertex 0,
 //               Phi = X_0 + sum_k a_k m_k(t)): J_ij = sum_k a_k,i dm_k/dt_j
 //   J^{-1}      cofactors over the determinant, one double-float reciprocal
@@ -38,9 +38,7 @@ __device__ __forceinline__ df df_recip(df a) {
 // s = t - 1/2).  In a slice each row q has its value h = c_0 + s0 (c_1 + s0 c_2)
 // and its derivative along s0, h' = c_1 + 2 c_2 s0; the rows combine along s1
 // to the slice's value g and derivatives g0 (along s0) and g1 = h_1 + 2 h_2 s1;
-// along s2 the slices combine the same way.  As in q2_eval_df the 3D sums
-// without a constant or linear coefficient run on the component's grid: 337
-// operations per component against 564 with plain steps throughout.
+// along s2 the slices combine the same way.
 template <int D>
 __device__ __forceinline__ void q2_grad_mono_df(const float4* __restrict__ Qc, uint32_t K, const df t[D],
                                                 df Gu[D][D]) {
@@ -53,52 +51,31 @@ __device__ __forceinline__ void q2_grad_mono_df(const float4* __restrict__ Qc, u
 #pragma unroll 1
   for (int comp = 0; comp < D; ++comp) {
     const float4* cq = cell + comp * (5 * NS);
-    float hi[10], lo[10];
-    auto plain = [&](int k) { return df_make(hi[k], lo[k]); };
-    if constexpr (D == 2) {
-      load_slice(ld, cq, hi, lo);
+    df g0, g1, g2;  // sums over the slices so far: the derivatives along s0, s1 and s2
+#pragma unroll
+    for (int r = NS - 1; r >= 0; --r) {
+      float hi[10], lo[10];
+      load_slice(ld, cq + 5 * r, hi, lo);
+      auto c = [&](int k) { return df_make(hi[k], lo[k]); };
       df h[3], h0[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        h[q] = df_horner(df_horner(plain(3 * q + 2), s[0], plain(3 * q + 1)), s[0], plain(3 * q));
-        h0[q] = df_horner(df_scale2(plain(3 * q + 2), 2.0f), s[0], plain(3 * q + 1));
+        if (D == 2 || r > 0 || q > 0) h[q] = df_horner(df_horner(c(3 * q + 2), s[0], c(3 * q + 1)), s[0], c(3 * q));
+        h0[q] = df_horner(df_scale2(c(3 * q + 2), 2.0f), s[0], c(3 * q + 1));
       }
-      Gu[comp][0] = df_norm(df_horner(df_horner(h0[2], s[1], h0[1]), s[1], h0[0]));
-      Gu[comp][1] = df_norm(df_horner(df_scale2(h[2], 2.0f), s[1], h[1]));
-    } else {
-      auto grid = [&](int k) { return biased{hi[k], lo[k]}; };
-      auto flat = [&](biased v) { return unbias(v, hi[9]); };
-      auto inner = [&](int q) { return flat(grid_step(plain(3 * q + 2), s[0], grid(3 * q + 1))); };
-      auto value = [&](int q) { return grid_step(inner(q), s[0], grid(3 * q)); };
-      auto deriv = [&](int q) { return grid_step(df_scale2(plain(3 * q + 2), 2.0f), s[0], grid(3 * q + 1)); };
-      df g2, d0, d1;  // sums over the slices r >= 1 so far: the value's 2 g_2 s2, and g0, g1 along s2
-      load_slice(ld, cq + 10, hi, lo);  // r = 2
-      {
-        const df h2 = flat(value(2));
-        const biased h1 = value(1);
-        g2 = flat(grid_step(flat(grid_step(h2, s[1], h1)), s[1], value(0)));
-        d1 = flat(grid_step(df_scale2(h2, 2.0f), s[1], h1));
-        d0 = flat(grid_step(flat(grid_step(flat(deriv(2)), s[1], deriv(1))), s[1], deriv(0)));
-      }
-      load_slice(ld, cq + 5, hi, lo);  // r = 1: row 0 is led by the linear coefficient along s2
-      {
-        const df h2 = flat(value(2));
-        const biased h1 = value(1);
-        const df h0 = df_horner(inner(0), s[0], plain(0));
-        const df g1 = df_horner(flat(grid_step(h2, s[1], h1)), s[1], h0);
-        Gu[comp][2] = df_norm(df_horner(df_scale2(g2, 2.0f), s[2], g1));
-        d1 = flat(grid_step(d1, s[2], grid_step(df_scale2(h2, 2.0f), s[1], h1)));
-        d0 = flat(grid_step(d0, s[2], grid_step(flat(grid_step(flat(deriv(2)), s[1], deriv(1))), s[1], deriv(0))));
-      }
-      load_slice(ld, cq, hi, lo);  // r = 0: the linear coefficients along s0 and s1
-      {
-        const df h1 = df_horner(inner(1), s[0], plain(3));
-        Gu[comp][1] = df_norm(df_horner(d1, s[2], df_horner(df_scale2(flat(value(2)), 2.0f), s[1], h1)));
-        const df h0 = df_horner(df_scale2(plain(2), 2.0f), s[0], plain(1));
-        const df v = flat(grid_step(flat(deriv(2)), s[1], deriv(1)));
-        Gu[comp][0] = df_norm(df_horner(d0, s[2], df_horner(v, s[1], h0)));
+      const df r0 = df_horner(df_horner(h0[2], s[1], h0[1]), s[1], h0[0]);
+      const df r1 = df_horner(df_scale2(h[2], 2.0f), s[1], h[1]);
+      g0 = r == NS - 1 ? r0 : df_horner(g0, s[D - 1], r0);
+      g1 = r == NS - 1 ? r1 : df_horner(g1, s[D - 1], r1);
+      if constexpr (D == 3) {
+        if (r == 0) continue;
+        const df v = df_horner(df_horner(h[2], s[1], h[1]), s[1], h[0]);
+        g2 = r == 2 ? df_scale2(v, 2.0f) : df_horner(g2, s[2], v);
       }
     }
+    Gu[comp][0] = df_norm(g0);
+    Gu[comp][1] = df_norm(g1);
+    if constexpr (D == 3) Gu[comp][2] = df_norm(g2);
   }
 }
 

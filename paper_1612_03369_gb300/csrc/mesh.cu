@@ -139,9 +139,7 @@ __global__ void __launch_bounds__(256) to_df_nodes_kernel(const double* __restri
 // exact; sums and differences carry ~2^-47 of their operands, the order of
 // the storage rounding itself), stored as double-float pairs:
 // per cell and component, slice r (3 in 3D, 1 in 2D) holds C[r][q][p] at
-// pair q*3 + p of 5 float4.  In 3D the coefficients that q2_eval_df adds in
-// grid steps (qc_on_grid) are stored biased by the component's grid bias and
-// the tenth pair holds that bias; in 2D the tenth pair is zero.
+// pair q*3 + p of 5 float4 (the tenth pair is zero).
 __device__ __forceinline__ void t_axis(df v0, df v1, df v2, df& c0, df& c1, df& c2) {
   c0 = v1;
   c1 = df_sub(v2, v0);
@@ -209,37 +207,13 @@ __global__ void __launch_bounds__(32 * D) q2_coeff_kernel(const __grid_constant_
 #pragma unroll
           for (int p = 0; p < 3; ++p) t_axis(V[0][q][p], V[1][q][p], V[2][q][p], V[0][q][p], V[1][q][p], V[2][q][p]);
       }
-      // 3D: the bound of the partial sums of q2_eval_df's grid steps (|s| <= 1/2;
-      // the inner ones without the half, which covers their derivatives)
-      float bias = 0.f;
-      if constexpr (D == 3) {
-        auto A = [&](int p, int q, int r) { return fabsf(V[r][q][p].hi); };
-        float M = A(2, 0, 0), h[3][3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            const float x = (q + r > 0 ? A(1, q, r) : 0.f) + A(2, q, r);
-            h[r][q] = (q + r >= 2 ? A(0, q, r) : 0.f) + 0.5f * x;
-            M = fmaxf(M, q + r >= 2 ? fmaxf(x, h[r][q]) : x);
-          }
-        M = fmaxf(M, fmaxf(h[1][1] + h[1][2], h[2][1] + h[2][2]));
-        M = fmaxf(M, h[2][0] + 0.5f * (h[2][1] + h[2][2]));
-        bias = grid_bias(M);
-      }
       float4* out = sh + (lane * D + comp) * PER;
 #pragma unroll
       for (int r = 0; r < NS; ++r) {
         df pr[10];
 #pragma unroll
-        for (int e = 0; e < 9; ++e) {
-          pr[e] = V[r][e / 3][e % 3];
-          if (D == 3 && qc_on_grid(e % 3, e / 3, r)) {
-            const float b = __fadd_rn(bias, pr[e].hi);
-            pr[e] = df_make(b, __fadd_rn(__fsub_rn(pr[e].hi, __fsub_rn(b, bias)), pr[e].lo));
-          }
-        }
-        pr[9] = df_make(bias, 0.f);
+        for (int e = 0; e < 9; ++e) pr[e] = V[r][e / 3][e % 3];
+        pr[9] = df_make(0.f, 0.f);
         float f[20];  // the ten high parts, then the ten low parts
 #pragma unroll
         for (int e = 0; e < 10; ++e) {

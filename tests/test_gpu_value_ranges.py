@@ -73,3 +73,88 @@ def test_steps_in_cells_of_large_units(P, oracle_mod, n, h):
     parts.advect(wl.dt, 4, 3)
     op = oracle_mod.advect(om, op, wl.dt, 4, 3)
     H.assert_same_store(H.gpu_state(parts), op, wl, tol_x=H.TOL_X * unit.max())
+
+
+def _affine(d, shear):
+    """Rotation times shear: an affine map that leaves a box's cells as well shaped as
+    its singular values, about `shear` and 1 / `shear`."""
+    c, s = np.cos(0.6), np.sin(0.6)
+    A = np.eye(d)
+    A[0, 1] = shear
+    R = np.eye(d)
+    R[:2, :2] = [[c, -s], [s, c]]
+    if d == 3:
+        A[2, 0] = 0.5
+        Q = np.eye(3)
+        Q[1:, 1:] = [[c, -s], [s, c]]
+        R = Q @ R
+    return R @ A
+
+
+def _jacobians(n, X, U, cell, t):
+    """dPhi/dt and du/dt at reference coordinates t [N][d] of cells, in extended precision."""
+    d, L = len(n), np.longdouble
+    t = t.astype(L)
+    lin = [(1 - t, -np.ones_like(t)), (t, np.ones_like(t))]
+    quad = [(2 * (t - L(0.5)) * (t - 1), 4 * t - 3), (4 * t * (1 - t), 4 - 8 * t), (2 * t * (t - L(0.5)), 4 * t - 1)]
+    ijk = np.stack(np.unravel_index(cell, n[::-1])[::-1])
+
+    def deriv(basis, order, values):
+        out = np.zeros((len(cell), d, d), dtype=L)
+        for corner in np.ndindex(*[order + 1] * d):
+            at = np.zeros(len(cell), dtype=np.int64)
+            for a in reversed(range(d)):
+                at = at * (order * n[a] + 1) + order * ijk[a] + corner[a]
+            for j in range(d):
+                w = np.ones(len(cell), dtype=L)
+                for a in range(d):
+                    w = w * basis[corner[a]][1 if a == j else 0][:, a]
+                out[:, :, j] += values[:, at].T * w[:, None]
+        return out
+
+    return deriv(lin, 1, X), deriv(quad, 2, U)
+
+
+def _check_reverse_step(P, n, shear, unit, seeds):
+    """One Euler step: dL/dx0 = lambda + dt J^-T (du/dt)^T lambda at the seeds' own
+    reference coordinates.  Double-float cofactors lose the condition of J times a few
+    2^-47 relative to |J^-1| |du/dt| |lambda|; 60 of them are allowed, and of |lambda|
+    itself its double-float rounding."""
+    import torch
+
+    d = len(n)
+    A = _affine(d, shear) * 2.0**unit
+    g = np.random.default_rng(12)
+    X0 = W.jittered_vertices(n, 4)
+    X = A @ X0
+    # displacements of 0.02 cells a unit time, whatever the cells' shape
+    U = A @ (W.zero_wall_normal(n, g.uniform(-0.02, 0.02, (d, W.q2_node_coords(n, X0).shape[1]))) / np.array(n)[:, None])
+    mesh = P.Mesh(n, X, U)
+    parts = P.Particles(mesh, uniform_count=50, seed=3, n_props=0)
+    st = H.gpu_state(parts)
+    N = st["id"].shape[0]
+    tape = P.pic_advect_record(parts.h, mesh.h, 1.0, 1, 1)
+    ids = H.gpu_state(parts)["id"].astype(np.int64)
+    assert len(ids) > N // 2
+    lam = g.standard_normal((d, N)) * 2.0**seeds
+    dU = torch.empty(U.shape, dtype=torch.float64, device="cuda")
+    dx0 = torch.empty((d, N), dtype=torch.float64, device="cuda")
+    P.pic_tape_adjoint(tape, torch.as_tensor(np.ascontiguousarray(lam[:, ids]), device="cuda"), dU, dx0)
+    P.pic_destroy_tape(tape)
+    J, Gu = _jacobians(n, X, U, st["cell"], st["xhat"])
+    Jf = J.astype(float)
+    inv = np.linalg.inv(Jf).astype(np.longdouble)
+    for _ in range(4):  # to extended precision
+        inv = inv + np.einsum("nij,njk->nik", inv, np.eye(d) - np.einsum("nij,njk->nik", J, inv))
+    lt = lam.T.astype(np.longdouble)
+    want = lt + np.einsum("nij,ni->nj", inv, np.einsum("nij,ni->nj", Gu, lt))
+    size = np.linalg.norm(inv.astype(float), axis=(1, 2)) * np.linalg.norm(Gu.astype(float), axis=(1, 2)) * np.linalg.norm(lam, axis=0)
+    tol = 60 * 2.0**-47 * np.linalg.cond(Jf) * size + 2.0**-46 * np.linalg.norm(lam, axis=0)
+    err = np.abs((dx0.cpu().numpy().T - want).astype(float)).max(axis=1)
+    assert np.all(err[ids] <= tol[ids]), (err[ids] / tol[ids]).max()
+
+
+# nodal values without smoothness: the second and higher coefficients are the largest
+@pytest.mark.parametrize("n", [(6, 5), (4, 3, 4), (2, 2, 2), (7, 2, 3)])
+def test_gradient_of_rough_fields(P, n):
+    _check_reverse_step(P, n, 0.0, 0, 0)
