@@ -168,8 +168,15 @@ __global__ void __launch_bounds__(128, PIC_REVERSE_MIN_BLOCKS) reverse_lambda_ke
         const df w = df_mul(dt, lk[a]);
         rec_w[a * rcap + r] = make_float2(w.hi, w.lo);
       }
-      // G_s^T lambda_k = J^{-T} ((du/dx-hat)^T lambda_k)
+      // G_s^T lambda_k = J^{-T} ((du/dx-hat)^T lambda_k), linear in lambda_k, which
+      // takes whatever scale the loss has: solved for a lambda_k near 1
       df Gu[D][D], v[D], z[D];
+      float largest = 0.f, scale, back;
+#pragma unroll
+      for (int a = 0; a < D; ++a) largest = fmaxf(largest, fabsf(lk[a].hi));
+      pow2_near_one(largest, scale, back);
+#pragma unroll
+      for (int a = 0; a < D; ++a) lk[a] = df_scale2(lk[a], scale);
       q2_grad_mono_df<D>(m.Qc, K, t, Gu);
 #pragma unroll
       for (int q = 0; q < D; ++q) {
@@ -181,7 +188,7 @@ __global__ void __launch_bounds__(128, PIC_REVERSE_MIN_BLOCKS) reverse_lambda_ke
       solve_transposed_df<D>(m, K, t, v, z);
 #pragma unroll
       for (int q = 0; q < D; ++q) {
-        lam_ynext[q] = df_mul(dt, z[q]);
+        lam_ynext[q] = df_mul(dt, df_scale2(z[q], back));
         lam_x[q] = df_add(lam_x[q], lam_ynext[q]);
       }
     }

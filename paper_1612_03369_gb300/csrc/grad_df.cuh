@@ -156,10 +156,38 @@ __device__ __forceinline__ void invert_df(const df J[D][D], df Ji[D][D]) {
   }
 }
 
-// z = J^{-T} v in double-float, J = dPhi/dt at t in cell K: the FP32 adjugate's
+// z = J^{-T} v by double-float cofactors.  Out of line: the cells that
+// solve_transposed_df cannot serve.
+template <int D>
+struct DfVec {
+  df v[D];
+};
+template <int D>
+__device__ __noinline__ DfVec<D> solve_transposed_cofactors_df(const MeshView& m, uint32_t K, DfVec<D> t, DfVec<D> v) {
+  df J[D][D], Ji[D][D];
+  map_jacobian_df<D>(LdgLoader(), m.blk + (size_t)K * block_float4s<D>(), t.v, J);
+  invert_df<D>(J, Ji);
+  DfVec<D> z;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    df_acc acc = acc_zero();
+#pragma unroll
+    for (int j = 0; j < D; ++j) acc_mad(acc, Ji[j][i], v.v[j]);
+    z.v[i] = acc_result(acc);
+  }
+  return z;
+}
+
+// z = J^{-T} v in double-float, J = dPhi/dt at t in cell K: the FP32 inverse's
 // solution and two corrections by the double-float residual v - J^T z, each of
-// which takes the error down by the FP32 inverse's 3e-7 (double-float cofactors
-// and their product with the field's gradient took 660 operations, this 390).
+// which takes the error down by the FP32 inverse's own, some 1e-7 times the
+// condition of J (double-float cofactors and their product with the field's
+// gradient took 660 operations, this 390).  The first correction shows that
+// factor: above 2^-16 of z, where two of them would leave more than the
+// cofactors do (a cell sheared to a condition of a few hundred), and where FP32
+// has no inverse, the cofactors take over.  The inverse's entries, of order
+// 1 / h, multiply the residual; cofactors would take it down by h^(D-1) first.
+// The residuals go down to 2^-48 of v: the caller scales v where it may be small.
 template <int D>
 __device__ __forceinline__ void solve_transposed_df(const MeshView& m, uint32_t K, const df t[D], const df v[D],
                                                     df z[D]) {
@@ -173,32 +201,60 @@ __device__ __forceinline__ void solve_transposed_df(const MeshView& m, uint32_t 
 #pragma unroll
     for (int j = 0; j < D; ++j) J32[i][j] = J[i][j].hi;
   Adjugate32<D> A;
-  if (!adjugate32<D>(J32, A)) A.inv = __int_as_float(0x7fc00000);  // singular: as dividing by it, not a number
+  bool ok = adjugate32<D>(J32, A);
+  if (ok) {
 #pragma unroll
-  for (int i = 0; i < D; ++i) z[i] = df_make(0.f, 0.f);
+    for (int i = 0; i < D; ++i)
 #pragma unroll
-  for (int pass = 0; pass < 3; ++pass) {
-    float r[D];
+      for (int j = 0; j < D; ++j) A.c[i][j] = __fmul_rn(A.c[i][j], A.inv);  // (J^{-T})_ij
 #pragma unroll
-    for (int j = 0; j < D; ++j) {
-      df_acc acc = acc_init(v[j]);
+    for (int i = 0; i < D; ++i) z[i] = df_make(0.f, 0.f);
+#pragma unroll
+    for (int pass = 0; pass < 3; ++pass) {
+      float r[D], first = 0.f, total = 0.f;
+#pragma unroll
+      for (int j = 0; j < D; ++j) {
+        df_acc acc = acc_init(v[j]);
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+          if (pass == 1) acc_mad_f(acc, J[i][j], -z[i].hi);
+          if (pass == 2) acc_mad(acc, J[i][j], df_make(-z[i].hi, -z[i].lo));
+        }
+        r[j] = __fadd_rn(acc.s, acc.e);
+      }
 #pragma unroll
       for (int i = 0; i < D; ++i) {
-        if (pass == 1) acc_mad_f(acc, J[i][j], -z[i].hi);
-        if (pass == 2) acc_mad(acc, J[i][j], df_make(-z[i].hi, -z[i].lo));
+        float q = __fmul_rn(A.c[i][0], r[0]);
+#pragma unroll
+        for (int j = 1; j < D; ++j) q = __fmaf_rn(A.c[i][j], r[j], q);
+        if (pass == 1) {
+          first = __fadd_rn(first, fabsf(q));  // sums: not a number if any is not
+          total = __fadd_rn(total, fabsf(z[i].hi));
+        }
+        z[i] = pass == 0 ? df_make(q, 0.f) : (pass == 1 ? two_sum(z[i].hi, q) : df_add(z[i], df_make(q, 0.f)));
       }
-      r[j] = __fadd_rn(acc.s, acc.e);
-    }
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      // (J^{-T})_ij = c[i][j] inv
-      float q = __fmul_rn(A.c[i][0], r[0]);
-#pragma unroll
-      for (int j = 1; j < D; ++j) q = __fmaf_rn(A.c[i][j], r[j], q);
-      q = __fmul_rn(q, A.inv);
-      z[i] = pass == 0 ? df_make(q, 0.f) : (pass == 1 ? two_sum(z[i].hi, q) : df_add(z[i], df_make(q, 0.f)));
+      if (pass == 1) ok = first <= 0x1p-16f * total;
     }
   }
+  if (!ok) {
+    DfVec<D> tv, vv;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      tv.v[i] = t[i];
+      vv.v[i] = v[i];
+    }
+    const DfVec<D> zv = solve_transposed_cofactors_df<D>(m, K, tv, vv);
+#pragma unroll
+    for (int i = 0; i < D; ++i) z[i] = zv.v[i];
+  }
+}
+
+// A power of two that takes values of magnitude up to `largest` near 1, and its
+// inverse (both normal floats).
+__device__ __forceinline__ void pow2_near_one(float largest, float& scale, float& back) {
+  const int e = min(max(__float_as_int(largest) & 0x7f800000, 1 << 23), 253 << 23);
+  scale = __int_as_float((254 << 23) - e);
+  back = __int_as_float(e);
 }
 
 // G = du_h/dx at double-float reference coordinates t of cell K.

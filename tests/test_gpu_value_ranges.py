@@ -135,7 +135,7 @@ def _check_reverse_step(P, n, shear, unit, seeds):
     N = st["id"].shape[0]
     tape = P.pic_advect_record(parts.h, mesh.h, 1.0, 1, 1)
     ids = H.gpu_state(parts)["id"].astype(np.int64)
-    assert len(ids) > N // 2
+    assert len(ids) > N // 4  # the step may lose particles of the most sheared cells
     lam = g.standard_normal((d, N)) * 2.0**seeds
     dU = torch.empty(U.shape, dtype=torch.float64, device="cuda")
     dx0 = torch.empty((d, N), dtype=torch.float64, device="cuda")
@@ -158,3 +158,11 @@ def _check_reverse_step(P, n, shear, unit, seeds):
 @pytest.mark.parametrize("n", [(6, 5), (4, 3, 4), (2, 2, 2), (7, 2, 3)])
 def test_gradient_of_rough_fields(P, n):
     _check_reverse_step(P, n, 0.0, 0, 0)
+
+
+# J of condition 1 to 4e6, cells and seeds in units far from 1 (powers of two)
+@pytest.mark.parametrize("shear, unit, seeds", [(30.0, 0, 0), (300.0, 0, 0), (2000.0, 0, 0), (0.0, -20, -80), (0.0, -30, 0),
+                                                (30.0, -20, -80), (0.0, 20, 60)])
+@pytest.mark.parametrize("n", [(6, 5), (4, 3, 4)])
+def test_reverse_step_of_scaled_and_sheared_cells(P, n, shear, unit, seeds):
+    _check_reverse_step(P, n, shear, unit, seeds)
