@@ -166,3 +166,25 @@ def test_gradient_of_rough_fields(P, n):
 @pytest.mark.parametrize("n", [(6, 5), (4, 3, 4)])
 def test_reverse_step_of_scaled_and_sheared_cells(P, n, shear, unit, seeds):
     _check_reverse_step(P, n, shear, unit, seeds)
+
+
+# Newton's iterates are affine invariants, so a box and its affine image give every
+# particle the same cells and reference coordinates but for rounding: FP32's, 1e-7
+# times the condition A has, ends the FP32 phase and leaves that part of a last step
+# of 1e-6 at most; ten of these over the four stages
+@pytest.mark.parametrize("shear", [3.0, 10.0, 30.0])
+@pytest.mark.parametrize("n", [(6, 5), (4, 3, 4)])
+def test_steps_in_sheared_cells(P, n, shear):
+    d = len(n)
+    A = _affine(d, shear)
+    X = W.jittered_vertices(n, 4)
+    V = W.zero_wall_normal(n, np.random.default_rng(12).uniform(-0.3, 0.3, (d, W.q2_node_coords(n, X).shape[1]))) / np.array(n)[:, None]
+    got = []
+    for M in (np.eye(d), A):
+        mesh = P.Mesh(n, M @ X, M @ V)
+        parts = P.Particles(mesh, uniform_count=50, seed=3, n_props=0)
+        parts.advect(1.0, 4, 1)
+        got.append(H.gpu_state(parts))
+    np.testing.assert_array_equal(got[1]["id"], got[0]["id"])
+    np.testing.assert_array_equal(got[1]["cell"], got[0]["cell"])
+    assert np.abs(got[1]["xhat"] - got[0]["xhat"]).max() <= 10 * 1e-6 * 1e-7 * np.linalg.cond(A)
