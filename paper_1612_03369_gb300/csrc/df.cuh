@@ -58,6 +58,14 @@ __device__ __forceinline__ df df_add(df a, df b) {
 
 __device__ __forceinline__ df df_sub(df a, df b) { return df_add(a, df_make(-b.hi, -b.lo)); }
 
+// a - b with the low parts' rounding carried too (error <= ~2^-47 |a - b|, also
+// where a and b cancel; df_sub's is relative to |a| + |b|).
+__device__ __forceinline__ df df_sub_accurate(df a, df b) {
+  const df s = two_sum(a.hi, -b.hi), t = two_sum(a.lo, -b.lo);
+  const df u = fast_two_sum(s.hi, __fadd_rn(s.lo, t.hi));
+  return fast_two_sum(u.hi, __fadd_rn(u.lo, t.lo));
+}
+
 // a * b, a and b double-float.
 __device__ __forceinline__ df df_mul(df a, df b) {
   df p = two_prod(a.hi, b.hi);

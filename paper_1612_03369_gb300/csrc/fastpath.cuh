@@ -724,7 +724,9 @@ __device__ __forceinline__ uint32_t locate_df(const Cells& cs, const MeshView& m
   int left = kMaxIt32, hops = 0;
   bool ok = false;
   // to the neighbour across every facet that t32 violates; the offset from its
-  // X_0 by way of the old one's, so that y itself need not be kept
+  // X_0 by the step between the two, so that y itself need not be kept.  Both
+  // differences carry their low parts: added at the size of the coordinates, with
+  // df_add's rounding, two hops left x-hat 1.04 times less exact on 32^2 cells.
   auto hop = [&]() {
     if (hops++ == kPredictedHops) return false;
     flags |= kFlagWalk;
@@ -744,7 +746,7 @@ __device__ __forceinline__ uint32_t locate_df(const Cells& cs, const MeshView& m
     K = cell_index<D>(m, c[0] + pred[0], c[1] + pred[1], c[2] + pred[2]);
     cell_origin_df<D>(cs, cs.block(K), x1);
 #pragma unroll
-    for (int a = 0; a < D; ++a) dloc[a] = df_sub(df_add(dloc[a], x0[a]), x1[a]);
+    for (int a = 0; a < D; ++a) dloc[a] = df_sub_accurate(dloc[a], df_sub_accurate(x1[a], x0[a]));
     left = kMaxIt32 - 1;
     return true;
   };

@@ -188,3 +188,24 @@ def test_steps_in_sheared_cells(P, n, shear):
     np.testing.assert_array_equal(got[1]["id"], got[0]["id"])
     np.testing.assert_array_equal(got[1]["cell"], got[0]["cell"])
     assert np.abs(got[1]["xhat"] - got[0]["xhat"]).max() <= 10 * 1e-6 * 1e-7 * np.linalg.cond(A)
+
+
+# Translation across undistorted cells: x-hat follows from the position exactly.  What
+# may remain is the rounding of the position and of its offset from a vertex to 48
+# bits, 2^-48 of a coordinate of at most 1 each, in cells; crossing cells adds nothing
+# of that size.
+@pytest.mark.parametrize("cells", [0.3, 0.8, 1.6])
+def test_reference_coordinates_after_crossing_cells(P, cells):
+    n = (250, 2)  # vertices that are no double-floats
+    X = W.uniform_vertices(n)
+    U = np.zeros((2, W.q2_node_coords(n, X).shape[1]))
+    U[0] = 1.0
+    mesh = P.Mesh(n, X, U)
+    parts = P.Particles(mesh, uniform_count=2000, seed=3, n_props=0)
+    parts.advect(cells / n[0], 1, 1)
+    s = H.gpu_state(parts)
+    i = s["cell"] % n[0]
+    assert len(i) > 900000
+    x, v = s["x"][:, 0].astype(np.longdouble), X[0, : n[0] + 1].astype(np.longdouble)
+    t = (x - v[i]) / (v[i + 1] - v[i])
+    assert np.abs(s["xhat"][:, 0] - t).max() <= 2 * n[0] * 2.0**-48
