@@ -44,14 +44,18 @@ namespace pic {
 constexpr float kSettle32 = 2e-4f;
 constexpr int kMaxIt32 = 8;
 // Ends the FP32 phase after a step with the second-order term q: the error
-// left, ~2 |q|^2 / |d|, is then below 2e-7, the FP32 residual's own noise.
-constexpr float kSettleCheb32 = 1e-7f;
+// left, ~2 |q|^2 / |d|, is then below 2e-9, well under the FP32 residual's own noise
+// of ~1e-7.  (At a hundred times that, and kFinish32 at 1e-6, it showed: x of 6^3 cells
+// 2.44e-16 rms off instead of 2.2e-16, dL/dU of 4^3 1.71e-15 instead of 1.5e-15, for
+// no gain in time.)
+constexpr float kSettleCheb32 = 1e-9f;
 // A settled FP32 iterate this far outside [0,1] is still taken to the
 // double-float step, which decides (the two differ by a few 1e-7).
 constexpr float kInside32 = 5e-7f;
 // Largest double-float step after which the root is taken as found: the FP32
-// Jacobian leaves ~3e-7 of the step.
-constexpr float kFinish32 = 1e-6f;
+// Jacobian leaves ~3e-7 of the step (at 2e-7 the FP32 phase's noise alone has it
+// repeated: 2 % of the 64^3 step).
+constexpr float kFinish32 = 4e-7f;
 // Largest first double-float step of a root that is taken further: the FP32
 // iterate is off by ~1e-7 times the condition of the Jacobian (~1e-7 in cells
 // jittered by 10 %, 1e-4 in ones sheared 30 to 1).

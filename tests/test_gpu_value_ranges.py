@@ -209,3 +209,28 @@ def test_reference_coordinates_after_crossing_cells(P, cells):
     x, v = s["x"][:, 0].astype(np.longdouble), X[0, : n[0] + 1].astype(np.longdouble)
     t = (x - v[i]) / (v[i + 1] - v[i])
     assert np.abs(s["xhat"][:, 0] - t).max() <= 2 * n[0] * 2.0**-48
+
+
+# The FP32 phase ends with its residual's noise, ~1.5e-7, whatever the length of the
+# last step; the FP32 Jacobian, off by 3e-7 times a condition of 2 here, leaves
+# 9e-14 of that, and the position's 48 bits 1e-14.
+@pytest.mark.parametrize("amplitude", [0.05, 0.1, 0.3])
+@pytest.mark.parametrize("n", [(2, 2), (3, 3)])
+def test_end_of_the_inverse_map(P, n, amplitude):
+    X = W.jittered_vertices(n, 4, 0.25)
+    nodes = W.q2_node_coords(n, X).shape[1]
+    U = W.zero_wall_normal(n, np.random.default_rng(4).uniform(-amplitude, amplitude, (2, nodes))) / np.array(n)[:, None]
+    mesh = P.Mesh(n, X, U)
+    parts = P.Particles(mesh, uniform_count=8000, seed=4, n_props=0)
+    parts.advect(1.0, 1, 1)
+    s = H.gpu_state(parts)
+    i, j = s["cell"] % n[0], s["cell"] // n[0]
+    V = [X[:, (i + a) + (n[0] + 1) * (j + b)] for b in (0, 1) for a in (0, 1)]
+    t = s["xhat"].copy()
+    for _ in range(3):  # Newton in FP64 from the result
+        a, b = t.T
+        r = s["x"].T - (V[0] + (V[1] - V[0]) * a + (V[2] - V[0]) * b + (V[3] - V[2] - V[1] + V[0]) * a * b)
+        J0, J1 = (V[1] - V[0]) * (1 - b) + (V[3] - V[2]) * b, (V[2] - V[0]) * (1 - a) + (V[3] - V[1]) * a
+        det = J0[0] * J1[1] - J0[1] * J1[0]
+        t = t + np.stack([(r[0] * J1[1] - r[1] * J1[0]) / det, (J0[0] * r[1] - J0[1] * r[0]) / det], axis=1)
+    assert np.abs(s["xhat"] - t).max() <= 1e-13
