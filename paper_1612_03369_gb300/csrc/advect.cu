@@ -351,7 +351,7 @@ __device__ __forceinline__ bool polish_fp64(const MeshView& m, uint32_t K, const
 // point's cell in a uniform background grid over the mesh's bounding box.
 // The search runs on the FP32 / double-float fast path, and the reference
 // coordinates it finds are taken to FP64 by one residual in FP64; a point that
-// the fast path leaves, or that lies within kTieBandFast of a facet (where the
+// the fast path leaves, or that lies within the mesh's band of a facet (where the
 // lowest-index rule compares FP64 coordinates with the eps band), is located
 // in FP64 throughout (at kTieBand a dozen of those held the launch up by 0.3 ms).  All points in FP64 throughout took 6.3 ms for 1.77 M
 // points (48^3 cells), the FP64 pipe's ~2000 operations per point.
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(128) locate_points_kernel(const __grid_constan
         for (int a = 0; a < D; ++a) t[a] = df_to_double(td[a]);
         done = polish_fp64<D>(m, K, y, t);
 #pragma unroll
-        for (int a = 0; a < D; ++a) done = done && t[a] > (double)kTieBandFast && t[a] < 1.0 - (double)kTieBandFast;
+        for (int a = 0; a < D; ++a) done = done && t[a] > (double)m.tie_band && t[a] < 1.0 - (double)m.tie_band;
       }
     }
     if (!done) {

@@ -526,12 +526,17 @@ __device__ __noinline__ RarePath<D> lowest_owner_df_slow(const MeshView& m, DfPt
 }
 
 //
-// The fast path leaves a particle to the full step only within kTieBandFast of
-// a facet: a redone particle holds its warp up by several times a step's
-// latency, which a small store sees whole.  Reference coordinates at hand are
-// good to ~1e-12 (accurate == true), so a cell across the facet can hold the
-// point within kInsideEps only if it is a thousand times longer than this one.
+// The fast path leaves a particle to the full step only within the mesh's band
+// of a facet: a redone particle holds its warp up by several times a step's
+// latency, which a small store sees whole.  A cell across the facet holds the
+// point within kInsideEps only if the point is that part of the cell's size away,
+// in units of this one: no more than kInsideEps sqrt(D) times the largest |J| of
+// the mesh times the largest |J^-1|, which the set-up takes at the cells' corners.
+// Where that product is at most kTieRatio it makes 4.5e-8, and kTieBandFast, more
+// than twice that, is enough (reference coordinates at hand are good to ~1e-12,
+// accurate == true); meshes of more uneven cells keep kTieBand.
 constexpr float kTieBandFast = 1e-7f;
+constexpr double kTieRatio = 256.0;
 
 template <int D, bool kFast = false>
 __device__ __forceinline__ uint32_t lowest_owner_df(const MeshView& m, const df y[D], uint32_t found, df t[D],
@@ -539,7 +544,7 @@ __device__ __forceinline__ uint32_t lowest_owner_df(const MeshView& m, const df 
   // band test first (cheap); the cell's (i,j,k) only when some coordinate is
   // near a facet
   bool near = false;
-  const float band = accurate ? kTieBandFast : (float)kTieBand;
+  const float band = accurate ? m.tie_band : (float)kTieBand;
 #pragma unroll
   for (int a = 0; a < D; ++a) {
     if (accurate)

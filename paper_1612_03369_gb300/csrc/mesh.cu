@@ -27,9 +27,11 @@ __device__ __forceinline__ float widen_up(double v) {
   return f;
 }
 
+// Also clears the two words at shape for cell_block_kernel.
 template <int D>
 __global__ void cell_bbox_kernel(const __grid_constant__ MeshView m, double* __restrict__ bbox,
-                                 float4* __restrict__ bbox32) {
+                                 float4* __restrict__ bbox32, unsigned int* __restrict__ shape) {
+  if (blockIdx.x == 0 && threadIdx.x < 2) shape[threadIdx.x] = 0u;
   for (uint32_t K = blockIdx.x * blockDim.x + threadIdx.x; K < m.C; K += gridDim.x * blockDim.x) {
     CellGeom<D> g;
     load_cell<D>(m, K, g);
@@ -70,8 +72,12 @@ __device__ __forceinline__ float2 split_df(double v) {
 // Stored as one row (X_0, a_1, a_2, ...) per component, the high parts of every
 // row and then the low parts, so that the FP32 Newton iterations read only the
 // first half and take a component at a time.
+// shape[0] and shape[1] become the largest |J| and |J^-1| (Frobenius) over the
+// corners of every cell; infinite where FP32 has no inverse.
 template <int D>
-__global__ void cell_block_kernel(const __grid_constant__ MeshView m, float* __restrict__ blk) {
+__global__ void cell_block_kernel(const __grid_constant__ MeshView m, float* __restrict__ blk,
+                                  unsigned int* __restrict__ shape) {
+  float size = 0.f, inverse = 0.f;
   constexpr int NK = (1 << D) - 1;
   constexpr int NF = D + NK * D;
   for (uint32_t K = blockIdx.x * blockDim.x + threadIdx.x; K < m.C; K += gridDim.x * blockDim.x) {
@@ -84,6 +90,8 @@ __global__ void cell_block_kernel(const __grid_constant__ MeshView m, float* __r
       out[NF + idx] = p.y;
     };
     for (int a = 0; a < D; ++a) put(a * (NK + 1), g.x0[a]);
+    MapRow<D> row[D];
+#pragma unroll
     for (int a = 0; a < D; ++a) {
       double coef[NK];
       if constexpr (D == 2) {
@@ -99,8 +107,40 @@ __global__ void cell_block_kernel(const __grid_constant__ MeshView m, float* __r
         coef[5] = g.e[6][a] - g.e[2][a] - g.e[4][a];
         coef[6] = g.e[7][a] - g.e[3][a] - g.e[5][a] - g.e[6][a] + g.e[1][a] + g.e[2][a] + g.e[4][a];
       }
-      for (int k = 0; k < NK; ++k) put(a * (NK + 1) + 1 + k, coef[k]);
+#pragma unroll
+      for (int k = 0; k < NK; ++k) {
+        put(a * (NK + 1) + 1 + k, coef[k]);
+        row[a].a[k] = (float)coef[k];
+      }
     }
+#pragma unroll 1
+    for (int corner = 0; corner < (1 << D); ++corner) {
+      float t[D], mixed[4], J[D][D], j2 = 0.f, c2 = 0.f;
+      Adjugate32<D> A;
+#pragma unroll
+      for (int a = 0; a < D; ++a) t[a] = (float)((corner >> a) & 1);
+      mixed32<D>(t, mixed);
+#pragma unroll
+      for (int a = 0; a < D; ++a) jacobian_row32<D>(row[a], t, mixed, J[a]);
+      const bool regular = adjugate32<D>(J, A);
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int b = 0; b < D; ++b) {
+          j2 += J[a][b] * J[a][b];
+          c2 += A.c[a][b] * A.c[a][b];
+        }
+      const float si = sqrtf(j2), ii = sqrtf(c2) * fabsf(A.inv);
+      size = fmaxf(size, si <= 0x1p126f ? si : INFINITY);
+      inverse = fmaxf(inverse, regular && c2 >= 0x1p-126f && ii <= 0x1p126f ? ii : INFINITY);
+    }
+  }
+  // positive floats order as their bits do
+  const unsigned int s = __reduce_max_sync(0xffffffffu, __float_as_uint(size));
+  const unsigned int i = __reduce_max_sync(0xffffffffu, __float_as_uint(inverse));
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(shape, s);
+    atomicMax(shape + 1, i);
   }
 }
 
@@ -341,7 +381,7 @@ extern "C" pic_status pic_create_mesh(int dim, const int* n_cells, const double*
       cudaMalloc(&m->bbox, sizeof(double) * 6 * C) != cudaSuccess ||
       cudaMalloc(&m->bbox32, sizeof(float4) * 2 * C) != cudaSuccess ||
       cudaMalloc(&m->blk, sizeof(float4) * blk_f4 * C) != cudaSuccess ||
-      cudaMalloc(&m->qbase, sizeof(uint32_t) * C) != cudaSuccess) {
+      cudaMalloc(&m->qbase, sizeof(uint32_t) * (C > 2 ? C : 2)) != cudaSuccess) {
     cudaGetLastError();
     set_error("pic_create_mesh: device allocation failed");
     return fail(PIC_ERR_OOM);
@@ -376,18 +416,27 @@ extern "C" pic_status pic_create_mesh(int dim, const int* n_cells, const double*
   }
   const MeshView mv = mesh_view(m);
   const int grid = (int)((C + 255) / 256 < 4096 ? (C + 255) / 256 : 4096);
+  unsigned int* shape = m->qbase;  // its first two words, until they are filled
   if (dim == 2) {
-    cell_bbox_kernel<2><<<grid, 256, 0, st>>>(mv, m->bbox, m->bbox32);
-    cell_block_kernel<2><<<grid, 256, 0, st>>>(mv, (float*)m->blk);
-    cell_qbase_kernel<2><<<grid, 256, 0, st>>>(mv, m->qbase);
+    cell_bbox_kernel<2><<<grid, 256, 0, st>>>(mv, m->bbox, m->bbox32, shape);
+    cell_block_kernel<2><<<grid, 256, 0, st>>>(mv, (float*)m->blk, shape);
   } else {
-    cell_bbox_kernel<3><<<grid, 256, 0, st>>>(mv, m->bbox, m->bbox32);
-    cell_block_kernel<3><<<grid, 256, 0, st>>>(mv, (float*)m->blk);
-    cell_qbase_kernel<3><<<grid, 256, 0, st>>>(mv, m->qbase);
+    cell_bbox_kernel<3><<<grid, 256, 0, st>>>(mv, m->bbox, m->bbox32, shape);
+    cell_block_kernel<3><<<grid, 256, 0, st>>>(mv, (float*)m->blk, shape);
   }
+  float norms[2] = {INFINITY, INFINITY};
   e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(norms, shape, sizeof(norms), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) {
+    if (dim == 2)
+      cell_qbase_kernel<2><<<grid, 256, 0, st>>>(mv, m->qbase);
+    else
+      cell_qbase_kernel<3><<<grid, 256, 0, st>>>(mv, m->qbase);
+    e = cudaGetLastError();
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(cuda_fail(e, "pic_create_mesh: set-up kernels"));
+  m->tie_band = (double)norms[0] * (double)norms[1] <= kTieRatio ? kTieBandFast : (float)kTieBand;
   *out = m;
   return PIC_OK;
 }

@@ -114,6 +114,7 @@ struct pic_mesh_s {
   float4* Qfn;   // the same for the field at the end of the step
   int has_next;
   double dlo[3], dhi[3];  // padded domain bounding box
+  float tie_band;         // the fast path's band of the lowest-index rule (see fastpath.cuh)
   int has_velocity;
   // staged upload of the next field (pic_stage_velocity_dofs): FP64 buffer,
   // "copy done" and "buffer free" events, created on first use
@@ -212,6 +213,7 @@ struct MeshView {
   int has_next;
   int stage_df;  // FP32-basis form: stage points too take the double-float Newton step (set per pic_advect call)
   double dlo[3], dhi[3];
+  float tie_band;
 };
 
 inline MeshView mesh_view(const pic_mesh_s* m) {
@@ -225,6 +227,7 @@ inline MeshView mesh_view(const pic_mesh_s* m) {
   }
   v.div[0] = fast_div((uint32_t)m->n[0]);
   v.div[1] = fast_div((uint32_t)m->n[1]);
+  v.tie_band = m->tie_band;
   v.C = m->C;
   v.nverts = m->nverts;
   v.nnodes = m->nnodes;

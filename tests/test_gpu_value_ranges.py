@@ -234,3 +234,41 @@ def test_end_of_the_inverse_map(P, n, amplitude):
         det = J0[0] * J1[1] - J0[1] * J1[0]
         t = t + np.stack([(r[0] * J1[1] - r[1] * J1[0]) / det, (J0[0] * r[1] - J0[1] * r[0]) / det], axis=1)
     assert np.abs(s["xhat"] - t).max() <= 1e-13
+
+
+# A cell 2,000 or 8,000 times as long as its neighbour holds points, within its 1e-10
+# band, up to 2e-7 and 8e-7 of the neighbour's size into it: the lowest index decides.
+@pytest.mark.parametrize("step", [False, True])
+@pytest.mark.parametrize("ratio", [10.0, 2000.0, 8000.0])
+@pytest.mark.parametrize("d", [2, 3])
+def test_lowest_owner_among_uneven_cells(P, oracle_mod, d, ratio, step):
+    import torch
+
+    widths = [ratio, 1.0, 2.0, 0.5 * ratio]
+    lines = np.concatenate([[0.0], np.cumsum(widths)])
+    n = (4,) * d
+    X = np.stack([g.ravel() for g in np.meshgrid(*[lines] * d, indexing="ij")][::-1])
+    shift = 0.25 if step else 0.0
+    pts = []
+    for delta in np.array([-1.5, -0.9, -0.5, 0.5, 0.9, 1.5]) * 1e-10 * ratio:
+        for a in range(d):
+            for facet in lines[1:4]:
+                p = np.full(d, ratio + 0.4)
+                p[a] = facet + delta + shift
+                pts.append(p)
+    pts = np.array(pts)
+    U = np.full((d, W.q2_node_coords(n, X).shape[1]), -1.0)
+    mesh, om = P.Mesh(n, X, U), oracle_mod.Mesh(n, X, U)
+    if not step:
+        got = mesh.locate_points(torch.as_tensor(np.ascontiguousarray(pts.T), device="cuda"))[0].cpu().numpy()
+        np.testing.assert_array_equal(got.view(np.uint32).astype(np.int64), om.locate(pts)[0])
+        return
+    parts, outside = P.Particles.import_points(mesh, torch.as_tensor(np.ascontiguousarray(pts.T), device="cuda"))
+    c, t = om.locate(pts)
+    o = np.argsort(c, kind="stable")
+    op = oracle_mod.Particles(pts[o], t[o], c[o], o.astype(np.uint64), np.zeros((len(o), 0)))
+    parts.advect(shift, 1, 1)
+    op = oracle_mod.advect(om, op, shift, 1, 1)
+    s = H.gpu_state(parts)
+    np.testing.assert_array_equal(s["id"], op.id)
+    np.testing.assert_array_equal(s["cell"], op.cell)
