@@ -436,9 +436,12 @@ pic_status pic_interpolate_to_cells(pic_particles parts, pic_mesh mesh, int prop
  * over the particles i of the cells around vertex v, phi_v the (bi/tri)linear
  * nodal basis function of v (in a particle's cell: the map weight of v's
  * corner at the stored x-hat).  Each cell's particles are summed in store
- * order, then the cells' sums in increasing cell index (deterministic).  The
- * value at a quadrature point is the Q1 interpolation of avg.  The first
- * call allocates 2^(dim+4) bytes per cell of scratch, kept with the store.
+ * order, or its 1st, 5th, ..., 2nd, 6th, ... and so on in store order and these
+ * four sums added (where one of the 32 cells 32 k .. 32 k + 31 around it holds
+ * more than 14); then the cells' sums in increasing cell index.  The sums are a
+ * function of the particles and the mesh alone (deterministic).  The value at a
+ * quadrature point is the Q1 interpolation of avg.  The first call allocates
+ * 2^(dim+4) bytes per cell of scratch, kept with the store.
  *   avg     [nverts] FP64 device, vertex (i,j,k) at i + (n0+1)(j + (n1+1)k)
  *   weight  [nverts] FP64 device, the sum of the weights, or NULL
  * A vertex whose weights sum to 0 gets empty_fill.
@@ -450,7 +453,7 @@ pic_status pic_interpolate_to_vertices(pic_particles parts, pic_mesh mesh, int p
  * least-squares fit in reference coordinates,
  *   f(x-hat) = c_0 + sum_j c_{j+1} (x-hat_j - 1/2)
  * minimising sum over the cell's particles of (f(x-hat_i) - p_i)^2.  Solved
- * from the normal equations (folded in a fixed order) by Gaussian elimination
+ * from the normal equations (folded in store order) by Gaussian elimination
  * with partial pivoting.  A cell with at most dim particles, or a pivot
  * <= 1e-12 times the largest diagonal entry, gets the mean (c_0 = mean,
  * slopes 0); an empty cell gets c_0 = empty_fill.

@@ -8,9 +8,9 @@
 //        f(x-hat) = c_0 + sum_j c_{j+1} (x-hat_j - 1/2)
 // No atomics, so the results are reproducible run to run.  The linear fit folds a
 // cell's particles in store order.  The vertex sums are formed per cell first (one
-// left fold, or four strided ones added in a fixed pattern) and the cells' partial
-// sums then added in increasing cell index, which rounds differently from one left
-// fold over the support (the definition) by a few ulps of the sum.
+// left fold, or four strided ones added in a fixed pattern, by the cells' counts) and
+// the cells' partial sums then added in increasing cell index, which rounds differently
+// from one left fold over the support (the definition) by a few ulps of the sum.
 #include "df.cuh"
 #include "pic_internal.cuh"
 
@@ -32,17 +32,21 @@ __device__ __forceinline__ df minus_half(df t) {  // t - 1/2
 }
 __device__ __forceinline__ double df_to_f64(df a) { return (double)a.hi + (double)a.lo; }
 
-// In the vertex sums kLanes neighbouring lanes share a cell, lane q folding its
-// particles q, q + kLanes, ..., and the lanes' compensated sums are then added in a
-// fixed pattern of exchanges.  The lanes' loads are consecutive, a 32-byte sector
-// per cell and array: with a thread per cell every load of a warp touches 32 sectors
-// of as many lines.  The call (with the vertices' pass and the launches) takes 92 us
-// for 113 at 64^3 x 20, 141 for 180 at 36 per cell, 175 for 283 at 8 per cell unevenly
-// filled, 623 for 686 at 128^3.  At 4 per cell the exchanges cost more than the
-// loads (43 us for 32), so below kSharedFrom particles of capacity per cell a
-// thread takes a cell.
+// In the vertex sums a cell is taken by one lane or by kLanes neighbouring ones,
+// lane q then folding its particles q, q + kLanes, ..., and the lanes' compensated
+// sums are added in a fixed pattern of exchanges.  Shared, the lanes' loads are
+// consecutive, a 32-byte sector per cell and array, and a long cell holds its warp
+// up a quarter as long; alone, every load of a warp touches 32 sectors of as many
+// lines, but there are no exchanges.  The choice falls for 32 cells at a time, by the
+// largest of them, so that the order of the sums is a function of the store's
+// particles and the mesh (chosen by the store's capacity, two stores of the same
+// particles differed in the last bits).  64^3 cells, the call with the vertices' pass
+// and the launches, all alone / all shared: 6 per cell 61 / 78 us, 10 77 / 91, 14 94 /
+// 102, 16 134 / 102, 36 197 / 164; unevenly filled, 4.9 per cell on average and up to 48
+// in one, 135 / 107, 13 297 / 199; 500^2 cells cross at 13 per cell.  This rule: 65, 79,
+// 93, 103, 164; 111, 211.
 constexpr int kLanes = 4;
-constexpr size_t kSharedFrom = 6;
+constexpr uint32_t kAloneUpTo = 14;
 
 // The group's sums, dealt to its lanes: own[j] of lane q becomes the sum over the
 // group of acc[kLanes j + q].  Each round halves what a lane holds, so an entry
@@ -80,14 +84,13 @@ struct ParticleLoads {
   }
 };
 
-// The cell of a lane's group and its particles; a segment outside the store is
+// A cell's particles (none past the last cell); a segment outside the store is
 // flagged and taken as empty.
-__device__ __forceinline__ void group_cell(const uint32_t* __restrict__ cell_off, uint32_t K, uint32_t C, size_t cap,
-                                           uint32_t& beg, uint32_t& end, bool& bad, DevCounters* __restrict__ ctr) {
+__device__ __forceinline__ void cell_segment(const uint32_t* __restrict__ cell_off, uint32_t K, uint32_t C, size_t cap,
+                                             uint32_t& beg, uint32_t& end, DevCounters* __restrict__ ctr) {
   beg = K < C ? cell_off[K] : 0u;
   end = K < C ? cell_off[K + 1] : 0u;
-  bad = end > cap || beg > end;
-  if (bad) {
+  if (end > cap || beg > end) {
     latch_status(ctr, PIC_STATUS_BOUNDS);
     beg = end = 0;
   }
@@ -101,62 +104,79 @@ __device__ __forceinline__ void group_cell(const uint32_t* __restrict__ cell_off
 // stored as double-float pairs, corner-major ([c][C]) so that the phase-2
 // reads of a warp coalesce.
 template <int D, int L>
+__device__ __forceinline__ void vertex_partial_sums(uint32_t K, uint32_t beg, uint32_t end, uint32_t q,
+                                                    const float2* __restrict__ xh, const double* __restrict__ prop,
+                                                    uint32_t C, size_t cap, float2* __restrict__ part) {
+  constexpr int NC = 1 << D;
+  df_acc num[NC], den[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) num[c] = den[c] = acc_zero();
+  ParticleLoads<D> next;
+  next.load(xh, prop, cap, beg + q, end);
+  for (uint32_t i = beg + q; i < end; i += L) {
+    const ParticleLoads<D> now = next;
+    next.load(xh, prop, cap, i + L, end);
+    df f[D][2];  // f[a][0] = 1 - t_a, f[a][1] = t_a
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      f[a][1] = df_make(now.t[a].x, now.t[a].y);
+      f[a][0] = one_minus(f[a][1]);
+    }
+    const df p = split_f64(now.p);
+    df w01[4];  // the first two axes' products, corner bits 0 and 1
+#pragma unroll
+    for (int c = 0; c < 4; ++c) w01[c] = df_mul(f[0][c & 1], f[1][(c >> 1) & 1]);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const df w = D == 3 ? df_mul(w01[c & 3], f[D - 1][(c >> 2) & 1]) : w01[c];
+      acc_mad(num[c], w, p);
+      acc_add(den[c], w);
+    }
+  }
+  df_acc num_q[NC / L], den_q[NC / L];
+  if constexpr (L == 1) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      num_q[c] = num[c];
+      den_q[c] = den[c];
+    }
+  } else {
+    group_sums(num, num_q, q);
+    group_sums(den, den_q, q);
+  }
+  if (K < C)
+#pragma unroll
+    for (int j = 0; j < NC / L; ++j) {
+      const size_t c = (size_t)(L * j) + q;
+      const df a = acc_result(num_q[j]), b = acc_result(den_q[j]);
+      part[c * C + K] = make_float2(a.hi, a.lo);
+      part[(NC + c) * C + K] = make_float2(b.hi, b.lo);
+    }
+}
+
+// A block takes `per_block` (1 or 4) groups of 32 cells at a time: alone, one of its
+// warps takes a group; shared, every warp eight of the group's cells.
+template <int D>
 __global__ void __launch_bounds__(128) vertex_partial_kernel(const uint32_t* __restrict__ cell_off,
                                                              const float2* __restrict__ xh, const double* __restrict__ prop,
-                                                             uint32_t C, size_t cap, float2* __restrict__ part,
-                                                             DevCounters* __restrict__ ctr) {
-  constexpr int NC = 1 << D;
-  constexpr uint32_t kCells = 128 / L;  // per block and pass
-  const uint32_t q = threadIdx.x % L;
-  for (uint32_t K0 = blockIdx.x * kCells; K0 < C; K0 += gridDim.x * kCells) {
-    const uint32_t K = K0 + threadIdx.x / L;
-    uint32_t beg, end;
-    bool bad;
-    group_cell(cell_off, K, C, cap, beg, end, bad, ctr);
-    df_acc num[NC], den[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) num[c] = den[c] = acc_zero();
-    ParticleLoads<D> next;
-    next.load(xh, prop, cap, beg + q, end);
-    for (uint32_t i = beg + q; i < end; i += L) {
-      const ParticleLoads<D> now = next;
-      next.load(xh, prop, cap, i + L, end);
-      df f[D][2];  // f[a][0] = 1 - t_a, f[a][1] = t_a
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        f[a][1] = df_make(now.t[a].x, now.t[a].y);
-        f[a][0] = one_minus(f[a][1]);
-      }
-      const df p = split_f64(now.p);
-      df w01[4];  // the first two axes' products, corner bits 0 and 1
-#pragma unroll
-      for (int c = 0; c < 4; ++c) w01[c] = df_mul(f[0][c & 1], f[1][(c >> 1) & 1]);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const df w = D == 3 ? df_mul(w01[c & 3], f[D - 1][(c >> 2) & 1]) : w01[c];
-        acc_mad(num[c], w, p);
-        acc_add(den[c], w);
+                                                             uint32_t C, size_t cap, uint32_t per_block,
+                                                             float2* __restrict__ part, DevCounters* __restrict__ ctr) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t groups = (C + 31u) / 32u;
+  for (uint32_t g0 = blockIdx.x * per_block; g0 < groups; g0 += gridDim.x * per_block) {
+    for (uint32_t g = 0; g < per_block && g0 + g < groups; ++g) {
+      const uint32_t K0 = (g0 + g) * 32u;
+      uint32_t beg, end;
+      cell_segment(cell_off, K0 + lane, C, cap, beg, end, ctr);
+      if (__reduce_max_sync(0xffffffffu, end - beg) <= kAloneUpTo) {
+        if (warp == g) vertex_partial_sums<D, 1>(K0 + lane, beg, end, 0u, xh, prop, C, cap, part);
+      } else {
+        const uint32_t k = warp * (32 / kLanes) + lane / kLanes;
+        beg = __shfl_sync(0xffffffffu, beg, k);
+        end = __shfl_sync(0xffffffffu, end, k);
+        vertex_partial_sums<D, kLanes>(K0 + k, beg, end, lane % kLanes, xh, prop, C, cap, part);
       }
     }
-    df_acc num_q[NC / L], den_q[NC / L];
-    if constexpr (L == 1) {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        num_q[c] = num[c];
-        den_q[c] = den[c];
-      }
-    } else {
-      group_sums(num, num_q, q);
-      group_sums(den, den_q, q);
-    }
-    if (K < C)
-#pragma unroll
-      for (int j = 0; j < NC / L; ++j) {
-        const size_t c = (size_t)(L * j) + q;
-        const df a = acc_result(num_q[j]), b = acc_result(den_q[j]);
-        part[c * C + K] = make_float2(a.hi, a.lo);
-        part[(NC + c) * C + K] = make_float2(b.hi, b.lo);
-      }
   }
 }
 
@@ -362,16 +382,21 @@ extern "C" pic_status pic_interpolate_to_vertices(pic_particles p, pic_mesh mesh
     }
   }
   const double* pv = p->props[p->cur] + (size_t)prop * p->capacity;
-  const bool shared = p->capacity >= kSharedFrom * p->C;
-  const int g1 = transfer_grid((size_t)p->C * (shared ? kLanes : 1), 128), g2 = transfer_grid((size_t)m.nverts, 256);
+  // four groups per block where that leaves every SM its blocks and groups may be taken
+  // alone, so that each warp has one (64^3 x 12: 86 us, 101 with one group per block);
+  // otherwise one, as shared groups are 2 to 5 % faster that way.  Only the time depends
+  // on it.
+  const size_t groups = ((size_t)p->C + 31) / 32;
+  const uint32_t per_block = groups >= (size_t)num_sms() * 16 && p->capacity < (size_t)p->C * (kAloneUpTo + 1) ? 4u : 1u;
+  const int g1 = transfer_grid((groups + per_block - 1) / per_block * 128, 128), g2 = transfer_grid((size_t)m.nverts, 256);
   float2* part = reinterpret_cast<float2*>(p->xfer);  // [2 * 2^dim][C] double-float pairs
   if (mesh->dim == 2) {
-    auto partial = shared ? vertex_partial_kernel<2, kLanes> : vertex_partial_kernel<2, 1>;
-    partial<<<g1, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, part, p->ctr);
+    vertex_partial_kernel<2><<<g1, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, per_block, part,
+                                                  p->ctr);
     vertex_gather_kernel<2><<<g2, 256, 0, st>>>(m, part, empty_fill, avg, weight);
   } else {
-    auto partial = shared ? vertex_partial_kernel<3, kLanes> : vertex_partial_kernel<3, 1>;
-    partial<<<g1, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, part, p->ctr);
+    vertex_partial_kernel<3><<<g1, 128, 0, st>>>(p->cell_off, p->xhat[p->cur], pv, p->C, p->capacity, per_block, part,
+                                                  p->ctr);
     vertex_gather_kernel<3><<<g2, 256, 0, st>>>(m, part, empty_fill, avg, weight);
   }
   count_launches(2);

@@ -7,6 +7,7 @@ import pytest
 
 from paper_1612_03369_gb300 import workloads as W
 import gpu_helpers as H
+import test_gpu_transfer as T
 
 pytestmark = pytest.mark.gpu
 
@@ -272,3 +273,36 @@ def test_lowest_owner_among_uneven_cells(P, oracle_mod, d, ratio, step):
     s = H.gpu_state(parts)
     np.testing.assert_array_equal(s["id"], op.id)
     np.testing.assert_array_equal(s["cell"], op.cell)
+
+
+@pytest.mark.parametrize("ppc", [3, 5, 9, 20])
+def test_vertex_sums_do_not_depend_on_the_room_for_particles(P, ppc):
+    import torch
+
+    n = (7, 6, 5)
+    mesh = P.Mesh(n, W.jittered_vertices(n, 3))
+    C = int(np.prod(n))
+    v = torch.as_tensor(np.random.default_rng(2).standard_normal(C * ppc), device="cuda")
+    got = []
+    for capacity in (0, 6 * C + 40 * C):
+        parts = P.Particles(mesh, uniform_count=ppc, seed=5, n_props=1, capacity=capacity)
+        parts.set_property(0, v)
+        got.append(parts.vertex_average(0))
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+
+
+# the choice between one and four lanes a cell falls at 14 particles in the largest of
+# 32 cells; from 77,824 cells a block takes four such groups
+@pytest.mark.parametrize("n", [(8, 4), (9, 7), (331, 257)])
+@pytest.mark.parametrize("per_cell", ["14", "15", "0..14", "one long", "long groups"])
+def test_vertex_sums_of_cell_groups(P, oracle_mod, n, per_cell):
+    C = int(np.prod(n))
+    per = {"14": np.full(C, 14), "15": np.full(C, 15), "0..14": np.arange(C) % 15, "one long": np.arange(C) % 5,
+           "long groups": np.where(np.arange(C) // 32 % 3 == 1, 17 + np.arange(C) % 4, np.arange(C) % 3)}[per_cell]
+    if per_cell == "one long":
+        per[C // 2] = 75
+    if C > 10000:
+        per = np.where(np.arange(C) < 70000, per % 8, per)  # most cells short: the oracle's time
+    mesh, parts, om, op, vals = T._pair(P, oracle_mod, n, per_cell=per.astype(np.uint32))
+    T._check_vertex(oracle_mod, parts, om, op, vals)
