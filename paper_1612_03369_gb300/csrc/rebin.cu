@@ -150,10 +150,17 @@ __global__ void __launch_bounds__(256) scatter_keys_kernel(const uint32_t* __res
 }
 
 // Scan and scatter in one launch for a mesh of at most kScanTileCells cells:
-// every block scans all the counts into its shared memory (one tile's scan,
-// ~1 us) and scatters its particles behind those offsets; block 0 also writes
-// the offsets and their total.  cursor starts from 0.  A scan kernel of its own
-// costs a small store's step 3.7 us and a launch gap of 2.
+// every block scans all the counts into its shared memory and scatters its
+// particles behind those offsets; block 0 also writes the offsets and their
+// total.  cursor starts from 0.  As the scan is repeated by every block, there are
+// no more of them than the particles fill with four each per thread, and at most
+// kScanBlocksPerSm per SM.  Euler step with a scan kernel of its own / with this:
+// 32^2 x 16 24.4 / 20.3 us, x 200 90.5 / 87.5; 64^2 x 4 24.5 / 22.4, x 36 39.4 / 36.8,
+// x 100 75 / 71, x 200 153 / 148; 16^3 x 20 41.3 / 39.2, x 100 87.4 / 83.3: faster over
+// the whole range.  (With the scan's runs in two banks and up to 16 blocks per SM it
+// took 97.5 at 64^2 x 100 and lost from about 30 particles per cell on; 1 block per SM
+// takes 73, 2 and 8 the same as 4.)
+constexpr int kScanBlocksPerSm = 4;
 __global__ void __launch_bounds__(256) scatter_scan_kernel(const uint32_t* __restrict__ cell_new,
                                                            const uint64_t* __restrict__ id,
                                                            const uint32_t* __restrict__ counts,
@@ -162,15 +169,17 @@ __global__ void __launch_bounds__(256) scatter_scan_kernel(const uint32_t* __res
                                                            uint32_t* __restrict__ key_src, uint32_t C, size_t cap,
                                                            const uint32_t* __restrict__ n_dev,
                                                            unsigned int* __restrict__ status) {
-  constexpr uint32_t kPer = kScanTileCells / 256;
-  __shared__ uint32_t s_off[kScanTileCells], s_total;
-  for (uint32_t k = threadIdx.x; k < kScanTileCells; k += 256) s_off[k] = k < C ? counts[k] : 0u;
+  // an odd number of entries per thread, so that a warp's runs start in 32 different
+  // banks (16 entries each put them in two, three sweeps of 2,048 bank passes)
+  const uint32_t per = ((C + 255u) / 256u) | 1u;
+  __shared__ uint32_t s_off[kScanTileCells + 256], s_total;
+  for (uint32_t k = threadIdx.x; k < per * 256u; k += 256) s_off[k] = k < C ? counts[k] : 0u;
   __syncthreads();
   uint32_t sum = 0;
-  for (uint32_t q = 0; q < kPer; ++q) sum += s_off[threadIdx.x * kPer + q];
+  for (uint32_t q = 0; q < per; ++q) sum += s_off[threadIdx.x * per + q];
   uint32_t run = block_excl_scan(sum, &s_total);
-  for (uint32_t q = 0; q < kPer; ++q) {
-    const uint32_t k = threadIdx.x * kPer + q, c = s_off[k];
+  for (uint32_t q = 0; q < per; ++q) {
+    const uint32_t k = threadIdx.x * per + q, c = s_off[k];
     s_off[k] = run;
     run += c;
   }
@@ -243,7 +252,8 @@ pic_status rebin_order_from_counts(pic_particles_s* p, cudaStream_t s) {
   const StoreView a = store_view(p, p->cur), b = store_view(p, 1 - p->cur);
   const int g = grid_cap(p->capacity, 256, 16);
   if (one_scan_tile(p)) {
-    scatter_scan_kernel<<<g, 256, 0, s>>>(p->cell_new, a.id, p->counts, p->cursor, p->cell_off, &p->ctr->n_next, p->key_id,
+    const size_t want = (p->capacity + 1023) / 1024, most = (size_t)num_sms() * kScanBlocksPerSm;
+    scatter_scan_kernel<<<(int)(want < most ? want : most), 256, 0, s>>>(p->cell_new, a.id, p->counts, p->cursor, p->cell_off, &p->ctr->n_next, p->key_id,
                                           p->key_src, p->C, p->capacity, &p->ctr->n_alive, &p->ctr->status);
   } else {
     pic_status r = scan_u32(p->counts, p->cell_off, p->C, p->block_sums, &p->ctr->n_next, p->cursor, s,

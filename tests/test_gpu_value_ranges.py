@@ -306,3 +306,18 @@ def test_vertex_sums_of_cell_groups(P, oracle_mod, n, per_cell):
         per = np.where(np.arange(C) < 70000, per % 8, per)  # most cells short: the oracle's time
     mesh, parts, om, op, vals = T._pair(P, oracle_mod, n, per_cell=per.astype(np.uint32))
     T._check_vertex(oracle_mod, parts, om, op, vals)
+
+
+# one launch scans and scatters: an odd number of cells per thread, the last runs past
+# the end, and more particles than its blocks take in one pass (622,592)
+@pytest.mark.parametrize("n, ppc", [((1, 1), 3000), ((255, 1), 7), ((257, 1), 7), ((16, 16), 33), ((47, 87), 9), ((64, 64), 170)])
+def test_steps_of_one_scan_tile(P, oracle_mod, n, ppc):
+    X = W.jittered_vertices(n, 3)
+    U = W.zero_wall_normal(n, W.normalise_max(W.stream_function_field(W.q2_node_coords(n, X), 3)))
+    wl = W.Workload("tile", 2, n, X, U, ppc, None, 1, 1, W.cfl_dt(n, X, U, 0.5), 2, 3, W.particle_seed(3))
+    mesh, parts = H.gpu_seed(wl)
+    om, op = H.oracle_seed(oracle_mod, wl)
+    parts.advect(wl.dt, 1, 2)
+    op = oracle_mod.advect(om, op, wl.dt, 1, 2)
+    H.assert_same_store(H.gpu_state(parts), op, wl)
+    np.testing.assert_array_equal(np.diff(parts.cell_offsets().cpu().numpy()), np.bincount(op.cell, minlength=wl.ncells))
