@@ -148,11 +148,16 @@ static __device__ __noinline__ df df_from_double_call(double x) { return df_from
 // field, the low part the 29-bit signed remainder, converted and scaled.
 // (df_from_double's three conversions and a subtraction are 4 FP64-pipe
 // operations, 64 clocks of an SM each for a warp.)  Values outside the range
-// where both parts are normal floats take df_from_double.
+// where both parts are normal floats take df_from_double, but for zeros, which a
+// composition or a field at rest is full of (vertex sums of zeros at 64^3 x 20: 139 us
+// that way, 119 for other values).
 __device__ __forceinline__ df split_f64(double x) {
   const long long b = __double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff) - 896;  // the float's exponent field
-  if (e < 60 || e > 250) return df_from_double_call(x);
+  if (e < 60 || e > 250) {
+    if ((b << 1) == 0) return df_make(__int_as_float((int)(b >> 32)), 0.f);
+    return df_from_double_call(x);
+  }
   const long long r = b + (1ll << 28);  // round half up in the magnitude
   const unsigned mag = ((unsigned)(r >> 29) ^ 0x40000000u) & 0x7fffffffu;
   const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;

@@ -321,3 +321,22 @@ def test_steps_of_one_scan_tile(P, oracle_mod, n, ppc):
     op = oracle_mod.advect(om, op, wl.dt, 1, 2)
     H.assert_same_store(H.gpu_state(parts), op, wl)
     np.testing.assert_array_equal(np.diff(parts.cell_offsets().cpu().numpy()), np.bincount(op.cell, minlength=wl.ncells))
+
+
+# zeros (of either sign) among values at and beyond the range of the split without
+# conversions, and nothing but zeros
+@pytest.mark.parametrize("values", ["mixed", "zeros"])
+@pytest.mark.parametrize("n", [(9, 7), (5, 4, 3)])
+def test_transfers_of_zeros(P, oracle_mod, n, values):
+    import torch
+
+    per = (np.arange(int(np.prod(n))) * 5 % 19).astype(np.uint32)
+    mesh, parts, om, op, vals = T._pair(P, oracle_mod, n, per_cell=per)
+    g = np.random.default_rng(4)
+    v = np.array([0.0, -0.0, 1.0, -1.0, 2.0**-128, -(2.0**-100), 1e-30])[g.integers(0, 7, op.n)] if values == "mixed" else np.zeros(op.n)
+    parts.set_property(0, torch.as_tensor(v, device="cuda"))
+    T._check_vertex(oracle_mod, parts, om, op, v)
+    T._check_lsq(oracle_mod, parts, om, op, v, len(n))
+    if values == "zeros":
+        avg, w = parts.vertex_average(0)
+        assert (avg[w > 0] == 0).all()
