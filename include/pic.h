@@ -152,7 +152,7 @@ pic_status pic_cell_weights(pic_mesh mesh, const double *rho, double *w, void *s
  *   w       [n_cells] FP64 device, finite and >= 0, positive sum
  *   counts  [n_cells] u32 device (overwritten); usable as pic_seed_particles'
  *           or pic_seed_particles_mh's per_cell
- * The fold runs on one warp (one-time set-up cost, about 5 ns per cell).
+ * The fold runs on one block (one-time set-up cost, about 2 ns per cell).
  * Synchronises `stream` to check the weights.
  * Errors: PIC_ERR_ARG (bad weights), PIC_ERR_CAPACITY (n_particles >= 2^32),
  * PIC_ERR_OOM, PIC_ERR_CUDA. */

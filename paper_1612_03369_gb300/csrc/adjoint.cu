@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256) rank_records_kernel(const uint32_t* __res
 
 // Checkpoint tapes: the step replayed from the store as it was at the start
 // of the step, for every particle then alive, by the forward's own
-// advect_particle (so the stage records are the forward's bit for bit); the
+// advect_particle_step (so the stage records are the forward's bit for bit); the
 // new positions go to a sink.
 template <int D, int RK>
 __global__ void __launch_bounds__(128, PIC_ADVECT_MIN_BLOCKS) replay_step_kernel(const __grid_constant__ MeshView m, const __grid_constant__ StoreView s, const __grid_constant__ StoreView sink,

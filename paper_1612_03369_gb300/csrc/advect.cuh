@@ -249,12 +249,6 @@ __device__ __forceinline__ uint32_t advect_particle_to(const MeshView& m, const 
                                                  static_cast<Hook&&>(hook));
 }
 
-template <int D, int RK, bool F32B, int TWO = kSteady, class Hook = NoHook>
-__device__ __forceinline__ uint32_t advect_particle(const MeshView& m, const StoreView& s, uint32_t i, uint32_t K,
-                                                    df dt, int& iters, unsigned& flags, Hook&& hook = Hook()) {
-  return advect_particle_to<D, RK, F32B, TWO>(m, s, i, s, i, K, dt, iters, flags, static_cast<Hook&&>(hook));
-}
-
 // The full step of one particle (every rare path of the locate available),
 // out of line: the fallback of a fast-path step that returned kDefer.  It
 // re-reads the particle from s, so nothing of the abandoned fast step is

@@ -451,7 +451,6 @@ __device__ __noinline__ RarePath<D> test_cell_fp64(const MeshView& m, uint32_t K
   return o;
 }
 
-// Fast path, then the FP64 Newton when the fast path does not settle.
 // y inside cell K's padded bounding box (padding 1e-6 of the cell's extent,
 // far wider than the kInsideEps band in reference coordinates): a point
 // outside it is not in K.  The FP32 copy of the box is widened outward, so
@@ -466,6 +465,7 @@ __device__ __forceinline__ bool in_cell_box(const MeshView& m, uint32_t K, const
   return in;
 }
 
+// Fast path, then the FP64 Newton when the fast path does not settle.
 template <int D, class Cells>
 __device__ __forceinline__ int test_cell(const Cells& cs, const MeshView& m, uint32_t K, const df y[D], float t32[D],
                                          df t[D], int& iters, unsigned& flags) {
