@@ -100,7 +100,12 @@ pic_status pic_destroy_mesh(pic_mesh mesh);
  *           (Sec. 2.3, eq. position-ode-approx; c = 0, 1/2, 1/2, 1 for RK4,
  *           0, 1/2 for RK2, 0 for Euler).  Not supported by the adjoint.
  * The library copies the fields (stream-ordered); the caller may reuse them.
- * Errors: PIC_ERR_ARG, PIC_ERR_CUDA. */
+ * It keeps per-cell tables of them, allocated on first use: 720 B per hex (160
+ * per quad) for U, and with U_next as much again for it and for the mean of the
+ * two, which the middle of a step reads (1.5 GB at 128^3).  Without room for the
+ * mean's table the steps evaluate both fields instead: slower, and the same but
+ * for rounding.
+ * Errors: PIC_ERR_ARG, PIC_ERR_OOM, PIC_ERR_CUDA. */
 pic_status pic_set_velocity_dofs(pic_mesh mesh, const double *U, const double *U_next, void *stream);
 
 /* Staged upload of the next field, so that its copy overlaps the current

@@ -340,3 +340,59 @@ def test_transfers_of_zeros(P, oracle_mod, n, values):
     if values == "zeros":
         avg, w = parts.vertex_average(0)
         assert (avg[w > 0] == 0).all()
+
+
+def test_committed_field_with_a_second_field_set(P):
+    """A staged field committed while a second field is set: as both set directly, bit
+    for bit, so the mean's table follows the committed field."""
+    import torch
+
+    wl = W.curl_cube(6, 6, 2, 3)
+    second = torch.as_tensor(np.ascontiguousarray(-0.4 * wl.U), device="cuda")
+    fields = [torch.as_tensor(np.ascontiguousarray(s * wl.U), device="cuda") for s in (1.0, 0.7, 1.2)]
+    got = []
+    for staged in (False, True):
+        mesh, parts = H.gpu_seed(wl)
+        P.pic_set_velocity_dofs(mesh.h, fields[0], U_next=second)
+        for f in fields[1:]:
+            parts.advect(wl.dt, 4, 1)
+            if staged:
+                P.pic_stage_velocity_dofs(mesh.h, f)
+                P.pic_commit_velocity_dofs(mesh.h)
+            else:
+                P.pic_set_velocity_dofs(mesh.h, f, U_next=second)
+        parts.advect(wl.dt, 4, 1)
+        got.append(H.gpu_state(parts))
+    for k in got[0]:
+        np.testing.assert_array_equal(got[0][k], got[1][k])
+
+
+def test_two_fields_without_room_for_the_table_of_their_mean(P, oracle_mod):
+    """With 95 MB left on the device the second field's arrays (72 MB) fit and the
+    mean's table (46 MB) does not: the step evaluates both fields in its middle."""
+    import torch
+
+    wl = W.curl_cube(40, 1, 1, 3)
+    mesh, parts = H.gpu_seed(wl)
+    om, op = H.oracle_seed(oracle_mod, wl)
+    second = -0.4 * wl.U
+    first_d, second_d = (torch.as_tensor(np.ascontiguousarray(f), device="cuda") for f in (wl.U, second))
+    P.pic_set_velocity_dofs(mesh.h, first_d)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    room = torch.cuda.mem_get_info()[0] - (95 << 20)
+    try:
+        fill = torch.empty(room, dtype=torch.uint8, device="cuda")
+        before = P.pic_kernel_launches()
+        P.pic_set_velocity_dofs(mesh.h, first_d, U_next=second_d)
+        built = P.pic_kernel_launches() - before
+    except (P.PicError, torch.OutOfMemoryError):
+        pytest.skip("the device's memory could not be filled to within 95 MB")
+    finally:
+        fill = None
+        torch.cuda.empty_cache()
+    if built != 4:  # a fifth launch builds the mean's table
+        pytest.skip("the device's memory could not be filled to within 95 MB")
+    om.set_velocity_next(second)
+    parts.advect(wl.dt, 4, 1)
+    H.assert_same_store(H.gpu_state(parts), oracle_mod.advect(om, op, wl.dt, 4, 1), wl)
