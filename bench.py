@@ -72,16 +72,16 @@ def advect_bytes(dim: int, ppc: float, n_props: int, xhat_bytes: int = 8, dof_by
 # multi-step call; traffic grows with the particle count, so a launch at
 # another size is scaled by its particles.  Keyed by precision (0 FP64
 # form, 1 FP32-basis form).
-ADVECT_DRAM_BYTES_PER_PARTICLE = {0: 1209.017e6 / 5242880, 1: 1012.980e6 / 5242880}
+ADVECT_DRAM_BYTES_PER_PARTICLE = {0: 1298.444e6 / 5242880, 1: 1013.848e6 / 5242880}
 # Warp instructions per 32 particle-steps and pipe utilisation of the same
 # captures: the advect kernel is bound by instruction issue (double-float
 # arithmetic on the FP32 pipe) in the FP64 form, and by issue and load
 # latency in the FP32-basis form, not by HBM.
 ADVECT_ISSUE = {
-    0: {"warp_instructions_per_32_particle_steps": 8052, "issue_active_pct": 74.2, "fma_pipe_active_pct": 56.6,
-        "top_stall": "long_scoreboard 3.10 per issue, not_selected 2.45"},
-    1: {"warp_instructions_per_32_particle_steps": 4234, "issue_active_pct": 64.2, "fma_pipe_active_pct": 39.4,
-        "top_stall": "long_scoreboard 3.68 per issue"},
+    0: {"warp_instructions_per_32_particle_steps": 9232, "issue_active_pct": 75.1, "fma_pipe_active_pct": 59.7,
+        "top_stall": "not_selected 2.74 per issue, long_scoreboard 2.54"},
+    1: {"warp_instructions_per_32_particle_steps": 4231, "issue_active_pct": 65.2, "fma_pipe_active_pct": 41.4,
+        "top_stall": "long_scoreboard 3.58 per issue"},
 }
 
 
@@ -593,9 +593,9 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # (1,048,576 particles, RK4), counted by an ncu capture of these kernels:
 # reverse_lambda_kernel (G and lambda at 4.19M stage points, double-float)
 # and cell_partial_kernel (the per-cell sums, double-float).
-ADJOINT_C4_FP32_FLOPS_PER_REVERSE_STEP = 1.186e10 + 6.538e9
+ADJOINT_C4_FP32_FLOPS_PER_REVERSE_STEP = 1.377e10 + 6.538e9
 # DRAM bytes (read + write) of the same two kernels per reverse step, same capture.
-ADJOINT_C4_DRAM_BYTES_PER_REVERSE_STEP = (195.3e6 + 97.2e6) + (220.8e6 + 15.3e6)
+ADJOINT_C4_DRAM_BYTES_PER_REVERSE_STEP = (199.0e6 + 102.1e6) + (221.1e6 + 16.3e6)
 
 
 def run_adjoint(args):
@@ -792,16 +792,14 @@ def run_props(args):
 
 
 # FP32 flops (FADD + FMUL + 2 FFMA) per particle-step of the property-ODE
-# work beyond the plain step: the stage-gradient kernel (12,016) and the ODE
+# work beyond the plain step: the stage-gradient kernel (13,768) and the ODE
 # kernel (4,480), both in double-float, counted by ncu on the 64^3 x 20
 # workload (an ncu capture of these kernels).
-PROPS_ODE_FP32_FLOPS_PER_PARTICLE_STEP = 16496.0
+PROPS_ODE_FP32_FLOPS_PER_PARTICLE_STEP = 18248.0
 
-# FP64 operations per unit of the FP64-bound kernels (dadd + dmul + 2 dfma,
-# counted by ncu captures on 48^3 x 16, J = 8).  The chains decide most of their
-# steps in FP32 and emit in FP64; the FP64 pipe also carries their conversions.
+# FP64 operations per unit of the FP64-bound kernel (dadd + dmul + 2 dfma,
+# counted by an ncu capture on 48^3 x 16).
 FP64_FLOPS = {
-    "mh_seed_kernel<3>": 8.97,             # per chain step
     "cell_weights_kernel<3>": 1455.5,      # per cell
 }
 # FP64 peak: the GB300's nominal FP64 rate, 1.25 TFLOP/s (FMA = 2 flops).
@@ -816,6 +814,14 @@ def _fp64_roof(kernel, units, ms):
     ach = f * units / (ms / 1e3) / 1e12
     return {"kernel": kernel, "bound": "fp64", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": ach / FP64_PEAK_TFLOPS, "fp64_flops_per_unit": f, "peak_kind": "derived (nominal FP64 rate)"}
+
+
+def _chain_rate(steps, particles, ms):
+    """The chains decide most of their steps from FP32 values beside the
+    generator's 64-bit integer products, and map each emitted particle in FP64:
+    no one pipe's peak bounds them at every thinning, so the line gives times."""
+    return {"kernel": "mh_seed_kernel<3>", "bound": "FP32 and integer issue per chain step, FP64 pipe per emitted particle",
+            "ns_per_chain_step": ms * 1e6 / steps, "ns_per_particle": ms * 1e6 / particles}
 
 
 # The transfers fold each particle's x-hat (three double-float pairs) and its
@@ -963,7 +969,7 @@ def run_next(args):
                          "roofline": _fp64_roof("cell_weights_kernel<3>", wl.ncells, ms_w)},
         "metropolis_hastings_ms": ms_m, "mh_thinning": J, "import_ms": ms_i,
         "mh": {"value": N * J / (ms_m / 1e3), "unit": "chain steps/s",
-               "roofline": _fp64_roof("mh_seed_kernel<3>", N * J, ms_m)},
+               "roofline": _chain_rate(N * J, N, ms_m)},
         "import": {"value": N / (ms_i / 1e3), "unit": "points/s"},
         "cpu_baseline": {
             "cell_weights": cpu(lambda: O.cell_weights(om, rho), wl.ncells, "all %d cells" % wl.ncells),

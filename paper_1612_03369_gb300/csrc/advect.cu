@@ -89,8 +89,8 @@ __device__ __forceinline__ void finish_tile(DevCounters* __restrict__ ctr, uint3
 }
 
 // Resident blocks per SM of the step kernel.  Five steps and an export on 64^3 x
-// 20, one node: FP64 form 9.15 / 8.92 / 8.76 / 8.94 ms at 5 / 6 / 7 / 8 blocks;
-// FP32-basis form 6.11 / 5.76 / 5.75 / 5.75 ms, where earlier builds at 7 and 8
+// 20, one node: FP64 form 9.15 / 9.15 / 9.00 / 9.15 ms at 5 / 6 / 7 / 8 blocks;
+// FP32-basis form 5.59 / 5.24 / 5.22 / 5.25 ms, where earlier builds at 7 and 8
 // blocks ran up to a third slower on some nodes, so it takes 6 (80 registers).
 #ifndef PIC_ADVECT_MIN_BLOCKS_F64
 #define PIC_ADVECT_MIN_BLOCKS_F64 7

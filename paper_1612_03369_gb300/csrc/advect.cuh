@@ -47,7 +47,8 @@ __device__ __forceinline__ void flush_counters(DevCounters* ctr, unsigned steps,
 // fields so the kernel holds one copy of it.  The double-float form reads the
 // middle of the step from a table of the mean coefficients, set up with the
 // fields: four evaluations per RK4 step where two fields at two stages made
-// six (1.54 against 2.06 ms per step at 64^3 x 20, for 86 us more per field).
+// six (a new field, a step and three averages at 64^3 x 20: 2.46 against 2.81 ms,
+// with the 86 us that the table takes).
 enum : int {
   kSteady = 0,
   kMidTable = 1,  // two fields and the table of their mean

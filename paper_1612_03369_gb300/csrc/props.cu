@@ -33,8 +33,8 @@ struct OdeArgs {
 // Phase 2, thread per (stage, surviving particle): G_p = grad u_h at the
 // recorded stage point, in double-float, stored as G[(p D^2 + e) cap + i].
 // A kernel of its own, so that neither it nor the ODE kernel outgrows the
-// instruction cache.  80 registers, 6 blocks per SM: 1.82 ms at 64^3 x 20, four
-// stages, against 1.97 at 4 (96 registers).
+// instruction cache.  80 registers, 6 blocks per SM: two steps with both ODEs and
+// an export at 64^3 x 20 take 10.15 ms, 10.5 at 4 and 5.
 template <int D>
 __global__ void __launch_bounds__(128, 6) props_grad_kernel(const __grid_constant__ MeshView m, const __grid_constant__ StageRec rec, int S,
                                                            const uint32_t* __restrict__ cell_new,
